@@ -11,11 +11,20 @@ namespace {
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Tile shape used without measurement: the widest unit block that still
-// gives every resident warp a column, and enough chunks per column to give
-// each resident warp about two tiles when columns are scarce.
+// Tile shape used without measurement.  Whole columns of 32 units (the ring
+// kernel, no chunk read twice) unless there are too few of them to keep the
+// SMs' memory pipes full AND the sequence is long: a lone warp walks about 65
+// sites per us (8 x 2704 x 32: 50 us whole, 26 us in look-back chunks of
+// 256; 64 x 700 x 64, 128 columns: 16 us whole, 38 us in chunks).  Many
+// short columns take the 128-unit block, whose rows are 512 bytes (16384 x
+// 100 x 128: 369 us against 401 us; from 256 sites on the two are equal).
+// Otherwise (H not a multiple of 32, or few long columns): the widest unit
+// block that still gives every resident warp a column, and enough chunks per
+// column to give each resident warp about two tiles when columns are scarce.
 psr_scan_tile scan_default_tile(const psr_context *ctx, int64_t n, int N, int H) {
     const int64_t resident = (int64_t)ctx->num_sms * 32;  // warps at 4 CTAs of 8 warps per SM
+    if (H % 128 == 0 && N < 256 && n * (H / 128) >= resident) return psr_scan_tile{128, N};
+    if (H % 32 == 0 && (n * (H / 32) >= 64 || N <= 1024)) return psr_scan_tile{32, N};
     int units = 4;
     const int widths[4] = {128, 32, 16, 4};
     for (int w : widths)
