@@ -6,9 +6,8 @@
 // Launches of one call: parameter packing, bit-packing and the connected-set
 // generator per item (small), then ONE sample forward over the samples of all
 // items, ONE persistent forward over the connected configurations of all
-// items (ragged over samples and lattices), the E_loc gathers, ONE FP32
-// forward on gradient chunks and ONE reverse-scan gradient over the samples
-// of all gradient items.  With graphs enabled the whole sequence is captured
+// items (ragged over samples and lattices), the E_loc gathers, and the
+// gradients item by item (each a whole batch of samples per launch).  With graphs enabled the whole sequence is captured
 // once per argument set and replayed.
 #include "psr_api_common.cuh"
 
@@ -63,6 +62,7 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         float *carries_g, *lpsi_g;             // gradient forward
         int N, W, nb;
         int64_t cap;
+        int64_t B;                             // samples per batch of the FP32 layer gradient (0: chunk recompute)
     } w[kMaxGroups];
     int64_t n_grad = 0;
     for (int i = 0; i < n_items; ++i) {
@@ -80,17 +80,6 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         x.cap = it.eloc ? it.n * max_entries_per_sample(&it.ham) : 0;
         if (it.grad) n_grad += it.n;
     }
-    // gradient launch geometry: as psr_grad (CTAs per SM by shared memory)
-    int grad_grid = 0;
-    if (n_grad > 0) {
-        int dev_smem = 0;
-        cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ctx->device);
-        int occ = (int)(dev_smem / (bwd_smem_bytes(H, nL) + 1024));
-        occ = occ < 1 ? 1 : (occ > 4 ? 4 : occ);
-        int64_t g = (int64_t)ctx->num_sms * occ;
-        grad_grid = (int)(g > n_grad ? n_grad : g);
-    }
-
     // BF16 gradients run on the tensor cores one item after another (as
     // psr_grad does), through one set of batch buffers sized for the largest
     const bool use_tc = bf16 && H == 128;
@@ -104,8 +93,41 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
             tc_stash = st_i > tc_stash ? st_i : tc_stash;
             tc_arr = ar_i > tc_arr ? ar_i : tc_arr;
         }
-        grad_grid = 0;
     }
+    // FP32 gradients: layer by layer, one item after another through one set
+    // of arrays, as psr_grad does; samples too long for that share one launch
+    // of the chunk-recompute kernel (CTAs per SM by shared memory).
+    const bool copy_theta = d_theta && !aligned16p(params->theta);
+    int grad_grid = 0;
+    size_t layer_bytes = 0;
+    bool by_chunk = false;  // some item takes the chunk-recompute kernel
+    auto plan_grad = [&](bool layers, int shift) {
+        int64_t n_chunk = 0;
+        layer_bytes = 0;
+        for (int i = 0; i < n_items; ++i) {
+            w[i].B = 0;
+            if (!items[i].grad || use_tc) continue;
+            if (layers) w[i].B = grad_f32_batch(nL, H, w[i].N, items[i].n);
+            if (w[i].B == 0) {
+                n_chunk += items[i].n;
+                continue;
+            }
+            w[i].B = w[i].B >> shift ? w[i].B >> shift : 1;
+            GradF32Args A{};
+            Carver c;
+            grad_f32_carve(c, nL, H, w[i].N, w[i].B, false, copy_theta, A);
+            layer_bytes = c.off > layer_bytes ? c.off : layer_bytes;
+        }
+        by_chunk = n_chunk > 0;
+        int dev_smem = 0;
+        cudaDeviceGetAttribute(&dev_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, ctx->device);
+        int occ = (int)(dev_smem / (bwd_smem_bytes(H, nL) + 1024));
+        occ = occ < 1 ? 1 : (occ > 4 ? 4 : occ);
+        const int64_t g = (int64_t)ctx->num_sms * occ;
+        grad_grid = (int)(g > n_chunk ? n_chunk : g);
+    };
+    plan_grad(true, 0);
+    char *layer_ws = nullptr;
     GradTcWs tw{};
     float *theta_ws = nullptr, *pk = nullptr, *tape = nullptr;
     void *pkb = nullptr;
@@ -116,6 +138,7 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         pkb = c.get<char>(bf16 ? bf16_packed_bytes() : 0);
         counters = c.get<unsigned long long>(3);
         tape = c.get<float>((size_t)grad_grid * bwd_tape_floats_per_cta(nL, H));
+        layer_ws = c.get<char>(layer_bytes);
         if (use_tc && n_grad > 0) {
             tw.images = c.get<char>(bwd_tc_image_bytes(nL));
             tw.stash = c.get<float>(tc_stash);
@@ -149,13 +172,22 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
             x.logp = c.get<float>(it.eloc ? (size_t)n * x.N : 0);
             x.carries = c.get<float>(it.eloc ? (size_t)n * nch * nL * H : 0);
             x.delta = c.get<float>(x.cap);
-            x.carries_g = c.get<float>(it.grad && !use_tc ? (size_t)n * nchg * nL * H : 0);
-            x.lpsi_g = c.get<float>(it.grad && !use_tc ? n : 0);
+            const bool chunked = it.grad && !use_tc && x.B == 0;
+            x.carries_g = c.get<float>(chunked ? (size_t)n * nchg * nL * H : 0);
+            x.lpsi_g = c.get<float>(chunked ? n : 0);
         }
     };
-    Carver sz;
-    carve(sz);
-    if ((rc = ensure_ws(ctx, sz.off)) != PSR_OK) return rc;
+    // without room for the layers' arrays: smaller batches, then chunks
+    for (int shift = 0;;) {
+        Carver sz;
+        carve(sz);
+        rc = ensure_ws(ctx, sz.off);
+        if (rc != PSR_ENOMEM || layer_bytes == 0) break;
+        bool smaller = false;
+        for (int i = 0; i < n_items; ++i) smaller = smaller || w[i].B > 1;
+        plan_grad(smaller, ++shift);
+    }
+    if (rc != PSR_OK) return rc;
     Carver cv;
     cv.base = static_cast<char *>(ctx->ws);
     carve(cv);
@@ -190,7 +222,7 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         }
         // kernel attributes are set outside the capture
         if (bf16) PSR_TRY(prepare_fwd_bf16());
-        if (n_grad > 0 && !use_tc) PSR_TRY(prepare_bwd_f32(H, nL));
+        if (by_chunk) PSR_TRY(prepare_bwd_f32(H, nL));
         if (n_grad > 0 && use_tc) PSR_TRY(prepare_bwd_tc());
         PSR_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
         ctx->capturing = true;
@@ -296,8 +328,24 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
                     return r;
             }
         }
-        // ---- gradient: FP32 forward on gradient chunks, then the reverse scan
-        if (n_grad > 0 && !use_tc) {
+        // ---- gradient in FP32, layer by layer
+        if (layer_bytes > 0) {
+            StageScope sc(ctx, PSR_STAGE_BWD);
+            for (int i = 0; i < n_items; ++i) {
+                const StepItem &it = items[i];
+                if (w[i].B == 0) continue;
+                GradF32Args A{};
+                Carver sub;
+                sub.base = layer_ws;
+                grad_f32_carve(sub, nL, H, w[i].N, w[i].B, false, copy_theta, A);
+                float *rows = w[i].d_g ? it.grad : w[i].g_ws;
+                if ((r = enqueue_grad_f32(ctx, nL, H, it.u1, theta, pk, w[i].bits, it.n, w[i].N, w[i].W, nullptr,
+                                          rows, w[i].B, A)) != PSR_OK)
+                    return r;
+            }
+        }
+        // ---- gradient of long samples: FP32 forward on short chunks, then the reverse scan
+        if (by_chunk) {
             FwdJobs jg{};
             jg.mode = 0;
             jg.job_counter = counters + 2;
@@ -306,7 +354,7 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
             bj.first[0] = 0;
             for (int i = 0; i < n_items; ++i) {
                 const StepItem &it = items[i];
-                if (!it.grad) continue;
+                if (!it.grad || w[i].B > 0) continue;
                 FwdGroup &a = jg.g[jg.n_groups++];
                 a.u1 = it.u1;
                 a.N = w[i].N;

@@ -397,5 +397,92 @@ inline int enqueue_grad_tc(psr_context *ctx, int nL, int u1, const float *theta,
     return PSR_OK;
 }
 
+// ------------------------------------------------ FP32 gradients by layers
+// The layer-by-layer FP32 gradients hold every layer's arrays of a batch of
+// samples; batches are sized to kGradBudget bytes of them.  A sample that
+// needs more by itself goes to the chunk-recompute kernel of its model, which
+// keeps only chunk carries.
+constexpr size_t kGradBudget = size_t(2) << 30;
+
+// Samples per batch for `per` floats of arrays a sample; 0: too long.
+inline int64_t grad_batch(size_t per, int64_t sites, int64_t n) {
+    const size_t bytes = per * sizeof(float);
+    if (bytes > kGradBudget || sites >= (int64_t)1 << 30) return 0;
+    int64_t B = (int64_t)(kGradBudget / bytes);
+    const int64_t most = ((int64_t)1 << 30) / sites;
+    if (B > most) B = most;
+    return B < n ? B : n;
+}
+
+inline bool aligned16p(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+inline int64_t grad_f32_batch(int nL, int H, int L, int64_t n) {
+    return grad_batch(grad_f32_floats_per_site(nL, H) * (size_t)L, L, n);
+}
+
+// Carves the batch arrays of launch_grad_f32 into A (sum: a weighted sum over
+// the samples, else O_k rows).
+inline void grad_f32_carve(Carver &c, int nL, int H, int L, int64_t B, bool sum, bool copy_theta, GradF32Args &A) {
+    const size_t M = (size_t)B * L, arr = M * H;
+    const int64_t P = theta_layout(nL, H).total;
+    A.theta = c.get<float>(copy_theta ? P : 0);
+    for (int l = 0; l < nL; ++l) {
+        A.a[l] = c.get<float>(l ? arr : 0);
+        A.c[l] = c.get<float>(l ? arr : 0);
+        A.h[l] = c.get<float>(arr);
+        A.dy[l] = c.get<float>(arr);
+        A.u[l] = c.get<float>(arr);
+    }
+    A.gy[0] = c.get<float>(arr);
+    A.gy[1] = c.get<float>(arr);
+    A.gh = c.get<float>(arr);
+    A.dc = c.get<float>(arr);
+    A.g = c.get<float>(M);
+    const size_t range = grad_f32_range(H);
+    A.rows = c.get<float>(sum ? (M + range - 1) / range * P : 0);
+    A.small = c.get<float>(sum ? (size_t)B * grad_f32_small_floats(H) : 0);
+}
+
+// Enqueues the gradient of n samples of L sites (bit-packed, W words a row) in
+// batches of B through the arrays in A: O_k rows (dout == NULL) or the
+// dout-weighted sum into out.
+inline int enqueue_grad_f32(psr_context *ctx, int nL, int H, int u1, const float *theta, const float *pk,
+                            const uint64_t *bits, int64_t n, int L, int W, const float *dout, float *out,
+                            int64_t B, GradF32Args A) {
+    cudaStream_t st = ctx->stream;
+    A.tl = theta_layout(nL, H);
+    A.fl = f32_layout(nL, H);
+    const int64_t P = A.tl.total;
+    if (!aligned16p(theta)) {
+        PSR_TRY(cudaMemcpyAsync(const_cast<float *>(A.theta), theta, P * sizeof(float), cudaMemcpyDeviceToDevice, st));
+    } else {
+        A.theta = theta;
+    }
+    A.N = L;
+    A.W = W;
+    A.u1 = u1;
+    A.nL = nL;
+    A.H = H;
+    A.pk = pk;
+    if (dout) {
+        A.sm = GradSmall{0, 2 * H, 3 * H, 5 * H, 6 * H, 8 * H, 10 * H};
+        A.small_stride = grad_f32_small_floats(H);
+        A.sum_out = out;
+    } else {
+        A.sm = GradSmall{A.tl.Wz[0], A.tl.bz[0], A.tl.Wh[0], A.tl.bh[0], A.tl.D[0], A.tl.Wo, A.tl.bo};
+        A.small_stride = P;
+        A.sum_out = nullptr;
+    }
+    for (int64_t s0 = 0; s0 < n; s0 += B) {
+        A.n = (int)(n - s0 < B ? n - s0 : B);
+        A.bits = bits + s0 * W;
+        A.dout = dout ? dout + s0 : nullptr;
+        if (!dout) A.rows = A.small = out + s0 * P;
+        A.add = s0 > 0;
+        PSR_TRY(launch_grad_f32(A, st));
+    }
+    return PSR_OK;
+}
+
 }  // namespace apiutil
 }  // namespace psr

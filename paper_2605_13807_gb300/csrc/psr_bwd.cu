@@ -1,4 +1,6 @@
-// Reverse-mode gradient d log psi / d theta (FP32, SIMT).
+// Reverse-mode gradient d log psi / d theta (FP32, SIMT) with chunk recompute:
+// the form for samples whose layer arrays would not fit (psr_grad_f32.cu is
+// the fast one; this one keeps only chunk carries).
 //
 // For each sample the chunks are visited in reverse order.  A chunk is first
 // recomputed from the chunk-boundary carries stored by the forward (so no

@@ -1,0 +1,462 @@
+// Reverse-mode gradient d log psi / d theta of the chain minGRU in FP32
+// (derivative of Eq. minGRU and of the output map, Sec. II.F-G; the
+// energy-gradient estimates of Sec. III.B), layer by layer over a whole batch
+// of samples in site-major arrays [sample][site][unit]:
+//   forward   z | c = [W_z; W_h] u + b (layer 0: lookups of the one-hot input),
+//             a = sigmoid(z); h_t = a_t h_{t-1} + (1 - a_t) c_t;
+//             y = C h + D u [+ h of layer l-1 for l >= 2], u of the next layer
+//             = GELU(y); readout adjoint g_t = 1/2 (s_t - P(1 | s_<t)) dout
+//   backward  gy = gx GELU'(y);  gh = C^T gy (+ gy of layer l+1, l+1 >= 2);
+//             lambda_t = gh_t + a_{t+1} lambda_{t+1};
+//             dz = lambda (h_{t-1} - c) a (1 - a),  dc = lambda (1 - a);
+//             gx of layer l-1 = W_z^T dz + W_h^T dc + D^T gy
+//   weights   dC = sum gy h^T, dD = sum gy u^T, dW_z = sum dz u^T, dW_h = sum dc u^T
+// The products are the FP32 tiles of psr_gemm.cuh; the scans are one thread
+// per (sample, unit), coalesced over units.
+//
+// What bounds it: the FP32 rate in the products (54 H^2 operations a site) and
+// HBM for the arrays between them (about 75 arrays of 4 H bytes a site): at
+// hidden 64, 4096 samples of 100 sites (weighted sum) 2.4 ms of the 3.1 ms are
+// products at 31 to 46 TFLOP/s, the rest streams.  The chunk-recompute kernel
+// (psr_bwd.cu: a CTA per sample, a thread per unit, the sum by reductions in
+// L2 every 16 sites) takes 11.3 ms there.
+#include <cuda_runtime.h>
+
+#include "psr_device.cuh"
+#include "psr_gemm.cuh"
+#include "psr_internal.cuh"
+
+namespace psr {
+
+namespace {
+
+// input code of site t: 0 at the first site, 1 + s_{t-1} otherwise
+__device__ __forceinline__ int code_at(const uint64_t *row, int t) {
+    return t == 0 ? 0 : 1 + (int)((row[(t - 1) >> 6] >> ((t - 1) & 63)) & 1ull);
+}
+
+struct NoCtx {};
+
+struct EpiProj {  // a = sigmoid(z), c
+    const float *bz, *bh;
+    float *a, *c;
+    int H;
+    __device__ NoCtx row(int) const { return {}; }
+    __device__ void operator()(NoCtx, int m, int u, float z, float cc) const {
+        const size_t i = (size_t)m * H + u;
+        a[i] = sigmoid_f(z + bz[u]);
+        c[i] = cc + bh[u];
+    }
+};
+
+struct EpiOut {  // the next layer's input u = GELU(y), and GELU'(y) for the way back
+    const float *du0;      // layer 0: D of the one-hot input by code, else null
+    const float *h_below;  // residual, or null
+    const uint64_t *bits;
+    float *dy, *u;
+    int H, N, W;
+    __device__ int row(int m) const {
+        if (!du0) return 0;
+        const int s = m / N;
+        return code_at(bits + (int64_t)s * W, m - s * N);
+    }
+    __device__ void operator()(int code, int m, int j, float v) const {
+        const size_t i = (size_t)m * H + j;
+        if (du0) v += du0[code * H + j];
+        if (h_below) v += h_below[i];
+        const float cdf = 0.5f * (1.0f + erff(v * 0.70710678118654752f));
+        u[i] = v * cdf;
+        dy[i] = fmaf(v * 0.39894228040143268f, expf(-0.5f * v * v), cdf);
+    }
+};
+
+struct EpiStore {
+    float *out;
+    int H;
+    __device__ NoCtx row(int) const { return {}; }
+    __device__ void operator()(NoCtx, int m, int j, float v) const { out[(size_t)m * H + j] = v; }
+};
+
+struct EpiGy {  // adjoint of the pre-activation of the layer below
+    const float *dy;
+    float *gy;
+    int H;
+    __device__ NoCtx row(int) const { return {}; }
+    __device__ void operator()(NoCtx, int m, int j, float v) const {
+        const size_t i = (size_t)m * H + j;
+        gy[i] = v * dy[i];
+    }
+};
+
+constexpr int kScanStep = 8;
+
+// h of one layer; layer 0 takes a and b = (1 - a) c from the input code
+__global__ void __launch_bounds__(128) grad_scan_fwd_kernel(const __grid_constant__ GradF32Args A, int l) {
+    const int H = A.H, N = A.N;
+    const int64_t idx = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    const int64_t s = idx / H;
+    const int j = (int)(idx % H);
+    if (s >= A.n) return;
+    const int64_t base = s * N * H + j;
+    float *hp = A.h[l] + base;
+    float h = 0.0f;
+    if (l == 0) {
+        const uint64_t *row = A.bits + s * A.W;
+        float ta[3], tb[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            ta[q] = A.pk[A.fl.A0 + q * H + j];
+            tb[q] = A.pk[A.fl.B0 + q * H + j];
+        }
+        h = tb[0];
+        hp[0] = h;
+        for (int t = 1; t < N; ++t) {
+            const bool up = (row[(t - 1) >> 6] >> ((t - 1) & 63)) & 1ull;
+            h = (up ? ta[2] : ta[1]) * h + (up ? tb[2] : tb[1]);
+            hp[(int64_t)t * H] = h;
+        }
+        return;
+    }
+    const float *ap = A.a[l] + base, *cp = A.c[l] + base;
+    float na[kScanStep], nc[kScanStep];
+    auto fetch = [&](int t) {
+#pragma unroll
+        for (int i = 0; i < kScanStep; ++i) {
+            const bool in = t + i < N;
+            na[i] = in ? ap[(int64_t)(t + i) * H] : 0.0f;
+            nc[i] = in ? cp[(int64_t)(t + i) * H] : 0.0f;
+        }
+    };
+    fetch(0);
+    for (int t = 0; t < N; t += kScanStep) {
+        float a[kScanStep], c[kScanStep];
+#pragma unroll
+        for (int i = 0; i < kScanStep; ++i) {
+            a[i] = na[i];
+            c[i] = nc[i];
+        }
+        fetch(t + kScanStep);  // in flight while this step is computed
+#pragma unroll
+        for (int i = 0; i < kScanStep; ++i) {
+            h = a[i] * h + (1.0f - a[i]) * c[i];
+            if (t + i < N) hp[(int64_t)(t + i) * H] = h;
+        }
+    }
+}
+
+// readout adjoint g and gy of the top layer: one warp per kSites sites, E = H / 32
+// units a lane
+template <int E>
+__global__ void __launch_bounds__(256) grad_readout_kernel(const __grid_constant__ GradF32Args A) {
+    constexpr int kSites = 4;
+    const int lane = threadIdx.x & 31;
+    const int M = A.n * A.N, m0 = (int)(blockIdx.x * 8 + (threadIdx.x >> 5)) * kSites;
+    if (m0 >= M) return;
+    constexpr int H = 32 * E;
+    const int top = A.nL - 1;
+    float wd[E], u[kSites][E], dy[kSites][E], d[kSites];
+    auto load = [&](const float *p, float (&v)[E]) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[e] = p[32 * e + lane];
+    };
+    load(A.pk + A.fl.wd, wd);
+#pragma unroll
+    for (int i = 0; i < kSites; ++i) {
+        const size_t o = (size_t)min(m0 + i, M - 1) * H;
+        load(A.u[top] + o, u[i]);
+        load(A.dy[top] + o, dy[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < kSites; ++i) {
+        d[i] = 0.0f;
+#pragma unroll
+        for (int e = 0; e < E; ++e) d[i] = fmaf(wd[e], u[i][e], d[i]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) d[i] += __shfl_xor_sync(0xffffffffu, d[i], o);
+    }
+    const float bd = A.pk[A.fl.bd];
+#pragma unroll
+    for (int i = 0; i < kSites; ++i) {
+        const int m = m0 + i;
+        if (m >= M) break;
+        const int s = m / A.N, t = m - s * A.N;
+        const uint64_t *row = A.bits + (int64_t)s * A.W;
+        const int sv = (int)((row[t >> 6] >> (t & 63)) & 1ull);
+        int forced = -1;  // forced sites carry no parameter dependence
+        if (A.u1) {
+            int up = 0;
+            for (int w = lane; w < (t >> 6); w += 32) up += __popcll(row[w]);
+            if (lane == 0 && (t & 63)) up += __popcll(row[t >> 6] & ((1ull << (t & 63)) - 1ull));
+            forced = u1_forced(1, A.N, t, (int)__reduce_add_sync(0xffffffffu, (unsigned)up));
+        }
+        float g = forced >= 0 ? 0.0f : 0.5f * ((float)sv - 1.0f / (1.0f + expf(-(d[i] + bd))));
+        if (A.dout) g *= A.dout[s];
+        if (lane == 0) A.g[m] = g;
+        float *gy = A.gy[top & 1] + (size_t)m * H;
+#pragma unroll
+        for (int e = 0; e < E; ++e) gy[32 * e + lane] = g * wd[e] * dy[i][e];
+    }
+}
+
+// gradient of the readout: per (sample, unit) the sum of g u over the sites
+__global__ void __launch_bounds__(128) grad_wo_kernel(const __grid_constant__ GradF32Args A) {
+    const int H = A.H, N = A.N;
+    const int64_t idx = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    const int64_t s = idx / H;
+    const int j = (int)(idx % H);
+    if (s >= A.n) return;
+    const float *u = A.u[A.nL - 1] + s * N * H + j, *g = A.g + s * N;
+    float wo = 0.0f, bo = 0.0f;
+    for (int t0 = 0; t0 < N; t0 += 16) {
+        float uv[16], gv[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const bool in = t0 + i < N;
+            uv[i] = in ? u[(int64_t)(t0 + i) * H] : 0.0f;
+            gv[i] = in ? g[t0 + i] : 0.0f;
+        }
+        float sw = 0.0f, sb = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            sw = fmaf(gv[i], uv[i], sw);
+            sb += gv[i];
+        }
+        wo += sw;
+        bo += sb;
+    }
+    float *out = A.small + s * A.small_stride;
+    // logit difference d = (W_o[1] - W_o[0]) x + (b_o[1] - b_o[0])
+    out[A.sm.Wo + j] = -wo;
+    out[A.sm.Wo + H + j] = wo;
+    if (j == 0) {
+        out[A.sm.bo] = -bo;
+        out[A.sm.bo + 1] = bo;
+    }
+}
+
+// reverse scan of a layer l >= 1: dz (in place of gh) and dc
+template <bool kResid>
+__global__ void __launch_bounds__(128) grad_scan_bwd_kernel(const __grid_constant__ GradF32Args A, int l) {
+    const int H = A.H, N = A.N;
+    const int64_t idx = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    const int64_t s = idx / H;
+    if (s >= A.n) return;
+    const int64_t base = s * N * H + idx % H;
+    float *dzp = A.gh + base, *dcp = A.dc + base;
+    const float *hp = A.h[l] + base, *ap = A.a[l] + base, *cp = A.c[l] + base;
+    const float *rp = A.gy[(l + 1) & 1] + base;
+    float lam = 0.0f, an = 0.0f;
+    float g[kScanStep], a[kScanStep], c[kScanStep], h[kScanStep], r[kScanStep];
+    auto fetch = [&](int t) {  // sites t .. t + kScanStep - 1; h one site earlier
+#pragma unroll
+        for (int i = 0; i < kScanStep; ++i) {
+            const int64_t o = (int64_t)(t + i) * H;
+            g[i] = a[i] = c[i] = h[i] = r[i] = 0.0f;
+            if (t + i >= 0) {
+                g[i] = dzp[o];
+                a[i] = ap[o];
+                c[i] = cp[o];
+                if (kResid) r[i] = rp[o];
+                if (t + i >= 1) h[i] = hp[o - H];
+            }
+        }
+    };
+    // steps end at the last site; the first one may reach before site 0
+    fetch(N - kScanStep);
+    for (int t = N - kScanStep; t > -kScanStep; t -= kScanStep) {
+        float dz[kScanStep], dc[kScanStep];
+#pragma unroll
+        for (int i = kScanStep - 1; i >= 0; --i) {
+            lam = (kResid ? g[i] + r[i] : g[i]) + an * lam;
+            dz[i] = lam * (h[i] - c[i]) * a[i] * (1.0f - a[i]);
+            dc[i] = lam * (1.0f - a[i]);
+            an = a[i];
+        }
+        fetch(t - kScanStep);
+#pragma unroll
+        for (int i = 0; i < kScanStep; ++i) {
+            if (t + i < 0) continue;
+            const int64_t o = (int64_t)(t + i) * H;
+            dzp[o] = dz[i];
+            dcp[o] = dc[i];
+        }
+    }
+}
+
+// reverse scan of layer 0 (one-hot input): the sums of dz, dc and gy by input
+// code, which are its W_z, W_h, D and bias gradients
+__global__ void __launch_bounds__(128) grad_scan_bwd0_kernel(const __grid_constant__ GradF32Args A) {
+    const int H = A.H, N = A.N;
+    const int64_t idx = (int64_t)blockIdx.x * 128 + threadIdx.x;
+    const int64_t s = idx / H;
+    const int j = (int)(idx % H);
+    if (s >= A.n) return;
+    const int64_t base = s * N * H + j;
+    const float *gp = A.gh + base, *hp = A.h[0] + base, *gyp = A.gy[0] + base;
+    const uint64_t *row = A.bits + s * A.W;
+    float ta[3], tc[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        ta[q] = A.pk[A.fl.A0 + q * H + j];
+        tc[q] = A.pk[A.fl.CD0 + q * H + j];
+    }
+    // [0]: spin before the site down, [1]: up; a step's sums first, so that
+    // their rounding grows with the square root of the steps
+    float z[2] = {0, 0}, cs[2] = {0, 0}, ds[2] = {0, 0};
+    float lam = 0.0f, an = 0.0f;
+    float g[kScanStep], h[kScanStep], gy[kScanStep];
+    unsigned up = 0;
+    auto fetch = [&](int t) {
+        up = 0;
+#pragma unroll
+        for (int i = 0; i < kScanStep; ++i) {
+            const int64_t o = (int64_t)(t + i) * H;
+            g[i] = h[i] = gy[i] = 0.0f;
+            if (t + i >= 0) {
+                g[i] = gp[o];
+                gy[i] = gyp[o];
+                if (t + i >= 1) {
+                    h[i] = hp[o - H];
+                    const int q = t + i - 1;
+                    up |= (unsigned)((row[q >> 6] >> (q & 63)) & 1ull) << i;
+                }
+            }
+        }
+    };
+    fetch(N - kScanStep);
+    float dz0 = 0.0f, dc0 = 0.0f;
+    for (int t = N - kScanStep; t > -kScanStep; t -= kScanStep) {
+        float sz[2] = {0, 0}, sc[2] = {0, 0}, sd[2] = {0, 0};
+#pragma unroll
+        for (int i = kScanStep - 1; i >= 0; --i) {
+            const bool first = t + i == 0, on = (up >> i) & 1u;
+            const float a = first ? ta[0] : on ? ta[2] : ta[1];
+            const float c = first ? tc[0] : on ? tc[2] : tc[1];
+            lam = g[i] + an * lam;
+            const float dz = lam * (h[i] - c) * a * (1.0f - a), dc = lam * (1.0f - a);
+            an = a;
+            if (t + i > 0) {
+                sz[0] += on ? 0.0f : dz;
+                sz[1] += on ? dz : 0.0f;
+                sc[0] += on ? 0.0f : dc;
+                sc[1] += on ? dc : 0.0f;
+                sd[0] += on ? 0.0f : gy[i];
+                sd[1] += on ? gy[i] : 0.0f;
+            } else if (first) {  // no input there: the biases only
+                dz0 = dz;
+                dc0 = dc;
+            }
+        }
+        fetch(t - kScanStep);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            z[q] += sz[q];
+            cs[q] += sc[q];
+            ds[q] += sd[q];
+        }
+    }
+    float *out = A.small + s * A.small_stride;
+    const GradSmall &o = A.sm;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        out[o.Wz0 + 2 * j + q] = z[q];
+        out[o.Wh0 + 2 * j + q] = cs[q];
+        out[o.D0 + 2 * j + q] = ds[q];
+    }
+    out[o.bz0 + j] = dz0 + (z[0] + z[1]);
+    out[o.bh0 + j] = dc0 + (cs[0] + cs[1]);
+}
+
+}  // namespace
+
+int grad_f32_range(int H) { return H <= 64 ? 256 : 512; }
+
+size_t grad_f32_floats_per_site(int nL, int H) { return (size_t)(5 * nL - 2 + 4) * H + 1; }
+
+int64_t grad_f32_small_floats(int H) { return 10 * (int64_t)H + 2; }
+
+cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t st) {
+    using namespace gemm;
+    const int H = A.H, M = A.n * A.N, nL = A.nL;
+    const ThetaLayout &tl = A.tl;
+    const unsigned scan_blocks = (unsigned)(((int64_t)A.n * H + 127) / 128);
+    cudaError_t e;
+    // ------------------------------------------------ forward
+    for (int l = 0; l < nL; ++l) {
+        if (l > 0) {
+            Args g{M, H, 1, {{A.u[l - 1], A.theta + tl.Wz[l], A.theta + tl.Wh[l], H, H, H}}};
+            if ((e = launch<true>(g, EpiProj{A.pk + A.fl.bz[l], A.pk + A.fl.bh[l], A.a[l], A.c[l], H}, st))) return e;
+        }
+        grad_scan_fwd_kernel<<<scan_blocks, 128, 0, st>>>(A, l);
+        if ((e = cudaGetLastError())) return e;
+        Args g{M, H, l ? 2 : 1, {{A.h[l], A.theta + tl.C[l], nullptr, H, H, H}, {}}};
+        if (l) g.seg[1] = Seg{A.u[l - 1], A.theta + tl.D[l], nullptr, H, H, H};
+        const EpiOut eo{l ? nullptr : A.pk + A.fl.DU0, l >= 2 ? A.h[l - 1] : nullptr, A.bits, A.dy[l], A.u[l], H, A.N, A.W};
+        if ((e = launch<false>(g, eo, st))) return e;
+    }
+    const unsigned ro_blocks = (unsigned)((M + 31) / 32);
+    if (H == 32) grad_readout_kernel<1><<<ro_blocks, 256, 0, st>>>(A);
+    else if (H == 64) grad_readout_kernel<2><<<ro_blocks, 256, 0, st>>>(A);
+    else grad_readout_kernel<4><<<ro_blocks, 256, 0, st>>>(A);
+    if ((e = cudaGetLastError())) return e;
+    grad_wo_kernel<<<scan_blocks, 128, 0, st>>>(A);
+    if ((e = cudaGetLastError())) return e;
+    // ------------------------------------------------ backward, top down
+    const int range = A.sum_out ? grad_f32_range(H) : A.N;
+    for (int l = nL - 1; l >= 0; --l) {
+        float *gy = A.gy[l & 1];
+        Args gc{M, H, 1, {{gy, A.pk + A.fl.CT[l], nullptr, H, H, H}}};
+        if ((e = launch<false>(gc, EpiStore{A.gh, H}, st))) return e;
+        if (l == 0) grad_scan_bwd0_kernel<<<scan_blocks, 128, 0, st>>>(A);
+        else if (l + 1 < nL) grad_scan_bwd_kernel<true><<<scan_blocks, 128, 0, st>>>(A, l);
+        else grad_scan_bwd_kernel<false><<<scan_blocks, 128, 0, st>>>(A, l);
+        if ((e = cudaGetLastError())) return e;
+        WgArgs w{};
+        w.n_pair = l ? 4 : 1;
+        w.p[0] = Pair{gy, A.h[l], H, H, H, H, H, M, tl.C[l], H, -1};
+        if (l) {
+            const float *u = A.u[l - 1];
+            w.p[1] = Pair{gy, u, H, H, H, H, H, M, tl.D[l], H, -1};
+            w.p[2] = Pair{A.gh, u, H, H, H, H, H, M, tl.Wz[l], H, tl.bz[l]};
+            w.p[3] = Pair{A.dc, u, H, H, H, H, H, M, tl.Wh[l], H, tl.bh[l]};
+        }
+        w.n_range = A.sum_out ? (M + range - 1) / range : A.n;
+        w.len = w.step = range;
+        w.seg_len = range;
+        w.seg_stride = range;
+        w.out = A.rows;
+        w.out_stride = tl.total;
+        if ((e = launch_wgrad(w, st))) return e;
+        if (l > 0) {
+            // W^T as [input unit][output unit] rows: the packed transposes
+            Args gx{M, H, 3,
+                    {{A.gh, A.pk + A.fl.WzT[l], nullptr, H, H, H},
+                     {A.dc, A.pk + A.fl.WhT[l], nullptr, H, H, H},
+                     {gy, A.pk + A.fl.DT[l], nullptr, H, H, H}}};
+            if ((e = launch<false>(gx, EpiGy{A.dy[l - 1], A.gy[(l - 1) & 1], H}, st))) return e;
+        }
+    }
+    if (!A.sum_out) return cudaSuccess;
+    SumArgs sa{};
+    sa.add = A.add;
+    sa.out = A.sum_out;
+    const int n_range = (M + range - 1) / range;
+    auto part = [&](int64_t off, int64_t len) { sa.s[sa.n++] = SumSeg{A.rows + off, tl.total, off, n_range, (int)len}; };
+    auto small = [&](int64_t src, int64_t dst, int len) {
+        sa.s[sa.n++] = SumSeg{A.small + src, A.small_stride, dst, A.n, len};
+    };
+    for (int l = 0; l < nL; ++l) {
+        if (l) part(tl.Wz[l], 4 * (int64_t)H * H + 2 * H);
+        else part(tl.C[0], (int64_t)H * H);
+    }
+    small(A.sm.Wz0, tl.Wz[0], 2 * H);
+    small(A.sm.bz0, tl.bz[0], H);
+    small(A.sm.Wh0, tl.Wh[0], 2 * H);
+    small(A.sm.bh0, tl.bh[0], H);
+    small(A.sm.D0, tl.D[0], 2 * H);
+    small(A.sm.Wo, tl.Wo, 2 * H);
+    small(A.sm.bo, tl.bo, 2);
+    return launch_sum_rows(sa, st);
+}
+
+}  // namespace psr

@@ -10,7 +10,7 @@ namespace psr {
 
 constexpr int kMaxLayers = 8;
 constexpr int kChunkF32 = 32;   // scan chunk of the FP32 SIMT path (sites)
-constexpr int kChunkGrad = 16;  // chunk of the gradient path (carries, recompute)
+constexpr int kChunkGrad = 16;  // short chunk: forward shape, carries and recompute of launch_bwd_f32
 constexpr int kChunkBF16 = 32;  // scan chunk of the tcgen05 path (sites = MMA N)
 
 // Device status word values (first error wins).
@@ -399,7 +399,40 @@ cudaError_t launch_vmc_dout(const float *eloc, const double *stats, const float 
 cudaError_t launch_adam(const float *theta, const float *grad, int64_t P, float lr, float b1, float b2,
                         float eps, int step, float *m, float *v, float *out, cudaStream_t st);
 
-// Backward (FP32).  Samples of up to kMaxGroups sample sets (one lattice
+// FP32 gradient of a batch of samples, layer by layer (psr_grad_f32.cu).
+// Arrays [n * N][H] (site-major): per layer a, c (layers >= 1), state h,
+// GELU'(y) of the pre-activation y, next input u = GELU(y); adjoints gy (two layers), gh
+// (turns into dz), dc; readout adjoint g [n * N].
+// rows: [n][P] O_k rows with small = rows, small_stride = P and sm the
+// tensors' places in theta (sum_out == NULL), or partial rows
+// [ceil(n N / grad_f32_range)][P] and per-sample entries small
+// [n][grad_f32_small_floats], summed into sum_out [P] (added to it if add).
+struct GradSmall {
+    int64_t Wz0, bz0, Wh0, bh0, D0, Wo, bo;
+};
+struct GradF32Args {
+    int n, N, W, u1, nL, H;
+    const float *theta;  // 16-byte aligned
+    ThetaLayout tl;
+    const float *pk;
+    F32Layout fl;
+    const uint64_t *bits;
+    const float *dout;
+    float *a[kMaxLayers], *c[kMaxLayers], *h[kMaxLayers], *dy[kMaxLayers], *u[kMaxLayers];
+    float *gy[2], *gh, *dc, *g;
+    float *rows, *small;
+    int64_t small_stride;
+    GradSmall sm;
+    float *sum_out;
+    bool add;
+};
+int grad_f32_range(int H);
+size_t grad_f32_floats_per_site(int nL, int H);
+int64_t grad_f32_small_floats(int H);
+cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t stream);
+
+// Backward (FP32) with chunk recompute: the gradient of samples too long for
+// launch_grad_f32's arrays.  Samples of up to kMaxGroups sample sets (one lattice
 // each) in one launch: group g holds samples first[g] .. first[g+1]-1 of the
 // launch; its chunk carries come from a forward on kChunkGrad-site chunks;
 // rows: [n][P] O_k rows (dout == NULL) or per-CTA partial sums of
