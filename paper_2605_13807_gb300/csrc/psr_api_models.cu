@@ -882,11 +882,122 @@ int psr_lru_sample(const psr_params *params, const float *uniforms, int64_t n, i
     return PSR_OK;
 }
 
+// psr_lru_grad layer by layer; PSR_ENOMEM if even a batch of one sample finds
+// no room (the caller then takes the chunk-recompute kernel).
+static int lru_grad_layers(const psr_params *params, const uint8_t *spins, int64_t n, int32_t L, const float *dout,
+                           float *dparams, int64_t B) {
+    psr_context *ctx = params->ctx;
+    const int nL = params->n_layers, H = params->hidden, N = L;
+    const int64_t P = param_count_lru(nL, H);
+    const int W = (int)words_per_row(N);
+    const bool d_theta = is_device_ptr(params->theta), d_s = is_device_ptr(spins),
+               d_dout = dout ? is_device_ptr(dout) : true, d_g = is_device_ptr(dparams);
+    const bool copy_theta = d_theta && !aligned16p(params->theta);
+    GradLruArgs A{};
+    A.N = N;
+    A.W = W;
+    A.u1 = params->u1_mask;
+    A.nL = nL;
+    A.H = H;
+    A.tl = tlru_layout(nL, H);
+    A.f = lru_layout(nL, H);
+    int64_t small_floats = 0;
+    A.sm = grad_lru_small(nL, H, &small_floats);
+    if (!dout) {  // per-sample entries go to their places in the O_k rows
+        for (int l = 0; l < nL; ++l) {
+            A.sm.nu[l] = A.tl.nu[l];
+            A.sm.th[l] = A.tl.th[l];
+            A.sm.ga[l] = A.tl.ga[l];
+            A.sm.D[l] = A.tl.D[l];
+        }
+        A.sm.Bre0 = A.tl.Bre[0];
+        A.sm.Bim0 = A.tl.Bim[0];
+        A.sm.Wo = A.tl.Wo;
+        A.sm.bo = A.tl.bo;
+    }
+    A.small_stride = dout ? small_floats : P;
+    float *theta_ws = nullptr, *dout_ws = nullptr, *g_ws = nullptr, *pk = nullptr;
+    uint8_t *s_ws = nullptr;
+    uint64_t *bits = nullptr;
+    auto carve = [&](Carver &c) {
+        theta_ws = c.get<float>(d_theta && !copy_theta ? 0 : P);
+        s_ws = c.get<uint8_t>(d_s ? 0 : (size_t)n * N);
+        dout_ws = c.get<float>(d_dout ? 0 : n);
+        g_ws = c.get<float>(d_g ? 0 : (dout ? P : (size_t)n * P));
+        pk = c.get<float>(A.f.total);
+        bits = c.get<uint64_t>((size_t)n * W);
+        const size_t M = (size_t)B * N, arr = M * H;
+        for (int l = 0; l < nL; ++l) {
+            A.br[l] = c.get<float>(l ? arr : 0);
+            A.bi[l] = c.get<float>(l ? arr : 0);
+            float **per[] = {&A.hr[l], &A.hn[l], &A.y[l], &A.p1[l], &A.p2[l], &A.x[l]};
+            for (float **p : per) *p = c.get<float>(arr);
+        }
+        float **adj[] = {&A.gx, &A.da, &A.dg, &A.dy, &A.dhr, &A.dhi};
+        for (float **p : adj) *p = c.get<float>(arr);
+        A.g = c.get<float>(M);
+        const size_t range = grad_f32_range(H);
+        A.rows = c.get<float>(dout ? (M + range - 1) / range * P : 0);
+        A.small = c.get<float>(dout ? (size_t)B * small_floats : 0);
+    };
+    int rc = PSR_ENOMEM;
+    for (; B > 0; B /= 2) {
+        Carver sz;
+        carve(sz);
+        if ((rc = ensure_ws(ctx, sz.off)) != PSR_ENOMEM) break;
+    }
+    if (rc != PSR_OK) return rc;
+    Carver cv;
+    cv.base = static_cast<char *>(ctx->ws);
+    carve(cv);
+    cudaStream_t st = ctx->stream;
+    const float *theta = nullptr, *dv = nullptr;
+    const uint8_t *sp = nullptr;
+    if ((rc = stage_in(params->theta, theta_ws, P, d_theta, st, &theta)) != PSR_OK) return rc;
+    if (copy_theta) {
+        PSR_TRY(cudaMemcpyAsync(theta_ws, theta, P * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        theta = theta_ws;
+    }
+    if ((rc = stage_in(spins, s_ws, (size_t)n * N, d_s, st, &sp)) != PSR_OK) return rc;
+    if (dout && (rc = stage_in(dout, dout_ws, n, d_dout, st, &dv)) != PSR_OK) return rc;
+    float *g = d_g ? dparams : g_ws;
+    reset_stages(ctx);
+    {
+        StageScope sc(ctx, PSR_STAGE_PACK);
+        PSR_TRY(launch_pack_theta_lru(theta, A.f, pk, st));
+        PSR_TRY(launch_bitpack(sp, n, N, W, bits, ctx->status, st));  // spin-byte check
+    }
+    {
+        StageScope sc(ctx, PSR_STAGE_BWD);  // the layers' forward and the reverse pass
+        A.theta = theta;
+        A.pk = pk;
+        A.sum_out = dout ? g : nullptr;
+        for (int64_t s0 = 0; s0 < n; s0 += B) {
+            A.n = (int)(n - s0 < B ? n - s0 : B);
+            A.bits = bits + s0 * W;
+            A.dout = dout ? dv + s0 : nullptr;
+            if (!dout) A.rows = A.small = g + s0 * P;
+            A.add = s0 > 0;
+            PSR_TRY(launch_grad_lru(A, st));
+        }
+    }
+    if (!d_g)
+        PSR_TRY(cudaMemcpyAsync(dparams, g_ws, (dout ? P : (size_t)n * P) * sizeof(float),
+                                cudaMemcpyDeviceToHost, st));
+    if (!d_g || !d_s || !d_theta || !d_dout) return take_status(ctx);
+    return PSR_OK;
+}
+
 int psr_lru_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_t L, const float *dout,
                  float *dparams) {
     int rc = check_params_lru(params, n, L);
     if (rc != PSR_OK) return rc;
     if (!spins || !dparams) return PSR_EINVAL;
+    const size_t per = grad_lru_floats_per_site(params->n_layers, params->hidden) * (size_t)L;
+    if (const int64_t B = grad_batch(per, L, n)) {
+        rc = lru_grad_layers(params, spins, n, L, dout, dparams, B);
+        if (rc != PSR_ENOMEM) return rc;
+    }
     psr_context *ctx = params->ctx;
     const int nL = params->n_layers, H = params->hidden, N = L;
     const int64_t P = param_count_lru(nL, H);

@@ -1,5 +1,7 @@
 // Reverse-mode gradient d log psi / d theta of the deep 1D LRU ansatz
-// (Sec. II.B Eq. lru, Sec. II.G 1D residual, Sec. III.B GLU blocks), FP32.
+// (Sec. II.B Eq. lru, Sec. II.G 1D residual, Sec. III.B GLU blocks), FP32, with
+// chunk recompute: the form for samples whose layer arrays would not fit
+// (psr_grad_lru.cu is the fast one; this one keeps only chunk carries).
 //
 // One CTA per sample (grid-stride), thread j owns hidden unit j.  Chunks of
 // 32 sites are visited from the last to the first; each is recomputed from

@@ -55,12 +55,14 @@ struct Args {
     Seg seg[kMaxSeg];
 };
 
+// two stages; the epilogue's tile of BM x (BN + 8) floats reuses them
 constexpr size_t smem_bytes(int BN) { return (size_t)2 * (BM + BN) * LDT * sizeof(float); }
 constexpr int threads(int BN) { return BN == 128 ? 256 : 128; }
 
 // BN columns per tile (a pair is two).  A warp covers 4 x 8 lanes; lane
 // (ty, tx) of warp (wm, wn) owns sites 16 i + 4 wm + ty and columns 64 wn + tx
-// + 8 j.  Epi: row(m) -> per-site context, then one call per unit.
+// + 8 j.  Epi: load(m, u) -> what the four units u .. u + 3 of site m need
+// from memory, then store(m, u, values[, second values], loaded).
 template <int BN, bool kPair, class Epi>
 __global__ void __launch_bounds__(threads(BN), BN == 128 ? 2 : 4)
     gemm_kernel(const __grid_constant__ Args g, const __grid_constant__ Epi epi) {
@@ -135,21 +137,73 @@ __global__ void __launch_bounds__(threads(BN), BN == 128 ? 2 : 4)
         }
         __syncthreads();
     }
+    // The tile goes through shared memory, so that the epilogue reads and
+    // writes whole rows (16 bytes a lane) and the reads of kRows rows are in
+    // flight together; straight from the registers (32-byte pieces, one row
+    // after another) the epilogues that read arrays took up to twice as long.
+    constexpr int C = kPair ? BN / 2 : BN;  // units of the tile
+    constexpr int LDC = BN + 8;             // 8 x 4 lanes of a store hit 32 banks
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-        const int m = m0 + 16 * i + 4 * wm + ty;
-        if (m >= g.M) break;
-        const auto ctx = epi.row(m);
-        if constexpr (kPair) {
+        float *row = smem + (16 * i + 4 * wm + ty) * LDC;
 #pragma unroll
-            for (int j = 0; j < TN; j += 2)
-                epi(ctx, m, u0 + 32 * wn + tx + 4 * j, acc[i][j], acc[i][j + 1]);
-        } else {
+        for (int j = 0; j < TN; ++j) {
+            if constexpr (kPair) row[(j & 1) * C + 32 * wn + 8 * (j >> 1) + tx] = acc[i][j];
+            else row[64 * wn + 8 * j + tx] = acc[i][j];
+        }
+    }
+    __syncthreads();
+    constexpr int kQuads = C / 4, kStep = T / kQuads, kRows = 4;
+    static_assert(BM % (kStep * kRows) == 0, "whole groups of rows");
+    const int q = (tid % kQuads) * 4, r0 = tid / kQuads;
+    const int u = u0 + q;
+#pragma unroll 1
+    for (int r = r0; r < BM; r += kStep * kRows) {
+        typename Epi::In in[kRows];
 #pragma unroll
-            for (int j = 0; j < TN; ++j) epi(ctx, m, u0 + 64 * wn + tx + 8 * j, acc[i][j]);
+        for (int k = 0; k < kRows; ++k) in[k] = epi.load(min(m0 + r + k * kStep, g.M - 1), u);
+#pragma unroll
+        for (int k = 0; k < kRows; ++k) {
+            const int m = m0 + r + k * kStep;
+            if (m >= g.M) break;
+            const float *row = smem + (r + k * kStep) * LDC + q;
+            const float4 v = *reinterpret_cast<const float4 *>(row);
+            if constexpr (kPair) epi.store(m, u, v, *reinterpret_cast<const float4 *>(row + C), in[k]);
+            else epi.store(m, u, v, in[k]);
         }
     }
 }
+
+// element-wise helpers of the epilogues, four units at a time
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ void st4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
+template <class F>
+__device__ __forceinline__ float4 map4(F f, float4 a) {
+    return make_float4(f(a.x), f(a.y), f(a.z), f(a.w));
+}
+template <class F>
+__device__ __forceinline__ float4 map4(F f, float4 a, float4 b) {
+    return make_float4(f(a.x, b.x), f(a.y, b.y), f(a.z, b.z), f(a.w, b.w));
+}
+__device__ __forceinline__ float4 add4(float4 a, float4 b) {
+    return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+__device__ __forceinline__ float4 mul4(float4 a, float4 b) {
+    return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
+}
+__device__ __forceinline__ float4 fma4(float4 a, float4 b, float4 c) {
+    return make_float4(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y), fmaf(a.z, b.z, c.z), fmaf(a.w, b.w, c.w));
+}
+
+struct NoIn {};
+
+struct EpiStore {  // out = the product
+    using In = NoIn;
+    float *out;
+    int H;
+    __device__ NoIn load(int, int) const { return {}; }
+    __device__ void store(int m, int j, float4 v, NoIn) const { st4(out + (size_t)m * H + j, v); }
+};
 
 template <int BN, bool kPair, class Epi>
 inline cudaError_t launch_bn(const Args &g, const Epi &epi, cudaStream_t st) {

@@ -16,76 +16,71 @@
 //
 // What bounds it: the FP32 rate in the products (54 H^2 operations a site) and
 // HBM for the arrays between them (about 75 arrays of 4 H bytes a site): at
-// hidden 64, 4096 samples of 100 sites (weighted sum) 2.4 ms of the 3.1 ms are
-// products at 31 to 46 TFLOP/s, the rest streams.  The chunk-recompute kernel
+// hidden 64, 4096 samples of 100 sites (weighted sum) 2.1 ms of the 2.9 ms are
+// products at 33 to 46 TFLOP/s, the rest streams.  The chunk-recompute kernel
 // (psr_bwd.cu: a CTA per sample, a thread per unit, the sum by reductions in
 // L2 every 16 sites) takes 11.3 ms there.
 #include <cuda_runtime.h>
 
 #include "psr_device.cuh"
 #include "psr_gemm.cuh"
+#include "psr_grad_common.cuh"
 #include "psr_internal.cuh"
 
 namespace psr {
 
 namespace {
 
-// input code of site t: 0 at the first site, 1 + s_{t-1} otherwise
-__device__ __forceinline__ int code_at(const uint64_t *row, int t) {
-    return t == 0 ? 0 : 1 + (int)((row[(t - 1) >> 6] >> ((t - 1) & 63)) & 1ull);
-}
-
-struct NoCtx {};
+using namespace gemm;
 
 struct EpiProj {  // a = sigmoid(z), c
+    using In = NoIn;
     const float *bz, *bh;
     float *a, *c;
     int H;
-    __device__ NoCtx row(int) const { return {}; }
-    __device__ void operator()(NoCtx, int m, int u, float z, float cc) const {
+    __device__ NoIn load(int, int) const { return {}; }
+    __device__ void store(int m, int u, float4 z, float4 cc, NoIn) const {
         const size_t i = (size_t)m * H + u;
-        a[i] = sigmoid_f(z + bz[u]);
-        c[i] = cc + bh[u];
+        st4(a + i, map4(sigmoid_f, add4(z, ld4(bz + u))));
+        st4(c + i, add4(cc, ld4(bh + u)));
     }
 };
 
 struct EpiOut {  // the next layer's input u = GELU(y), and GELU'(y) for the way back
+    struct In {
+        float4 more;  // layer 0: D of the one-hot input; l >= 2: h of the layer below
+    };
     const float *du0;      // layer 0: D of the one-hot input by code, else null
     const float *h_below;  // residual, or null
     const uint64_t *bits;
     float *dy, *u;
     int H, N, W;
-    __device__ int row(int m) const {
-        if (!du0) return 0;
-        const int s = m / N;
-        return code_at(bits + (int64_t)s * W, m - s * N);
+    __device__ In load(int m, int j) const {
+        if (du0) {
+            const int s = m / N;
+            return {ld4(du0 + code_at(bits + (int64_t)s * W, m - s * N) * H + j)};
+        }
+        return {h_below ? ld4(h_below + (size_t)m * H + j) : make_float4(0.0f, 0.0f, 0.0f, 0.0f)};
     }
-    __device__ void operator()(int code, int m, int j, float v) const {
+    __device__ void store(int m, int j, float4 v, In in) const {
         const size_t i = (size_t)m * H + j;
-        if (du0) v += du0[code * H + j];
-        if (h_below) v += h_below[i];
-        const float cdf = 0.5f * (1.0f + erff(v * 0.70710678118654752f));
-        u[i] = v * cdf;
-        dy[i] = fmaf(v * 0.39894228040143268f, expf(-0.5f * v * v), cdf);
+        v = add4(v, in.more);
+        const float4 cdf = map4([](float x) { return 0.5f * (1.0f + erff(x * 0.70710678118654752f)); }, v);
+        st4(u + i, mul4(v, cdf));
+        st4(dy + i, fma4(map4([](float x) { return x * 0.39894228040143268f; }, v),
+                         map4([](float x) { return expf(-0.5f * x * x); }, v), cdf));
     }
-};
-
-struct EpiStore {
-    float *out;
-    int H;
-    __device__ NoCtx row(int) const { return {}; }
-    __device__ void operator()(NoCtx, int m, int j, float v) const { out[(size_t)m * H + j] = v; }
 };
 
 struct EpiGy {  // adjoint of the pre-activation of the layer below
+    struct In {
+        float4 dy;
+    };
     const float *dy;
     float *gy;
     int H;
-    __device__ NoCtx row(int) const { return {}; }
-    __device__ void operator()(NoCtx, int m, int j, float v) const {
-        const size_t i = (size_t)m * H + j;
-        gy[i] = v * dy[i];
-    }
+    __device__ In load(int m, int j) const { return {ld4(dy + (size_t)m * H + j)}; }
+    __device__ void store(int m, int j, float4 v, In in) const { st4(gy + (size_t)m * H + j, mul4(v, in.dy)); }
 };
 
 constexpr int kScanStep = 8;
@@ -144,95 +139,11 @@ __global__ void __launch_bounds__(128) grad_scan_fwd_kernel(const __grid_constan
     }
 }
 
-// readout adjoint g and gy of the top layer: one warp per kSites sites, E = H / 32
-// units a lane
-template <int E>
-__global__ void __launch_bounds__(256) grad_readout_kernel(const __grid_constant__ GradF32Args A) {
-    constexpr int kSites = 4;
-    const int lane = threadIdx.x & 31;
-    const int M = A.n * A.N, m0 = (int)(blockIdx.x * 8 + (threadIdx.x >> 5)) * kSites;
-    if (m0 >= M) return;
-    constexpr int H = 32 * E;
-    const int top = A.nL - 1;
-    float wd[E], u[kSites][E], dy[kSites][E], d[kSites];
-    auto load = [&](const float *p, float (&v)[E]) {
-#pragma unroll
-        for (int e = 0; e < E; ++e) v[e] = p[32 * e + lane];
-    };
-    load(A.pk + A.fl.wd, wd);
-#pragma unroll
-    for (int i = 0; i < kSites; ++i) {
-        const size_t o = (size_t)min(m0 + i, M - 1) * H;
-        load(A.u[top] + o, u[i]);
-        load(A.dy[top] + o, dy[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < kSites; ++i) {
-        d[i] = 0.0f;
-#pragma unroll
-        for (int e = 0; e < E; ++e) d[i] = fmaf(wd[e], u[i][e], d[i]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) d[i] += __shfl_xor_sync(0xffffffffu, d[i], o);
-    }
-    const float bd = A.pk[A.fl.bd];
-#pragma unroll
-    for (int i = 0; i < kSites; ++i) {
-        const int m = m0 + i;
-        if (m >= M) break;
-        const int s = m / A.N, t = m - s * A.N;
-        const uint64_t *row = A.bits + (int64_t)s * A.W;
-        const int sv = (int)((row[t >> 6] >> (t & 63)) & 1ull);
-        int forced = -1;  // forced sites carry no parameter dependence
-        if (A.u1) {
-            int up = 0;
-            for (int w = lane; w < (t >> 6); w += 32) up += __popcll(row[w]);
-            if (lane == 0 && (t & 63)) up += __popcll(row[t >> 6] & ((1ull << (t & 63)) - 1ull));
-            forced = u1_forced(1, A.N, t, (int)__reduce_add_sync(0xffffffffu, (unsigned)up));
-        }
-        float g = forced >= 0 ? 0.0f : 0.5f * ((float)sv - 1.0f / (1.0f + expf(-(d[i] + bd))));
-        if (A.dout) g *= A.dout[s];
-        if (lane == 0) A.g[m] = g;
-        float *gy = A.gy[top & 1] + (size_t)m * H;
-#pragma unroll
-        for (int e = 0; e < E; ++e) gy[32 * e + lane] = g * wd[e] * dy[i][e];
-    }
-}
-
-// gradient of the readout: per (sample, unit) the sum of g u over the sites
-__global__ void __launch_bounds__(128) grad_wo_kernel(const __grid_constant__ GradF32Args A) {
-    const int H = A.H, N = A.N;
-    const int64_t idx = (int64_t)blockIdx.x * 128 + threadIdx.x;
-    const int64_t s = idx / H;
-    const int j = (int)(idx % H);
-    if (s >= A.n) return;
-    const float *u = A.u[A.nL - 1] + s * N * H + j, *g = A.g + s * N;
-    float wo = 0.0f, bo = 0.0f;
-    for (int t0 = 0; t0 < N; t0 += 16) {
-        float uv[16], gv[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const bool in = t0 + i < N;
-            uv[i] = in ? u[(int64_t)(t0 + i) * H] : 0.0f;
-            gv[i] = in ? g[t0 + i] : 0.0f;
-        }
-        float sw = 0.0f, sb = 0.0f;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            sw = fmaf(gv[i], uv[i], sw);
-            sb += gv[i];
-        }
-        wo += sw;
-        bo += sb;
-    }
-    float *out = A.small + s * A.small_stride;
-    // logit difference d = (W_o[1] - W_o[0]) x + (b_o[1] - b_o[0])
-    out[A.sm.Wo + j] = -wo;
-    out[A.sm.Wo + H + j] = wo;
-    if (j == 0) {
-        out[A.sm.bo] = -bo;
-        out[A.sm.bo + 1] = bo;
-    }
-}
+struct TopGy {  // gy of the top layer from gx = g wd
+    const float *dy;
+    float *gy;
+    __device__ void operator()(size_t i, float gx) const { gy[i] = gx * dy[i]; }
+};
 
 // reverse scan of a layer l >= 1: dz (in place of gh) and dc
 template <bool kResid>
@@ -376,7 +287,6 @@ size_t grad_f32_floats_per_site(int nL, int H) { return (size_t)(5 * nL - 2 + 4)
 int64_t grad_f32_small_floats(int H) { return 10 * (int64_t)H + 2; }
 
 cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t st) {
-    using namespace gemm;
     const int H = A.H, M = A.n * A.N, nL = A.nL;
     const ThetaLayout &tl = A.tl;
     const unsigned scan_blocks = (unsigned)(((int64_t)A.n * H + 127) / 128);
@@ -394,13 +304,9 @@ cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t st) {
         const EpiOut eo{l ? nullptr : A.pk + A.fl.DU0, l >= 2 ? A.h[l - 1] : nullptr, A.bits, A.dy[l], A.u[l], H, A.N, A.W};
         if ((e = launch<false>(g, eo, st))) return e;
     }
-    const unsigned ro_blocks = (unsigned)((M + 31) / 32);
-    if (H == 32) grad_readout_kernel<1><<<ro_blocks, 256, 0, st>>>(A);
-    else if (H == 64) grad_readout_kernel<2><<<ro_blocks, 256, 0, st>>>(A);
-    else grad_readout_kernel<4><<<ro_blocks, 256, 0, st>>>(A);
-    if ((e = cudaGetLastError())) return e;
-    grad_wo_kernel<<<scan_blocks, 128, 0, st>>>(A);
-    if ((e = cudaGetLastError())) return e;
+    const ReadoutArgs ro{A.n, A.N, H, A.W, A.u1, A.bits, A.u[nL - 1], A.pk + A.fl.wd, A.pk + A.fl.bd, A.dout, A.g,
+                         A.small + A.sm.Wo, A.small + A.sm.bo, A.small_stride};
+    if ((e = launch_readout(ro, TopGy{A.dy[nL - 1], A.gy[(nL - 1) & 1]}, st))) return e;
     // ------------------------------------------------ backward, top down
     const int range = A.sum_out ? grad_f32_range(H) : A.N;
     for (int l = nL - 1; l >= 0; --l) {

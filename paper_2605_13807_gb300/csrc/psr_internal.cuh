@@ -431,6 +431,34 @@ size_t grad_f32_floats_per_site(int nL, int H);
 int64_t grad_f32_small_floats(int H);
 cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t stream);
 
+// FP32 gradient of the LRU over a batch of samples, layer by layer
+// (psr_grad_lru.cu); arrays, rows and sums as for launch_grad_f32.  Per layer
+// br, bi (layers >= 1), hr, hn (state, imaginary part negated), y, p1, p2
+// (GLU derivatives), output x; adjoints gx, da, dg, dy, dhr, dhi; g.
+struct GradLruSmall {
+    int64_t nu[kMaxLayers], th[kMaxLayers], ga[kMaxLayers], D[kMaxLayers], Bre0, Bim0, Wo, bo;
+};
+struct GradLruArgs {
+    int n, N, W, u1, nL, H;
+    const float *theta;  // 16-byte aligned
+    TLruLayout tl;
+    const float *pk;
+    LruLayout f;
+    const uint64_t *bits;
+    const float *dout;
+    float *br[kMaxLayers], *bi[kMaxLayers], *hr[kMaxLayers], *hn[kMaxLayers], *y[kMaxLayers];
+    float *p1[kMaxLayers], *p2[kMaxLayers], *x[kMaxLayers];
+    float *gx, *da, *dg, *dy, *dhr, *dhi, *g;
+    float *rows, *small;
+    int64_t small_stride;
+    GradLruSmall sm;
+    float *sum_out;
+    bool add;
+};
+size_t grad_lru_floats_per_site(int nL, int H);
+GradLruSmall grad_lru_small(int nL, int H, int64_t *floats);
+cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t stream);
+
 // Backward (FP32) with chunk recompute: the gradient of samples too long for
 // launch_grad_f32's arrays.  Samples of up to kMaxGroups sample sets (one lattice
 // each) in one launch: group g holds samples first[g] .. first[g+1]-1 of the
