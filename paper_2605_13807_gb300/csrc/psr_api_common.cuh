@@ -9,6 +9,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <vector>
 
@@ -483,6 +484,13 @@ inline int enqueue_grad_f32(psr_context *ctx, int nL, int H, int u1, const float
     }
     return PSR_OK;
 }
+
+// psr2d_grad whose weights depend on log psi of the same samples: one forward
+// for both (psr_api_models.cu).  lp [n] receives log psi, then weights(stream)
+// enqueues what writes dout [n].  PSR_ENOMEM, with nothing enqueued, if the
+// samples do not fit one batch.  Device arrays only.
+int grad2d_after_logpsi(const psr_params *params, const uint8_t *spins, int64_t n, int32_t Lx, int32_t Ly, float *lp,
+                        const std::function<cudaError_t(cudaStream_t)> &weights, const float *dout, float *dparams);
 
 }  // namespace apiutil
 }  // namespace psr

@@ -228,11 +228,120 @@ int psr2d_sample(const psr_params *params, const float *uniforms, int64_t n, int
     return PSR_OK;
 }
 
+// Samples per batch of the layer-by-layer gradient, 0 if one does not fit.
+static int64_t grad2d_batch(const psr_params *params, int64_t n, int32_t Lx, int32_t Ly) {
+    const int64_t Np = (int64_t)(Lx / 2) * (Ly / 2);
+    return grad_batch(grad2d_floats_per_site(params->n_layers, params->hidden) * (size_t)Np, Np, n);
+}
+
+// psr2d_grad layer by layer; PSR_ENOMEM if even a batch of one sample finds no
+// room (the caller then takes the row-recompute kernel).  With `weights`, one
+// batch holds all samples (else PSR_ENOMEM): lp8 [n] receives log psi after the
+// forward, then weights(stream) enqueues what makes dout from it.
+static int grad2d_layers(const psr_params *params, const uint8_t *spins, int64_t n, int32_t Lx, int32_t Ly,
+                         const float *dout, float *dparams, int64_t B, float *lp8,
+                         const std::function<cudaError_t(cudaStream_t)> *weights) {
+    psr_context *ctx = params->ctx;
+    const int nL = params->n_layers, H = params->hidden, N = Lx * Ly;
+    const int64_t P = param_count2d(nL, H);
+    const int W = (int)words_per_row(N);
+    const bool d_theta = is_device_ptr(params->theta), d_s = is_device_ptr(spins),
+               d_dout = dout ? is_device_ptr(dout) : true, d_g = is_device_ptr(dparams);
+    const bool copy_theta = d_theta && !aligned16p(params->theta);
+    Grad2dArgs A{};
+    A.Lx = Lx;
+    A.Ly = Ly;
+    A.W = W;
+    A.u1 = params->u1_mask;
+    A.nL = nL;
+    A.H = H;
+    A.tl = t2_layout(nL, H);
+    A.f = f2_layout(nL, H);
+    float *theta_ws = nullptr, *dout_ws = nullptr, *g_ws = nullptr, *pk = nullptr;
+    uint8_t *s_ws = nullptr;
+    uint64_t *bits = nullptr;
+    auto carve = [&](Carver &c) {
+        theta_ws = c.get<float>(d_theta && !copy_theta ? 0 : P);
+        s_ws = c.get<uint8_t>(d_s ? 0 : (size_t)n * N);
+        dout_ws = c.get<float>(d_dout ? 0 : n);
+        g_ws = c.get<float>(d_g ? 0 : (dout ? P : (size_t)n * P));
+        pk = c.get<float>(A.f.total);
+        bits = c.get<uint64_t>((size_t)n * W);
+        const size_t M = (size_t)B * (N / 4), arr = M * H;
+        for (int l = 0; l < nL; ++l) {
+            float **per[] = {&A.a[l], &A.c[l], &A.h[l], &A.dy[l], &A.x[l]};
+            for (float **p : per) *p = c.get<float>(arr);
+        }
+        float **adj[] = {&A.gy[0], &A.gy[1], &A.gh, &A.dc};
+        for (float **p : adj) *p = c.get<float>(arr);
+        float **wide[] = {&A.u0, &A.logits, &A.g};
+        for (float **p : wide) *p = c.get<float>(M * 32);
+        A.logp = c.get<float>(M);
+        A.wo32 = c.get<float>(32 * (size_t)H);
+        A.wo32t = c.get<float>(32 * (size_t)H);
+        const size_t range = grad_f32_range(H);
+        A.rows = c.get<float>(dout ? (M + range - 1) / range * P : 0);
+    };
+    if (weights && B < n) return PSR_ENOMEM;
+    int rc = PSR_ENOMEM;
+    for (; B > 0; B /= 2) {
+        Carver sz;
+        carve(sz);
+        if ((rc = ensure_ws(ctx, sz.off)) != PSR_ENOMEM || weights) break;
+    }
+    if (rc != PSR_OK) return rc;
+    Carver cv;
+    cv.base = static_cast<char *>(ctx->ws);
+    carve(cv);
+    cudaStream_t st = ctx->stream;
+    const float *theta = nullptr, *dv = nullptr;
+    const uint8_t *sp = nullptr;
+    if ((rc = stage_in(params->theta, theta_ws, P, d_theta, st, &theta)) != PSR_OK) return rc;
+    if (copy_theta) {
+        PSR_TRY(cudaMemcpyAsync(theta_ws, theta, P * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        theta = theta_ws;
+    }
+    if ((rc = stage_in(spins, s_ws, (size_t)n * N, d_s, st, &sp)) != PSR_OK) return rc;
+    if (dout && (rc = stage_in(dout, dout_ws, n, d_dout, st, &dv)) != PSR_OK) return rc;
+    float *g = d_g ? dparams : g_ws;
+    reset_stages(ctx);
+    {
+        StageScope sc(ctx, PSR_STAGE_PACK);
+        PSR_TRY(launch_pack_theta_f2(theta, A.f, pk, st));
+        PSR_TRY(launch_bitpack(sp, n, N, W, bits, ctx->status, st));  // spin-byte check
+    }
+    {
+        StageScope sc(ctx, PSR_STAGE_BWD);  // the layers' forward and the reverse pass
+        A.theta = theta;
+        A.pk = pk;
+        A.sum_out = dout ? g : nullptr;
+        for (int64_t s0 = 0; s0 < n; s0 += B) {
+            A.n = (int)(n - s0 < B ? n - s0 : B);
+            A.bits = bits + s0 * W;
+            A.dout = dout ? dv + s0 : nullptr;
+            if (!dout) A.rows = g + s0 * P;
+            A.add = s0 > 0;
+            PSR_TRY(launch_grad2d_fwd(A, lp8, st));
+            if (weights) PSR_TRY((*weights)(st));
+            PSR_TRY(launch_grad2d_bwd(A, st));
+        }
+    }
+    if (!d_g)
+        PSR_TRY(cudaMemcpyAsync(dparams, g_ws, (dout ? P : (size_t)n * P) * sizeof(float),
+                                cudaMemcpyDeviceToHost, st));
+    if (!d_g || !d_s || !d_theta || !d_dout) return take_status(ctx);
+    return PSR_OK;
+}
+
 int psr2d_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_t Lx, int32_t Ly,
                const float *dout, float *dparams) {
     int rc = check_params2d(params, n, Lx, Ly);
     if (rc != PSR_OK) return rc;
     if (!spins || !dparams) return PSR_EINVAL;
+    if (const int64_t B = grad2d_batch(params, n, Lx, Ly)) {
+        rc = grad2d_layers(params, spins, n, Lx, Ly, dout, dparams, B, nullptr, nullptr);
+        if (rc != PSR_ENOMEM) return rc;
+    }
     psr_context *ctx = params->ctx;
     const int nL = params->n_layers, H = params->hidden, N = Lx * Ly, Py = Ly / 2;
     const int64_t P = param_count2d(nL, H);
@@ -1085,3 +1194,12 @@ int psr_lru_grad(const psr_params *params, const uint8_t *spins, int64_t n, int3
 }
 
 }  // extern "C"
+
+// Declared in psr_api_common.cuh.
+int psr::apiutil::grad2d_after_logpsi(const psr_params *params, const uint8_t *spins, int64_t n, int32_t Lx, int32_t Ly,
+                                      float *lp, const std::function<cudaError_t(cudaStream_t)> &weights,
+                                      const float *dout, float *dparams) {
+    const int64_t B = grad2d_batch(params, n, Lx, Ly);
+    if (B < n) return PSR_ENOMEM;
+    return grad2d_layers(params, spins, n, Lx, Ly, dout, dparams, B, lp, &weights);
+}

@@ -391,15 +391,23 @@ int psr2d_vmc_step(const psr_params *params, const psr_hamiltonian *ham, int32_t
     rc = symmetrize ? psr2d_sym_local_energy(params, used, n, ham, eloc, stats)
                     : psr2d_local_energy(params, used, n, ham, eloc, stats);
     if (rc != PSR_OK) return rc;
-    // 3. centred energy-gradient weights (per image when symmetrised)
+    // 3. centred energy-gradient weights (per image when symmetrised) and
+    // 4. gradient sum_i dout_i d log psi(s_i) / d theta; the image weights need
+    // log psi of the images, which the gradient's own forward gives
+    const auto weights = [&](cudaStream_t s) { return launch_vmc_dout(eloc, stats, lp8, n, n_img, dout, s); };
     if (symmetrize) {
         PSR_TRY(launch_c4v_images(used, n, Lx, imgs, st));
-        if ((rc = psr2d_logpsi(&p32, imgs, 8 * n, Lx, Ly, lp8)) != PSR_OK) return rc;
+        rc = grad2d_after_logpsi(&p32, imgs, 8 * n, Lx, Ly, lp8, weights, dout, grad);
+        if (rc == PSR_ENOMEM) {
+            if ((rc = psr2d_logpsi(&p32, imgs, 8 * n, Lx, Ly, lp8)) != PSR_OK) return rc;
+            PSR_TRY(weights(st));
+            rc = psr2d_grad(&p32, imgs, 8 * n, Lx, Ly, dout, grad);
+        }
+    } else {
+        PSR_TRY(weights(st));
+        rc = psr2d_grad(&p32, used, n, Lx, Ly, dout, grad);
     }
-    PSR_TRY(launch_vmc_dout(eloc, stats, lp8, n, n_img, dout, st));
-    // 4. gradient sum_i dout_i d log psi(s_i) / d theta
-    if ((rc = psr2d_grad(&p32, symmetrize ? imgs : used, n_img * n, Lx, Ly, dout, grad)) != PSR_OK)
-        return rc;
+    if (rc != PSR_OK) return rc;
     // 5. Adam update
     PSR_TRY(launch_adam(params->theta, grad, P, adam->lr, adam->beta1, adam->beta2, adam->eps,
                         adam->step, adam->m, adam->v, theta_out, st));

@@ -1,6 +1,8 @@
 // Reverse-mode gradient d log psi / d theta of the 2D patched minGRU
 // (Sec. II.F two-dimensional recurrences, Sec. II.G residual; the gradient
-// the VMC energy estimator needs, Sec. III.B), FP32.
+// the VMC energy estimator needs, Sec. III.B), FP32, with row recompute: the
+// form for samples whose layer arrays would not fit (psr_grad2d.cu is the fast
+// one; this one keeps only row checkpoints).
 //
 // One CTA per sample (grid-stride); thread j owns hidden unit j.  Patch rows
 // are visited from the last to the first.  A row is first recomputed from

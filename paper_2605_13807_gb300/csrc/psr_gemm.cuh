@@ -46,7 +46,7 @@ __device__ __forceinline__ void cp_wait() {
 // has two rows, W0[u] and W1[u], and one thread ends with both.
 struct Seg {
     const float *A, *W0, *W1;
-    int K, lda, ldw;
+    int K, lda, ldw, ldw1;
 };
 struct Args {
     int M;      // sites
@@ -97,8 +97,11 @@ __global__ void __launch_bounds__(threads(BN), BN == 128 ? 2 : 4)
             for (int r = 0; r < BN; r += T / 8) {
                 const int n = lrow + r;
                 if (BN < T / 8 && n >= BN) break;
-                const float *w = !kPair ? s.W0 + (size_t)(u0 + n) * s.ldw
-                                        : (n & 8 ? s.W1 : s.W0) + (size_t)(u0 + (n & 7) + 8 * (n >> 4)) * s.ldw;
+                const float *w = s.W0 + (size_t)(u0 + n) * s.ldw;
+                if constexpr (kPair) {
+                    const size_t u = u0 + (n & 7) + 8 * (n >> 4);
+                    w = n & 8 ? s.W1 + u * s.ldw1 : s.W0 + u * s.ldw;
+                }
                 cp16(ws + n * LDT + lcol, w + k_next + lcol);
             }
             k_next += BK;

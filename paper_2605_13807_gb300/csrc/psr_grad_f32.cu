@@ -294,13 +294,13 @@ cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t st) {
     // ------------------------------------------------ forward
     for (int l = 0; l < nL; ++l) {
         if (l > 0) {
-            Args g{M, H, 1, {{A.u[l - 1], A.theta + tl.Wz[l], A.theta + tl.Wh[l], H, H, H}}};
+            Args g{M, H, 1, {{A.u[l - 1], A.theta + tl.Wz[l], A.theta + tl.Wh[l], H, H, H, H}}};
             if ((e = launch<true>(g, EpiProj{A.pk + A.fl.bz[l], A.pk + A.fl.bh[l], A.a[l], A.c[l], H}, st))) return e;
         }
         grad_scan_fwd_kernel<<<scan_blocks, 128, 0, st>>>(A, l);
         if ((e = cudaGetLastError())) return e;
-        Args g{M, H, l ? 2 : 1, {{A.h[l], A.theta + tl.C[l], nullptr, H, H, H}, {}}};
-        if (l) g.seg[1] = Seg{A.u[l - 1], A.theta + tl.D[l], nullptr, H, H, H};
+        Args g{M, H, l ? 2 : 1, {{A.h[l], A.theta + tl.C[l], nullptr, H, H, H, H}, {}}};
+        if (l) g.seg[1] = Seg{A.u[l - 1], A.theta + tl.D[l], nullptr, H, H, H, H};
         const EpiOut eo{l ? nullptr : A.pk + A.fl.DU0, l >= 2 ? A.h[l - 1] : nullptr, A.bits, A.dy[l], A.u[l], H, A.N, A.W};
         if ((e = launch<false>(g, eo, st))) return e;
     }
@@ -311,7 +311,7 @@ cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t st) {
     const int range = A.sum_out ? grad_f32_range(H) : A.N;
     for (int l = nL - 1; l >= 0; --l) {
         float *gy = A.gy[l & 1];
-        Args gc{M, H, 1, {{gy, A.pk + A.fl.CT[l], nullptr, H, H, H}}};
+        Args gc{M, H, 1, {{gy, A.pk + A.fl.CT[l], nullptr, H, H, H, H}}};
         if ((e = launch<false>(gc, EpiStore{A.gh, H}, st))) return e;
         if (l == 0) grad_scan_bwd0_kernel<<<scan_blocks, 128, 0, st>>>(A);
         else if (l + 1 < nL) grad_scan_bwd_kernel<true><<<scan_blocks, 128, 0, st>>>(A, l);
@@ -336,9 +336,9 @@ cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t st) {
         if (l > 0) {
             // W^T as [input unit][output unit] rows: the packed transposes
             Args gx{M, H, 3,
-                    {{A.gh, A.pk + A.fl.WzT[l], nullptr, H, H, H},
-                     {A.dc, A.pk + A.fl.WhT[l], nullptr, H, H, H},
-                     {gy, A.pk + A.fl.DT[l], nullptr, H, H, H}}};
+                    {{A.gh, A.pk + A.fl.WzT[l], nullptr, H, H, H, H},
+                     {A.dc, A.pk + A.fl.WhT[l], nullptr, H, H, H, H},
+                     {gy, A.pk + A.fl.DT[l], nullptr, H, H, H, H}}};
             if ((e = launch<false>(gx, EpiGy{A.dy[l - 1], A.gy[(l - 1) & 1], H}, st))) return e;
         }
     }

@@ -339,15 +339,15 @@ cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t st) {
     for (int l = 0; l < nL; ++l) {
         const float *u = l ? A.x[l - 1] : nullptr;
         if (l) {
-            const Args g{M, H, 1, {{u, A.theta + tl.Bre[l], A.theta + tl.Bim[l], H, H, H}}};
+            const Args g{M, H, 1, {{u, A.theta + tl.Bre[l], A.theta + tl.Bim[l], H, H, H, H}}};
             if ((e = launch<true>(g, EpiBu{A.br[l], A.bi[l], H}, st))) return e;
         }
         lru_scan_fwd_kernel<<<scan_blocks, 128, 0, st>>>(A, l);
         if ((e = cudaGetLastError())) return e;
         const Args gy{M, H, 2,
-                      {{A.hr[l], A.theta + tl.Cre[l], nullptr, H, H, H}, {A.hn[l], A.theta + tl.Cim[l], nullptr, H, H, H}}};
+                      {{A.hr[l], A.theta + tl.Cre[l], nullptr, H, H, H, H}, {A.hn[l], A.theta + tl.Cim[l], nullptr, H, H, H, H}}};
         if ((e = launch<false>(gy, EpiY{A.pk + A.f.D[l], u, A.bits, A.y[l], H, A.N, A.W}, st))) return e;
-        const Args gg{M, H, 1, {{A.y[l], A.theta + tl.Wa[l], A.theta + tl.Wg[l], H, H, H}}};
+        const Args gg{M, H, 1, {{A.y[l], A.theta + tl.Wa[l], A.theta + tl.Wg[l], H, H, H, H}}};
         if ((e = launch<true>(gg, EpiGlu{A.pk + A.f.ba[l], A.pk + A.f.bg[l], u, A.p1[l], A.p2[l], A.x[l], H}, st))) return e;
     }
     const int top = nL - 1;
@@ -360,9 +360,9 @@ cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t st) {
     for (int l = top; l >= 0; --l) {
         const float *u = l ? A.x[l - 1] : nullptr;
         const Args gy{M, H, 2,
-                      {{A.da, A.pk + A.f.WaT[l], nullptr, H, H, H}, {A.dg, A.pk + A.f.WgT[l], nullptr, H, H, H}}};
+                      {{A.da, A.pk + A.f.WaT[l], nullptr, H, H, H, H}, {A.dg, A.pk + A.f.WgT[l], nullptr, H, H, H, H}}};
         if ((e = launch<false>(gy, EpiStore{A.dy, H}, st))) return e;
-        const Args gh{M, H, 1, {{A.dy, A.pk + A.f.CreT[l], A.pk + A.f.CimT[l], H, H, H}}};
+        const Args gh{M, H, 1, {{A.dy, A.pk + A.f.CreT[l], A.pk + A.f.CimT[l], H, H, H, H}}};
         if ((e = launch<true>(gh, EpiDh{A.dhr, A.dhi, H}, st))) return e;
         if (l) lru_scan_bwd_kernel<false><<<scan_blocks, 128, 0, st>>>(A, l);
         else lru_scan_bwd_kernel<true><<<scan_blocks, 128, 0, st>>>(A, l);
@@ -384,7 +384,7 @@ cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t st) {
         if ((e = launch_wgrad(w, st))) return e;
         if (l) {
             const Args gx{M, H, 2,
-                          {{A.dhr, A.pk + A.f.BreT[l], nullptr, H, H, H}, {A.dhi, A.pk + A.f.BimT[l], nullptr, H, H, H}}};
+                          {{A.dhr, A.pk + A.f.BreT[l], nullptr, H, H, H, H}, {A.dhi, A.pk + A.f.BimT[l], nullptr, H, H, H, H}}};
             const EpiGx ex{A.pk + A.f.D[l], A.dy, A.p1[l - 1], A.p2[l - 1], A.gx, A.da, A.dg, H};
             if ((e = launch<false>(gx, ex, st))) return e;
         }

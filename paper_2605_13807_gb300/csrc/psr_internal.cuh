@@ -459,6 +459,32 @@ size_t grad_lru_floats_per_site(int nL, int H);
 GradLruSmall grad_lru_small(int nL, int H, int64_t *floats);
 cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t stream);
 
+// FP32 gradient of the 2D patched minGRU over a batch of samples, layer by layer
+// (psr_grad2d.cu): sites [patch row][sample][column], M = n Np of them.  Per
+// layer gate a, candidate c, state h, GELU' dy, output x [M][H]; u0 [M][32]
+// one-hot inputs; logits, g [M][32], logp [M]; adjoints gy (two layers), gh, dc;
+// wo32, wo32t [32 H].  theta 16-byte aligned.  rows: [n][P] O_k rows, or
+// partial rows [ceil(M / grad_f32_range)][P] summed into sum_out [P] (added to
+// it if add).  launch_grad2d_fwd writes log psi [n] if asked; dout is read by
+// launch_grad2d_bwd only.
+struct Grad2dArgs {
+    int n, Lx, Ly, W, u1, nL, H;
+    const float *theta;
+    T2Layout tl;
+    const float *pk;
+    F2Layout f;
+    const uint64_t *bits;
+    const float *dout;
+    float *a[kMaxLayers], *c[kMaxLayers], *h[kMaxLayers], *dy[kMaxLayers], *x[kMaxLayers];
+    float *u0, *logits, *g, *logp, *gy[2], *gh, *dc, *wo32, *wo32t;
+    float *rows;
+    float *sum_out;
+    bool add;
+};
+size_t grad2d_floats_per_site(int nL, int H);
+cudaError_t launch_grad2d_fwd(const Grad2dArgs &A, float *logpsi, cudaStream_t stream);
+cudaError_t launch_grad2d_bwd(const Grad2dArgs &A, cudaStream_t stream);
+
 // Backward (FP32) with chunk recompute: the gradient of samples too long for
 // launch_grad_f32's arrays.  Samples of up to kMaxGroups sample sets (one lattice
 // each) in one launch: group g holds samples first[g] .. first[g+1]-1 of the
