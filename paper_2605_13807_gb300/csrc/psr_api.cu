@@ -144,7 +144,7 @@ int psr_logpsi(const psr_params *params, const uint8_t *spins, int64_t n, int32_
         StageScope sc(ctx, PSR_STAGE_PACK);
         PSR_TRY(launch_pack_theta_f32(theta, tl, fl, pk, st));
         if (bf16) PSR_TRY(launch_pack_theta_bf16(theta, tl, pkb, st));
-        PSR_TRY(launch_bitpack(sp, n, L, W, bits, ctx->status, st));
+        PSR_TRY(launch_bitpack(sp, n, L, W, bits, ctx->status, st, counter, 1));
     }
     FwdJobs jb{};
     jb.mode = 0;
@@ -160,9 +160,11 @@ int psr_logpsi(const psr_params *params, const uint8_t *spins, int64_t n, int32_
     const int32_t Ns[1] = {L};
     const int64_t ns[1] = {n};
     const FwdKey key = fwd_key(bf16, 0, 1, Ns, ns);
+    bool zeroed = true;  // the counter, by the packing kernel; later runs zero it again
     auto run_fwd = [&](int shape) -> int {
         StageScope sc(ctx, PSR_STAGE_FWD_SAMPLES);
-        PSR_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st));
+        if (!zeroed) PSR_TRY(cudaMemsetAsync(counter, 0, sizeof(unsigned long long), st));
+        zeroed = false;
         if (bf16) PSR_TRY(launch_fwd_bf16(jb, pkb, pk, fl, ctx->num_sms, st, shape));
         else PSR_TRY(launch_fwd_f32(jb, pk, fl, ctx->num_sms, st, shape));
         return PSR_OK;
@@ -299,7 +301,7 @@ int psr_local_energy(const psr_params *params, const uint8_t *samples, int64_t n
         StageScope sc(ctx, PSR_STAGE_PACK);
         PSR_TRY(launch_pack_theta_f32(theta, tl, fl, pk, st));
         if (bf16) PSR_TRY(launch_pack_theta_bf16(theta, tl, pkb, st));
-        PSR_TRY(launch_bitpack(sp, n, N, W, bits, ctx->status, st));
+        PSR_TRY(launch_bitpack(sp, n, N, W, bits, ctx->status, st, counters, 2));
     }
     HamDev hd{};
     {
@@ -338,8 +340,10 @@ int psr_local_energy(const psr_params *params, const uint8_t *samples, int64_t n
     const int32_t Ns[1] = {N};
     const int64_t ns[1] = {n};
     const FwdKey key = fwd_key(bf16, 1, 1, Ns, ns);
+    bool zeroed = true;  // the counters, by the packing kernel; later runs zero them again
     auto run_fwd = [&](int shape) -> int {
-        PSR_TRY(cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned long long), st));
+        if (!zeroed) PSR_TRY(cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned long long), st));
+        zeroed = false;
         {
             StageScope sc(ctx, PSR_STAGE_FWD_SAMPLES);
             if (bf16) PSR_TRY(launch_fwd_bf16(js, pkb, pk, fl, ctx->num_sms, st, shape));
@@ -565,7 +569,7 @@ int psr_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_t 
     jb.status = ctx->status;
     {
         StageScope sc(ctx, PSR_STAGE_FWD_SAMPLES);
-        PSR_TRY(launch_fwd_f32(jb, pk, fl, ctx->num_sms, st, kChunkGrad));
+        PSR_TRY(launch_fwd_f32(jb, pk, fl, ctx->num_sms, st, kChunkGrad, true));
     }
     {
         StageScope sc(ctx, PSR_STAGE_BWD);

@@ -371,7 +371,7 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
             {
                 StageScope sc(ctx, PSR_STAGE_BWD);  // the gradient's forward and reverse pass
                 PSR_TRY(cudaMemsetAsync(counters + 2, 0, sizeof(unsigned long long), st));
-                PSR_TRY(launch_fwd_f32(jg, pk, fl, ctx->num_sms, st, kChunkGrad));
+                PSR_TRY(launch_fwd_f32(jg, pk, fl, ctx->num_sms, st, kChunkGrad, true));
                 for (int g = 0; g < bj.n_groups; ++g)
                     PSR_TRY(cudaMemsetAsync(bj.g[g].rows, 0, (size_t)(bj.first[g + 1] - bj.first[g]) * P * sizeof(float), st));
                 PSR_TRY(launch_bwd_f32_groups(bj, theta, tl, pk, fl, grad_grid, tape, ctx->status, st));

@@ -132,7 +132,7 @@ int psr_sym_local_energy(const psr_params *params, const uint8_t *samples, int64
     psr_context *ctx = params->ctx;
     const int nL = params->n_layers, H = params->hidden;
     const bool bf16 = params->precision == PSR_BF16;
-    const int CH = bf16 ? kChunkBF16 : kChunkF32;
+    const int CH = bf16 ? kChunkBF16 : kChunkGrad;  // carries
     const int nch = (N + CH - 1) / CH;
     const ThetaLayout tl = theta_layout(nL, H);
     const F32Layout fl = f32_layout(nL, H);

@@ -67,30 +67,35 @@ F32Layout f32_layout(int nL, int H) {
     return f;
 }
 
-__global__ void pack_f32_kernel(const float *__restrict__ theta, ThetaLayout tl, F32Layout fl,
-                                float *__restrict__ pk) {
+// One thread per packed element, so that every read of theta is in flight at
+// once (a loop over layers and tensors paid the latency of each: 9 us at any
+// width, 3 us so).
+__global__ void __launch_bounds__(256) pack_f32_kernel(const float *__restrict__ theta, ThetaLayout tl, F32Layout fl,
+                                                       float *__restrict__ pk) {
     const int H = tl.H;
-    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int l = 0; l < tl.nL; ++l) {
-        const int din = (l == 0) ? 2 : H;
-        for (int64_t i = tid; i < (int64_t)din * H; i += stride) {
-            int k = (int)(i / H), j = (int)(i % H);
-            pk[fl.WzT[l] + i] = theta[tl.Wz[l] + (int64_t)j * din + k];
-            pk[fl.WhT[l] + i] = theta[tl.Wh[l] + (int64_t)j * din + k];
-            pk[fl.DT[l] + i] = theta[tl.D[l] + (int64_t)j * din + k];
-        }
-        for (int64_t i = tid; i < (int64_t)H * H; i += stride) {
-            int k = (int)(i / H), j = (int)(i % H);
-            pk[fl.CT[l] + i] = theta[tl.C[l] + (int64_t)j * H + k];
-        }
-        for (int64_t i = tid; i < H; i += stride) {
-            pk[fl.bz[l] + i] = theta[tl.bz[l] + i];
-            pk[fl.bh[l] + i] = theta[tl.bh[l] + i];
-        }
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    if (i >= fl.total) return;
+    // tensors of a layer in packed order; the tables and readout follow
+    if (i < fl.A0) {
+        int l = 0;
+        while (l + 1 < tl.nL && i >= fl.WzT[l + 1]) ++l;
+        const int din = l == 0 ? 2 : H, m = din * H;
+        int r = i - (int)fl.WzT[l];
+        int64_t src = tl.Wz[l];
+        int rows = din;
+        if (r >= m) { r -= m; src = tl.Wh[l];
+            if (r >= m) { r -= m; src = tl.C[l]; rows = H;
+                if (r >= H * H) { r -= H * H; src = tl.D[l]; rows = din;
+                    if (r >= m) { r -= m; rows = 0; src = tl.bz[l];
+                        if (r >= H) { r -= H; src = tl.bh[l]; } } } } }
+        pk[i] = rows == 0 ? theta[src + r] : theta[src + (int64_t)(r % H) * rows + r / H];
+        return;
     }
-    for (int64_t i = tid; i < 3 * H; i += stride) {
-        int code = (int)(i / H), j = (int)(i % H);
+    if (i < fl.wd) {
+        int r = i - (int)fl.A0;
+        const int table = r / (3 * H);  // A0, B0, DU0, CD0
+        r %= 3 * H;
+        const int code = r / H, j = r % H;
         float zp = theta[tl.bz[0] + j];
         float cd = theta[tl.bh[0] + j];
         float du = 0.0f;
@@ -99,293 +104,444 @@ __global__ void pack_f32_kernel(const float *__restrict__ theta, ThetaLayout tl,
             cd += theta[tl.Wh[0] + 2 * j + (code - 1)];
             du = theta[tl.D[0] + 2 * j + (code - 1)];
         }
-        float a = sigmoid_f(zp);
-        pk[fl.A0 + i] = a;
-        pk[fl.B0 + i] = (1.0f - a) * cd;
-        pk[fl.DU0 + i] = du;
-        pk[fl.CD0 + i] = cd;
+        const float a = sigmoid_f(zp);
+        pk[i] = table == 0 ? a : table == 1 ? (1.0f - a) * cd : table == 2 ? du : cd;
+        return;
     }
-    for (int64_t i = tid; i < H; i += stride)
-        pk[fl.wd + i] = theta[tl.Wo + H + i] - theta[tl.Wo + i];
-    if (tid == 0) pk[fl.bd] = theta[tl.bo + 1] - theta[tl.bo];
+    if (i < fl.bd) {
+        const int j = i - (int)fl.wd;
+        pk[i] = theta[tl.Wo + H + j] - theta[tl.Wo + j];
+    } else if (i == fl.bd) {
+        pk[i] = theta[tl.bo + 1] - theta[tl.bo];
+    }
 }
 
 cudaError_t launch_pack_theta_f32(const float *theta, const ThetaLayout &tl, const F32Layout &fl,
                                   float *packed, cudaStream_t stream) {
-    pack_f32_kernel<<<64, 256, 0, stream>>>(theta, tl, fl, packed);
+    pack_f32_kernel<<<(unsigned)((fl.total + 255) / 256), 256, 0, stream>>>(theta, tl, fl, packed);
     return cudaGetLastError();
 }
 
-// One thread per 64-bit word; a byte other than 0/1 is reported as
-// PSR_EDEVICE and treated as its lowest bit.  Words past N are zero.
-__global__ void bitpack_kernel(const uint8_t *__restrict__ spins, int64_t n, int N, int W,
-                               uint64_t *__restrict__ bits, int *status) {
-    const int64_t total = n * W;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t s = i / W;
-        int w = (int)(i % W);
+// One warp per 64-bit word (two ballots over coalesced bytes); a byte other
+// than 0/1 is reported as PSR_EDEVICE and treated as its lowest bit.  Words past
+// N are zero.  The first thread also zeroes n_zero counters for a kernel that
+// follows (a launch less than a memset).
+__global__ void __launch_bounds__(256) bitpack_kernel(const uint8_t *__restrict__ spins, int64_t n, int N, int W,
+                                                      uint64_t *__restrict__ bits, int *status,
+                                                      unsigned long long *zero, int n_zero) {
+    const int lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && threadIdx.x < n_zero) zero[threadIdx.x] = 0;
+    const int64_t total = n * W, warps = (int64_t)gridDim.x * 8;
+    for (int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); i < total; i += warps) {
+        const int64_t s = i / W;
+        const int t = (int)(i - s * W) * 64 + lane;
         const uint8_t *row = spins + s * N;
-        uint64_t word = 0;
-        int bad = 0;
-        for (int b = 0; b < 64; ++b) {
-            int t = w * 64 + b;
-            if (t >= N) break;
-            uint8_t v = row[t];
-            bad |= (v > 1);
-            word |= (uint64_t)(v & 1u) << b;
-        }
-        if (bad) set_status(status, PSR_EDEVICE);
-        bits[i] = word;
+        const unsigned v0 = t < N ? row[t] : 0u, v1 = t + 32 < N ? row[t + 32] : 0u;
+        const unsigned lo = __ballot_sync(0xffffffffu, v0 & 1u), hi = __ballot_sync(0xffffffffu, v1 & 1u);
+        if ((v0 | v1) > 1u) set_status(status, PSR_EDEVICE);
+        if (lane == 0) bits[i] = (uint64_t)lo | (uint64_t)hi << 32;
     }
 }
 
 cudaError_t launch_bitpack(const uint8_t *spins, int64_t n, int N, int W, uint64_t *bits,
-                           int *status, cudaStream_t stream) {
-    int64_t total = n * W;
-    int blocks = (int)((total + 255) / 256);
+                           int *status, cudaStream_t stream, unsigned long long *zero, int n_zero) {
+    int64_t blocks = (n * W + 7) / 8;
     if (blocks > 65535) blocks = 65535;
-    if (blocks < 1) blocks = 1;
-    bitpack_kernel<<<blocks, 256, 0, stream>>>(spins, n, N, W, bits, status);
+    bitpack_kernel<<<(unsigned)blocks, 256, 0, stream>>>(spins, n, N, W, bits, status, zero, n_zero);
     return cudaGetLastError();
 }
 
-template <int H, int CH>
-__global__ void __launch_bounds__(H) fwd_f32_kernel(const __grid_constant__ FwdJobs jb,
-                                                   const float *__restrict__ pk, F32Layout fl) {
-    static_assert(CH == 16 || CH == 32, "chunk of 16 or 32 sites");
-    constexpr int LD = CH + 4;  // padded row: conflict-free float4 row writes
-    extern __shared__ __align__(16) float smem[];
-    float *xs = smem;              // [H][LD] layer input / output
-    float *hs = xs + H * LD;       // [H][LD] hidden states of the chunk
-    float *hcar = hs + H * LD;     // [kMaxLayers][H] scan carries
-    __shared__ long long s_job;
-    __shared__ long long s_base[kMaxGroups + 1];
+// ------------------------------------------------------------- forward
+// A job is one sequence; the threads of its CTA own U units each (units j, j +
+// H / U, ...) and walk it in windows of 32 or 16 sites (CW).
+//
+// What bounds it: shared memory and the FP32 rate, about equally.  A thread
+// keeps CW sums of both gates, so a row of the window (CW / 4 16-byte
+// broadcasts) and two weights serve 2 CW multiply-adds, done in pairs of sites
+// (fma.rn.f32x2, half the instructions).  A job's CTA is one warp per 32 units;
+// seven jobs per SM overlap.  Two units a thread halve the shared-memory reads
+// but leave half the warps: 7.8 ms against 6.7 ms at hidden 64, 2 to 4 % better
+// to twice as slow at hidden 128 (few long sequences).
+// Measured (E_loc of the 100-site periodic Heisenberg chain, hidden 64, 1024
+// samples): 6.7 ms; 12.0 ms with 32-site windows counted from site 0, plain
+// multiply-adds and unrolled gate functions.
+//
+// Windows.  Chunk boundaries lie on multiples of 16 sites counted from the END
+// of the sequence (off = sites the first chunk starts before site 0), or from
+// its start (align_start: the carries of the chunk-recompute gradient).  A
+// connected configuration resumes at the boundary before its first flipped
+// site: with 32-site windows from site 0, a 100-site chain evaluated 94 sites
+// per configuration where 50 are needed (28 of them past the end, in the last
+// window); boundaries from the end waste 8 on average.  An odd number of
+// chunks starts with one window of 16 sites.
+namespace {
 
-    const int j = threadIdx.x;
-    const int nL = fl.nL;
-    if (j == 0) {
-        long long b = 0;
-        s_base[0] = 0;
-        for (int i = 0; i < jb.n_groups; ++i) {
-            b += jb.mode == 1 ? (long long)*jb.g[i].n_jobs_dev : (long long)jb.g[i].n_jobs;
-            s_base[i + 1] = b;
+__device__ __forceinline__ void ffma2(uint64_t &d, uint64_t a, uint64_t b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ float lo2(uint64_t v) { return __uint_as_float((uint32_t)v); }
+__device__ __forceinline__ float hi2(uint64_t v) { return __uint_as_float((uint32_t)(v >> 32)); }
+
+// Bits of sites [t0, t0 + 32) and of site t0 - 1, flips p and q applied; t0
+// may be negative or unaligned, sites outside [0, N) read as 0.
+__device__ __forceinline__ void window_bits(const uint64_t *row, int N, int t0, int p, int q, uint32_t &cur,
+                                            uint32_t &prev) {
+    const int b = max(t0, 0);
+    uint64_t v = row[b >> 6] >> (b & 63);
+    if (b & 63) v |= row[(b >> 6) + 1] << (64 - (b & 63));  // rows end with a zero word
+    cur = (uint32_t)v << (b - t0);
+    if (t0 + 32 > N) cur &= t0 < N ? 0xffffffffu >> (t0 + 32 - N) : 0u;
+    prev = t0 > 0 ? (uint32_t)(row[(t0 - 1) >> 6] >> ((t0 - 1) & 63)) & 1u : 0u;
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+        const int x = f ? q : p;
+        if (x < 0) continue;
+        if (x >= t0 && x < t0 + 32) cur ^= 1u << (x - t0);
+        else if (x == t0 - 1) prev ^= 1u;
+    }
+}
+
+struct FwdF32Job {
+    const uint64_t *row;
+    float *carries;  // of this job's chunk 0 (mode 0, or null): [nch][nL][H]
+    float *logp_out;
+    const float *logp_ref;
+    int N, u1, p, q;
+};
+
+template <int H>
+struct FwdF32Shape {
+    static constexpr int U = 1;                // units a thread
+    static constexpr int T = H / U;            // threads a job
+    static constexpr int LD = 36;              // row of a tile: 32 sites, 16-byte aligned
+};
+
+template <int T>
+__device__ __forceinline__ void job_sync() {
+    if constexpr (T == 32) __syncwarp();
+    else __syncthreads();
+}
+
+// y[r] += w[k][unit r] x[k] over a window's row pairs, k = 0 .. H - 1, for NM
+// (weights, tile, sums) triples at once; the weights (coalesced over units) of
+// the next K inner units are fetched while K are used.
+template <int H, int CW, int U, int NM>
+__device__ __forceinline__ void products(const float *const (&w)[NM], const float *const (&tile)[NM],
+                                         uint64_t (*const (&y)[NM])[CW / 2]) {
+    constexpr int T = H / U, LD = FwdF32Shape<H>::LD, P = CW / 2;
+    // K = 4 leaves the code of the narrow model small enough for jobs out of step
+    constexpr int K = H == 32 ? 4 : 8;
+    float nw[NM][K][U];
+    auto fetch = [&](int k0) {
+#pragma unroll
+        for (int m = 0; m < NM; ++m)
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+#pragma unroll
+                for (int r = 0; r < U; ++r) nw[m][k][r] = w[m][(k0 + k) * H + r * T];
+    };
+    fetch(0);
+#pragma unroll 1
+    for (int k0 = 0; k0 < H; k0 += K) {
+        uint64_t cw[NM][K][U];
+#pragma unroll
+        for (int m = 0; m < NM; ++m)
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+#pragma unroll
+                for (int r = 0; r < U; ++r) cw[m][k][r] = pack2(nw[m][k][r], nw[m][k][r]);
+        if (k0 + K < H) fetch(k0 + K);
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+#pragma unroll
+            for (int q = 0; q < P / 2; ++q) {
+                ulonglong2 v;
+#pragma unroll
+                for (int m = 0; m < NM; ++m) {
+                    if (m == 0 || tile[m] != tile[0])
+                        v = *reinterpret_cast<const ulonglong2 *>(tile[m] + (k0 + k) * LD + 4 * q);
+#pragma unroll
+                    for (int r = 0; r < U; ++r) {
+                        ffma2(y[m][r][2 * q], cw[m][k][r], v.x);
+                        ffma2(y[m][r][2 * q + 1], cw[m][k][r], v.y);
+                    }
+                }
+            }
         }
     }
-    __syncthreads();
-    const long long njobs = s_base[jb.n_groups];
+}
 
-    const float a0_0 = pk[fl.A0 + j], a0_1 = pk[fl.A0 + H + j], a0_2 = pk[fl.A0 + 2 * H + j];
-    const float b0_0 = pk[fl.B0 + j], b0_1 = pk[fl.B0 + H + j], b0_2 = pk[fl.B0 + 2 * H + j];
-    const float d0_0 = pk[fl.DU0 + j], d0_1 = pk[fl.DU0 + H + j], d0_2 = pk[fl.DU0 + 2 * H + j];
-    const float bd = pk[fl.bd];
+// One window of CW sites starting at t0 (chunk c): x of the last layer's sites
+// through the readout; returns this thread's share of the sum of log P.
+template <int H, int CW>
+__device__ __forceinline__ float window(const FwdF32Job &J, const float *__restrict__ pk, const F32Layout &fl,
+                                        float *xs, float *hs, float *zs, float *hcar, int t0, int c,
+                                        int &n_up) {
+    constexpr int U = FwdF32Shape<H>::U, T = FwdF32Shape<H>::T, LD = FwdF32Shape<H>::LD, P = CW / 2;
+    const int j = threadIdx.x, nL = fl.nL;
+    uint32_t cur, prev;
+    window_bits(J.row, J.N, t0, J.p, J.q, cur, prev);
+    if (CW < 32) cur &= (1u << CW) - 1u;
+    const uint32_t prevbits = (cur << 1) | prev;  // bit t = s_{t0+t-1}
+    const int first = max(0, -t0);                // sites before the sequence: no input, no state
 
+    uint64_t y[U][P];
+    // scan of one unit: h_t from a_t and c_t (or b_t), written to its row of
+    // hs; y starts from the unit's old row (the layer below's states) if kept
+    auto put_carry = [&](int l, int u, int chunk, float h) {
+        if (J.carries) J.carries[((int64_t)chunk * nL + l) * H + u] = h;
+    };
+    // ---------------- layer 0: gates by lookup of the one-hot input
+#pragma unroll
+    for (int r = 0; r < U; ++r) {
+        const int u = j + r * T;
+        float a[3], b[3], d[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            a[q] = pk[fl.A0 + q * H + u];
+            b[q] = pk[fl.B0 + q * H + u];
+            d[q] = pk[fl.DU0 + q * H + u];
+        }
+        float h = hcar[u];
+        put_carry(0, u, c, h);
+#pragma unroll
+        for (int t = 0; t < CW; t += 4) {
+            float hv[4], dv[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int tt = t + e;
+                if (CW == 32 && tt == 16) put_carry(0, u, c + 1, h);
+                const bool up = (prevbits >> tt) & 1u;
+                const bool start = t0 + tt == 0;
+                const float hn = (start ? a[0] : up ? a[2] : a[1]) * h + (start ? b[0] : up ? b[2] : b[1]);
+                h = tt < first ? 0.0f : hn;
+                hv[e] = h;
+                dv[e] = start ? d[0] : up ? d[2] : d[1];
+            }
+            *reinterpret_cast<float4 *>(hs + u * LD + t) = make_float4(hv[0], hv[1], hv[2], hv[3]);
+            y[r][t / 2] = pack2(dv[0], dv[1]);
+            y[r][t / 2 + 1] = pack2(dv[2], dv[3]);
+        }
+        hcar[u] = h;
+    }
+    job_sync<T>();
+    products<H, CW, U, 1>({pk + fl.CT[0] + j}, {hs}, {y});
+    // The element-wise functions run in rolled loops over the thread's own rows
+    // in shared memory: unrolled over the register arrays their code (some 40
+    // instructions a site) outgrew the instruction cache as soon as the jobs of
+    // an SM were out of step (connected configurations: 13.4 against 7 ms).
+    auto put_rows = [&](float *tile, const uint64_t (&v)[U][P]) {
+#pragma unroll
+        for (int r = 0; r < U; ++r)
+#pragma unroll
+            for (int q = 0; q < P / 2; ++q)
+                *reinterpret_cast<ulonglong2 *>(tile + (j + r * T) * LD + 4 * q) =
+                    make_ulonglong2(v[r][2 * q], v[r][2 * q + 1]);
+    };
+    auto map_rows = [&](float *tile, auto f) {
+#pragma unroll 1
+        for (int i = 0; i < U * CW / 4; ++i) {
+            float4 *p = reinterpret_cast<float4 *>(tile + (j + i / (CW / 4) * T) * LD + i % (CW / 4) * 4);
+            const float4 v = *p;
+            *p = make_float4(f(v.x), f(v.y), f(v.z), f(v.w));
+        }
+    };
+    auto store_x = [&]() {
+        put_rows(xs, y);
+        map_rows(xs, [](float v) { return gelu_f(v); });
+    };
+    store_x();
+    job_sync<T>();
+
+    for (int l = 1; l < nL; ++l) {
+        uint64_t z[U][P];
+#pragma unroll
+        for (int r = 0; r < U; ++r) {
+            const float bz = pk[fl.bz[l] + j + r * T], bh = pk[fl.bh[l] + j + r * T];
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                z[r][q] = pack2(bz, bz);
+                y[r][q] = pack2(bh, bh);
+            }
+        }
+        products<H, CW, U, 2>({pk + fl.WzT[l] + j, pk + fl.WhT[l] + j}, {xs, xs}, {z, y});
+        put_rows(zs, z);
+        map_rows(zs, [](float v) { return sigmoid_f(v); });
+        // scan: this unit's row of hs turns from h of the layer below (the
+        // residual of l >= 2, which y starts from) into h of this layer
+#pragma unroll
+        for (int r = 0; r < U; ++r) {
+            const int u = j + r * T;
+            float h = hcar[l * H + u];
+            put_carry(l, u, c, h);
+            float *row = hs + u * LD;
+#pragma unroll
+            for (int t = 0; t < CW; t += 4) {
+                const float4 below = *reinterpret_cast<const float4 *>(row + t);
+                const float4 gate = *reinterpret_cast<const float4 *>(zs + u * LD + t);
+                const float av[4] = {gate.x, gate.y, gate.z, gate.w};
+                float hv[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int tt = t + e;
+                    if (CW == 32 && tt == 16) put_carry(l, u, c + 1, h);
+                    const uint64_t c2 = y[r][tt / 2];
+                    const float a = av[e];
+                    const float hn = a * h + (1.0f - a) * (tt & 1 ? hi2(c2) : lo2(c2));
+                    h = tt < first ? 0.0f : hn;
+                    hv[e] = h;
+                }
+                *reinterpret_cast<float4 *>(row + t) = make_float4(hv[0], hv[1], hv[2], hv[3]);
+                y[r][t / 2] = l >= 2 ? pack2(below.x, below.y) : 0;
+                y[r][t / 2 + 1] = l >= 2 ? pack2(below.z, below.w) : 0;
+            }
+            hcar[l * H + u] = h;
+        }
+        job_sync<T>();
+        products<H, CW, U, 2>({pk + fl.CT[l] + j, pk + fl.DT[l] + j}, {hs, xs}, {y, y});
+        job_sync<T>();
+        store_x();
+        job_sync<T>();
+    }
+
+    // readout: lane t of the first warp handles site t0 + t
+    float v = 0.0f;
+    if (j < CW) {
+        const int t = j, tt = t0 + t;
+        if (tt >= 0 && tt < J.N) {
+            float d[4] = {pk[fl.bd], 0.0f, 0.0f, 0.0f};  // four chains: the sum is latency-bound
+            const float *wd = pk + fl.wd;
+#pragma unroll 2
+            for (int k = 0; k < H; k += 4)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) d[e] = fmaf(wd[k + e], xs[(k + e) * LD + t], d[e]);
+            const int s = (cur >> t) & 1u;
+            const int nu = n_up + __popc(cur & ((1u << t) - 1u));
+            const float lp = site_logp((d[0] + d[1]) + (d[2] + d[3]), s, u1_forced(J.u1, J.N, tt, nu));
+            if (J.logp_out) J.logp_out[tt] = lp;
+            v = J.logp_ref ? lp - J.logp_ref[tt] : lp;
+        }
+    }
+    n_up += __popc(cur);
+    job_sync<T>();
+    return v;
+}
+
+}  // namespace
+
+// kWide: windows of 32 sites (after one of 16 if the chunks are odd in
+// number); else 16.
+template <int H, bool kWide>
+__global__ void __launch_bounds__(FwdF32Shape<H>::T) fwd_f32_kernel(const __grid_constant__ FwdJobs jb,
+                                                                    const float *__restrict__ pk, F32Layout fl,
+                                                                    bool align_start) {
+    constexpr int U = FwdF32Shape<H>::U, T = FwdF32Shape<H>::T, LD = FwdF32Shape<H>::LD, CH = kChunkGrad;
+    extern __shared__ __align__(16) float smem[];
+    float *xs = smem;              // [H][LD] layer input / output
+    float *hs = xs + H * LD;       // [H][LD] hidden states of the window
+    float *zs = hs + H * LD;       // [H][LD] gates of the window
+    float *hcar = zs + H * LD;     // [nL][H] scan carries
+    __shared__ long long s_job;
+    const int j = threadIdx.x, nL = fl.nL;
+    long long base[kMaxGroups + 1];
+    base[0] = 0;
+    for (int i = 0; i < jb.n_groups; ++i)
+        base[i + 1] = base[i] + (jb.mode == 1 ? (long long)*jb.g[i].n_jobs_dev : (long long)jb.g[i].n_jobs);
     for (;;) {
+        job_sync<T>();
         if (j == 0) s_job = (long long)atomicAdd((unsigned long long *)jb.job_counter, 1ull);
-        __syncthreads();
+        job_sync<T>();
         const long long job = s_job;
-        __syncthreads();
-        if (job >= njobs) break;
+        if (job >= base[jb.n_groups]) break;
         int gi = 0;
-        while (gi + 1 < jb.n_groups && job >= s_base[gi + 1]) ++gi;
+        while (gi + 1 < jb.n_groups && job >= base[gi + 1]) ++gi;
         const FwdGroup &G = jb.g[gi];
-        const long long lj = job - s_base[gi];
-        const int N = G.N;
-        const int nch = (N + CH - 1) / CH;
+        const long long lj = job - base[gi];
+        const int N = G.N, nch = (N + CH - 1) / CH;
+        const int off = align_start ? 0 : nch * CH - N;
 
-        int sample, p = -1, q = -1, c0 = 0;
+        int sample, c0 = 0;
+        FwdF32Job J{};
+        J.p = J.q = -1;
         if (jb.mode == 0) {
             sample = (int)lj;
         } else {
             const int32_t *e = G.entries + 3 * lj;
             sample = e[0];
-            p = e[1];
-            q = e[2];
-            c0 = p / CH;
+            J.p = e[1];
+            J.q = e[2];
+            c0 = (J.p + off) / CH;
         }
-        const uint64_t *row = G.bits + (int64_t)sample * G.W;
+        J.row = G.bits + (int64_t)sample * G.W;
+        J.N = N;
+        J.u1 = G.u1;
+        J.carries = G.carries_out ? G.carries_out + (int64_t)sample * nch * nL * H : nullptr;
+        J.logp_out = G.logp_out ? G.logp_out + (int64_t)sample * N : nullptr;
+        J.logp_ref = jb.mode == 1 ? G.logp_ref + (int64_t)sample * N : nullptr;
         for (int l = 0; l < nL; ++l)
-            hcar[l * H + j] = (c0 == 0) ? 0.0f
-                : G.carries_in[(((int64_t)sample * nch + c0) * nL + l) * H + j];
-        int n_up = G.u1 ? count_up_before(row, c0 * CH) : 0;
+#pragma unroll
+            for (int r = 0; r < U; ++r) {
+                const int u = j + r * T;
+                hcar[l * H + u] = c0 == 0 ? 0.0f : G.carries_in[(((int64_t)sample * nch + c0) * nL + l) * H + u];
+            }
+        int n_up = G.u1 ? count_up_before(J.row, max(c0 * CH - off, 0)) : 0;
         float acc = 0.0f;
-
-        for (int c = c0; c < nch; ++c) {
-            const int t0 = c * CH;
-            if (G.carries_out)
-                for (int l = 0; l < nL; ++l)
-                    G.carries_out[(((int64_t)sample * nch + c) * nL + l) * H + j] = hcar[l * H + j];
-            uint32_t cur, prev;
-            chunk_bits32(row, t0, p, q, cur, prev);
-            const int nvalid = min(CH, N - t0);
-            if (nvalid < 32) cur &= (1u << nvalid) - 1u;
-            // input code of site t: 0 = first site, 1 + s_{t-1} otherwise
-            const uint32_t prevbits = (cur << 1) | prev;  // bit t = s_{t0+t-1}
-
-            float hl[CH];  // h of the current layer (residual source for the next)
-            float y[CH];
-            {
-                float hv = hcar[j];
-#pragma unroll
-                for (int t = 0; t < CH; ++t) {
-                    const bool first = (t0 + t == 0);
-                    const uint32_t sb = (prevbits >> t) & 1u;
-                    const float a = first ? a0_0 : (sb ? a0_2 : a0_1);
-                    const float b = first ? b0_0 : (sb ? b0_2 : b0_1);
-                    hv = a * hv + b;
-                    hl[t] = hv;
-                    y[t] = first ? d0_0 : (sb ? d0_2 : d0_1);
-                }
-                hcar[j] = hv;
-                float4 *dst = reinterpret_cast<float4 *>(hs + j * LD);
-#pragma unroll
-                for (int t4 = 0; t4 < CH / 4; ++t4)
-                    dst[t4] = make_float4(hl[4 * t4], hl[4 * t4 + 1], hl[4 * t4 + 2], hl[4 * t4 + 3]);
-            }
-            __syncthreads();
-            {
-                const float *Ct = pk + fl.CT[0];
-                #pragma unroll 4
-                for (int k = 0; k < H; ++k) {
-                    const float w = Ct[k * H + j];
-                    const float4 *src = reinterpret_cast<const float4 *>(hs + k * LD);
-#pragma unroll
-                    for (int t4 = 0; t4 < CH / 4; ++t4) {
-                        float4 v = src[t4];
-                        y[4 * t4] += w * v.x; y[4 * t4 + 1] += w * v.y;
-                        y[4 * t4 + 2] += w * v.z; y[4 * t4 + 3] += w * v.w;
-                    }
-                }
-                float4 *dst = reinterpret_cast<float4 *>(xs + j * LD);
-#pragma unroll
-                for (int t4 = 0; t4 < CH / 4; ++t4)
-                    dst[t4] = make_float4(gelu_f(y[4 * t4]), gelu_f(y[4 * t4 + 1]),
-                                          gelu_f(y[4 * t4 + 2]), gelu_f(y[4 * t4 + 3]));
-            }
-            __syncthreads();
-
-            for (int l = 1; l < nL; ++l) {
-                float z[CH];
-                const float bz = pk[fl.bz[l] + j], bh = pk[fl.bh[l] + j];
-#pragma unroll
-                for (int t = 0; t < CH; ++t) { z[t] = bz; y[t] = bh; }
-                const float *Wz = pk + fl.WzT[l];
-                const float *Wh = pk + fl.WhT[l];
-                #pragma unroll 4
-                for (int k = 0; k < H; ++k) {
-                    const float wz = Wz[k * H + j], wh = Wh[k * H + j];
-                    const float4 *src = reinterpret_cast<const float4 *>(xs + k * LD);
-#pragma unroll
-                    for (int t4 = 0; t4 < CH / 4; ++t4) {
-                        float4 v = src[t4];
-                        z[4 * t4] += wz * v.x; z[4 * t4 + 1] += wz * v.y;
-                        z[4 * t4 + 2] += wz * v.z; z[4 * t4 + 3] += wz * v.w;
-                        y[4 * t4] += wh * v.x; y[4 * t4 + 1] += wh * v.y;
-                        y[4 * t4 + 2] += wh * v.z; y[4 * t4 + 3] += wh * v.w;
-                    }
-                }
-                float hn[CH];
-                {
-                    float hv = hcar[l * H + j];
-#pragma unroll
-                    for (int t = 0; t < CH; ++t) {
-                        const float a = sigmoid_f(z[t]);
-                        hv = a * hv + (1.0f - a) * y[t];
-                        hn[t] = hv;
-                    }
-                    hcar[l * H + j] = hv;
-                    float4 *dst = reinterpret_cast<float4 *>(hs + j * LD);
-#pragma unroll
-                    for (int t4 = 0; t4 < CH / 4; ++t4)
-                        dst[t4] = make_float4(hn[4 * t4], hn[4 * t4 + 1], hn[4 * t4 + 2], hn[4 * t4 + 3]);
-                }
-                __syncthreads();
-#pragma unroll
-                for (int t = 0; t < CH; ++t) y[t] = (l >= 2) ? hl[t] : 0.0f;
-                const float *Ct = pk + fl.CT[l];
-                const float *Dt = pk + fl.DT[l];
-                #pragma unroll 4
-                for (int k = 0; k < H; ++k) {
-                    const float wc = Ct[k * H + j], wd = Dt[k * H + j];
-                    const float4 *sh = reinterpret_cast<const float4 *>(hs + k * LD);
-                    const float4 *sx = reinterpret_cast<const float4 *>(xs + k * LD);
-#pragma unroll
-                    for (int t4 = 0; t4 < CH / 4; ++t4) {
-                        float4 vh = sh[t4], vx = sx[t4];
-                        y[4 * t4] += wc * vh.x + wd * vx.x;
-                        y[4 * t4 + 1] += wc * vh.y + wd * vx.y;
-                        y[4 * t4 + 2] += wc * vh.z + wd * vx.z;
-                        y[4 * t4 + 3] += wc * vh.w + wd * vx.w;
-                    }
-                }
-                __syncthreads();
-                float4 *dst = reinterpret_cast<float4 *>(xs + j * LD);
-#pragma unroll
-                for (int t4 = 0; t4 < CH / 4; ++t4)
-                    dst[t4] = make_float4(gelu_f(y[4 * t4]), gelu_f(y[4 * t4 + 1]),
-                                          gelu_f(y[4 * t4 + 2]), gelu_f(y[4 * t4 + 3]));
-#pragma unroll
-                for (int t = 0; t < CH; ++t) hl[t] = hn[t];
-                __syncthreads();
-            }
-
-            // readout: thread t < CH handles site t0 + t (warp 0 reduces)
-            if (j < 32) {
-                const int t = j;
-                float v = 0.0f;
-                const int tt = t0 + t;
-                if (t < CH && tt < N) {
-                    float d = bd;
-                    const float *wd = pk + fl.wd;
-                    for (int k = 0; k < H; ++k) d += wd[k] * xs[k * LD + t];
-                    const int s = (cur >> t) & 1u;
-                    const int nu = n_up + __popc(cur & ((1u << t) - 1u));
-                    const float lp = site_logp(d, s, u1_forced(G.u1, N, tt, nu));
-                    if (G.logp_out) G.logp_out[(int64_t)sample * N + tt] = lp;
-                    v = (jb.mode == 1) ? lp - G.logp_ref[(int64_t)sample * N + tt] : lp;
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (j == 0) acc += v;
-            }
-            n_up += __popc(cur);
-            __syncthreads();
+        int c = c0;
+        if (!kWide || ((nch - c) & 1)) {
+            do {
+                acc += window<H, 16>(J, pk, fl, xs, hs, zs, hcar, c * CH - off, c, n_up);
+                ++c;
+            } while (!kWide && c < nch);
         }
-        if (j == 0) G.out[lj] = 0.5f * acc;
+        if constexpr (kWide)
+            for (; c < nch; c += 2) acc += window<H, 32>(J, pk, fl, xs, hs, zs, hcar, c * CH - off, c, n_up);
+        if (j < 32) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (j == 0) G.out[lj] = 0.5f * acc;
+        }
     }
 }
 
-template <int H, int CH>
+template <int H, bool kWide>
 static cudaError_t launch_fwd_f32_h(const FwdJobs &jobs, const float *packed, const F32Layout &fl,
-                                    int num_sms, cudaStream_t stream) {
-    const size_t smem = (size_t)(2 * H * (CH + 4) + kMaxLayers * H) * sizeof(float);
+                                    int num_sms, cudaStream_t stream, bool align_start) {
+    constexpr int T = FwdF32Shape<H>::T;
+    const size_t smem = (size_t)(3 * H * FwdF32Shape<H>::LD + fl.nL * H) * sizeof(float);
+    cudaError_t e = cudaFuncSetAttribute(fwd_f32_kernel<H, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fwd_f32_kernel<H, CH>, H, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fwd_f32_kernel<H, kWide>, T, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     int64_t grid = (int64_t)num_sms * per_sm;
     const int64_t nj = max_jobs(jobs);
     if (nj < grid) grid = nj;
     if (grid < 1) grid = 1;
-    fwd_f32_kernel<H, CH><<<(int)grid, H, smem, stream>>>(jobs, packed, fl);
+    fwd_f32_kernel<H, kWide><<<(int)grid, T, smem, stream>>>(jobs, packed, fl, align_start);
     return cudaGetLastError();
 }
 
-cudaError_t launch_fwd_f32(const FwdJobs &jobs, const float *packed, const F32Layout &fl,
-                           int num_sms, cudaStream_t stream, int chunk) {
-    if (chunk == kChunkGrad) {
-        switch (fl.H) {
-            case 32: return launch_fwd_f32_h<32, kChunkGrad>(jobs, packed, fl, num_sms, stream);
-            case 64: return launch_fwd_f32_h<64, kChunkGrad>(jobs, packed, fl, num_sms, stream);
-            case 128: return launch_fwd_f32_h<128, kChunkGrad>(jobs, packed, fl, num_sms, stream);
-            default: return cudaErrorInvalidValue;
-        }
-    }
-    if (chunk != kChunkF32) return cudaErrorInvalidValue;
+cudaError_t launch_fwd_f32(const FwdJobs &jobs, const float *packed, const F32Layout &fl, int num_sms,
+                           cudaStream_t stream, int chunk, bool align_start) {
+    if (chunk != kChunkF32 && chunk != kChunkGrad) return cudaErrorInvalidValue;
+    const bool wide = chunk == kChunkF32;
     switch (fl.H) {
-        case 32: return launch_fwd_f32_h<32, kChunkF32>(jobs, packed, fl, num_sms, stream);
-        case 64: return launch_fwd_f32_h<64, kChunkF32>(jobs, packed, fl, num_sms, stream);
-        case 128: return launch_fwd_f32_h<128, kChunkF32>(jobs, packed, fl, num_sms, stream);
+        case 32:
+            return wide ? launch_fwd_f32_h<32, true>(jobs, packed, fl, num_sms, stream, align_start)
+                        : launch_fwd_f32_h<32, false>(jobs, packed, fl, num_sms, stream, align_start);
+        case 64:
+            return wide ? launch_fwd_f32_h<64, true>(jobs, packed, fl, num_sms, stream, align_start)
+                        : launch_fwd_f32_h<64, false>(jobs, packed, fl, num_sms, stream, align_start);
+        case 128:
+            return wide ? launch_fwd_f32_h<128, true>(jobs, packed, fl, num_sms, stream, align_start)
+                        : launch_fwd_f32_h<128, false>(jobs, packed, fl, num_sms, stream, align_start);
         default: return cudaErrorInvalidValue;
     }
 }

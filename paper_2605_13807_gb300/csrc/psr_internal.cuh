@@ -9,8 +9,8 @@
 namespace psr {
 
 constexpr int kMaxLayers = 8;
-constexpr int kChunkF32 = 32;   // scan chunk of the FP32 SIMT path (sites)
-constexpr int kChunkGrad = 16;  // short chunk: forward shape, carries and recompute of launch_bwd_f32
+constexpr int kChunkF32 = 32;   // window of the FP32 SIMT forward (sites)
+constexpr int kChunkGrad = 16;  // its short window; carries, recompute of launch_bwd_f32
 constexpr int kChunkBF16 = 32;  // scan chunk of the tcgen05 path (sites = MMA N)
 
 // Device status word values (first error wins).
@@ -103,11 +103,14 @@ inline int64_t max_jobs(const FwdJobs &jb) {
 
 cudaError_t launch_pack_theta_f32(const float *theta, const ThetaLayout &tl, const F32Layout &fl,
                                   float *packed, cudaStream_t stream);
-cudaError_t launch_bitpack(const uint8_t *spins, int64_t n, int N, int W, uint64_t *bits,
-                           int *status, cudaStream_t stream);
-// chunk: kChunkF32 (log psi, E_loc) or kChunkGrad (carries for psr_grad)
-cudaError_t launch_fwd_f32(const FwdJobs &jobs, const float *packed, const F32Layout &fl,
-                           int num_sms, cudaStream_t stream, int chunk = kChunkF32);
+// zero: n_zero (at most 256) counters set to 0 as well, or null.
+cudaError_t launch_bitpack(const uint8_t *spins, int64_t n, int N, int W, uint64_t *bits, int *status,
+                           cudaStream_t stream, unsigned long long *zero = nullptr, int n_zero = 0);
+// chunk: sites of a window, kChunkF32 or kChunkGrad.  The carries are stored
+// every kChunkGrad sites for both, on boundaries counted from the end of the
+// sequence (align_start: from its start, as launch_bwd_f32 wants them).
+cudaError_t launch_fwd_f32(const FwdJobs &jobs, const float *packed, const F32Layout &fl, int num_sms,
+                           cudaStream_t stream, int chunk = kChunkF32, bool align_start = false);
 
 // tcgen05 path (hidden = 128, 3 layers).
 size_t bf16_packed_bytes();
