@@ -64,7 +64,6 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         int64_t cap;
         int64_t B;                             // samples per batch of the FP32 layer gradient (0: chunk recompute)
     } w[kMaxGroups];
-    int64_t n_grad = 0;
     for (int i = 0; i < n_items; ++i) {
         const StepItem &it = items[i];
         ItemWs &x = w[i];
@@ -78,23 +77,8 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         x.W = (int)words_per_row(x.N);
         x.nb = bond_count(it.ham.Lx, it.ham.Ly, it.ham.pbc);
         x.cap = it.eloc ? it.n * max_entries_per_sample(&it.ham) : 0;
-        if (it.grad) n_grad += it.n;
     }
-    // BF16 gradients run on the tensor cores one item after another (as
-    // psr_grad does), through one set of batch buffers sized for the largest
-    const bool use_tc = bf16 && H == 128;
-    size_t tc_stash = 0, tc_arr = 0;
-    if (use_tc) {
-        for (int i = 0; i < n_items; ++i) {
-            if (!items[i].grad) continue;
-            const int64_t B = grad_tc_batch(nL, w[i].N, items[i].n);
-            const size_t st_i = (size_t)B * stash_floats_per_sample(nL, 128, w[i].N);
-            const size_t ar_i = (size_t)B * 128 * stash_npad(w[i].N);
-            tc_stash = st_i > tc_stash ? st_i : tc_stash;
-            tc_arr = ar_i > tc_arr ? ar_i : tc_arr;
-        }
-    }
-    // FP32 gradients: layer by layer, one item after another through one set
+    // gradients: layer by layer, one item after another through one set
     // of arrays, as psr_grad does; samples too long for that share one launch
     // of the chunk-recompute kernel (CTAs per SM by shared memory).
     const bool copy_theta = d_theta && !aligned16p(params->theta);
@@ -106,7 +90,7 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         layer_bytes = 0;
         for (int i = 0; i < n_items; ++i) {
             w[i].B = 0;
-            if (!items[i].grad || use_tc) continue;
+            if (!items[i].grad) continue;
             if (layers) w[i].B = grad_f32_batch(nL, H, w[i].N, items[i].n);
             if (w[i].B == 0) {
                 n_chunk += items[i].n;
@@ -128,7 +112,6 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
     };
     plan_grad(true, 0);
     char *layer_ws = nullptr;
-    GradTcWs tw{};
     float *theta_ws = nullptr, *pk = nullptr, *tape = nullptr;
     void *pkb = nullptr;
     unsigned long long *counters = nullptr;
@@ -139,17 +122,6 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         counters = c.get<unsigned long long>(3);
         tape = c.get<float>((size_t)grad_grid * bwd_tape_floats_per_cta(nL, H));
         layer_ws = c.get<char>(layer_bytes);
-        if (use_tc && n_grad > 0) {
-            tw.images = c.get<char>(bwd_tc_image_bytes(nL));
-            tw.stash = c.get<float>(tc_stash);
-            for (int k = 0; k < 2; ++k) {
-                tw.gx[k] = c.get<float>(tc_arr);
-                tw.gy[k] = c.get<float>(tc_arr);
-            }
-            tw.gh = c.get<float>(tc_arr);
-            tw.dz = c.get<float>(tc_arr);
-            tw.dc = c.get<float>(tc_arr);
-        }
         for (int i = 0; i < n_items; ++i) {
             const StepItem &it = items[i];
             const int64_t n = it.n;
@@ -172,7 +144,7 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
             x.logp = c.get<float>(it.eloc ? (size_t)n * x.N : 0);
             x.carries = c.get<float>(it.eloc ? (size_t)n * nch * nL * H : 0);
             x.delta = c.get<float>(x.cap);
-            const bool chunked = it.grad && !use_tc && x.B == 0;
+            const bool chunked = it.grad && x.B == 0;
             x.carries_g = c.get<float>(chunked ? (size_t)n * nchg * nL * H : 0);
             x.lpsi_g = c.get<float>(chunked ? n : 0);
         }
@@ -223,7 +195,6 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         // kernel attributes are set outside the capture
         if (bf16) PSR_TRY(prepare_fwd_bf16());
         if (by_chunk) PSR_TRY(prepare_bwd_f32(H, nL));
-        if (n_grad > 0 && use_tc) PSR_TRY(prepare_bwd_tc());
         PSR_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
         ctx->capturing = true;
     }
@@ -315,20 +286,7 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
                 if (so) PSR_TRY(launch_stats(o, it.n, so, st));
             }
         }
-        // ---- gradient on the tensor cores (BF16), one item after another
-        if (n_grad > 0 && use_tc) {
-            StageScope sc(ctx, PSR_STAGE_BWD);
-            for (int i = 0; i < n_items; ++i) {
-                const StepItem &it = items[i];
-                if (!it.grad) continue;
-                tw.B = grad_tc_batch(nL, w[i].N, it.n);
-                float *rows = w[i].d_g ? it.grad : w[i].g_ws;
-                if ((r = enqueue_grad_tc(ctx, nL, it.u1, theta, pk, w[i].bits, it.n, w[i].N, w[i].W, rows, tw)) !=
-                    PSR_OK)
-                    return r;
-            }
-        }
-        // ---- gradient in FP32, layer by layer
+        // ---- gradients, layer by layer
         if (layer_bytes > 0) {
             StageScope sc(ctx, PSR_STAGE_BWD);
             for (int i = 0; i < n_items; ++i) {
@@ -340,7 +298,7 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
                 grad_f32_carve(sub, nL, H, w[i].N, w[i].B, false, copy_theta, A);
                 float *rows = w[i].d_g ? it.grad : w[i].g_ws;
                 if ((r = enqueue_grad_f32(ctx, nL, H, it.u1, theta, pk, w[i].bits, it.n, w[i].N, w[i].W, nullptr,
-                                          rows, w[i].B, A)) != PSR_OK)
+                                          rows, w[i].B, A, grad_bf16_rows(params, nullptr))) != PSR_OK)
                     return r;
             }
         }

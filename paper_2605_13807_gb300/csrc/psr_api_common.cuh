@@ -314,92 +314,8 @@ inline int tune_fwd_shape(psr_context *ctx, bool bf16, const FwdKey &k, Run run,
     return PSR_OK;
 }
 
-// ------------------------------------------- tensor-core gradient (H = 128)
-// Per-sample O_k rows on the tensor cores: used by psr_grad (BF16 precision,
-// dout == NULL) and by psr_step_batch for its BF16 gradient items.  Samples
-// go through in batches whose stash and layer arrays fit kTcBudget bytes.
-constexpr size_t kTcBudget = size_t(16) << 30;
-
-inline bool grad_tc_applies(const psr_params *p, const float *dout) {
-    return p->precision == PSR_BF16 && p->hidden == 128 && dout == nullptr;
-}
-
-struct GradTcWs {
-    int64_t B;          // samples per batch
-    float *stash, *gx[2], *gy[2], *gh, *dz, *dc;
-    void *images;
-};
-
-inline int64_t grad_tc_batch(int nL, int L, int64_t n) {
-    const size_t per = (stash_floats_per_sample(nL, 128, L) + 7 * (size_t)128 * stash_npad(L)) * sizeof(float);
-    int64_t B = (int64_t)(kTcBudget / per);
-    if (B < 1) B = 1;
-    if (B > n) B = n;
-    return B;
-}
-
-// Carves the batch buffers (call with a null-base Carver to size them).
-inline void grad_tc_carve(Carver &c, int nL, int L, int64_t B, GradTcWs &w) {
-    const size_t arr = (size_t)B * 128 * stash_npad(L);
-    w.B = B;
-    w.images = c.get<char>(bwd_tc_image_bytes(nL));
-    w.stash = c.get<float>((size_t)B * stash_floats_per_sample(nL, 128, L));
-    w.gx[0] = c.get<float>(arr);
-    w.gx[1] = c.get<float>(arr);
-    w.gy[0] = c.get<float>(arr);
-    w.gy[1] = c.get<float>(arr);
-    w.gh = c.get<float>(arr);
-    w.dz = c.get<float>(arr);
-    w.dc = c.get<float>(arr);
-}
-
-// Enqueues the O_k rows of n samples of L sites (bit-packed `bits`, W words
-// per row) into rows [n][P]; pk / theta: packed FP32 weights and the flat
-// parameters.  The transposed images are packed here.
-inline int enqueue_grad_tc(psr_context *ctx, int nL, int u1, const float *theta, const float *pk,
-                           const uint64_t *bits, int64_t n, int L, int W, float *rows, GradTcWs &w) {
-    cudaStream_t st = ctx->stream;
-    const ThetaLayout tl = theta_layout(nL, 128);
-    const F32Layout fl = f32_layout(nL, 128);
-    PSR_TRY(launch_pack_bwd_tc(theta, tl, w.images, st));
-    for (int64_t s0 = 0; s0 < n; s0 += w.B) {
-        const int64_t b = (n - s0 < w.B) ? n - s0 : w.B;
-        BwdTcArgs A{};
-        A.n = (int)b;
-        A.N = L;
-        A.Np = stash_npad(L);
-        A.W = W;
-        A.nL = nL;
-        A.P = tl.total;
-        A.tl = tl;
-        A.stash = w.stash;
-        A.stash_stride = (int64_t)stash_floats_per_sample(nL, 128, L);
-        A.wd = pk + fl.wd;
-        A.images = static_cast<const uint8_t *>(w.images);
-        A.bits = bits + s0 * W;
-        A.rows = rows + s0 * tl.total;
-        A.gh = w.gh;
-        A.dz = w.dz;
-        A.dc = w.dc;
-        A.pk = pk;
-        A.fl = fl;
-        A.u1 = u1;
-        A.status = ctx->status;
-        PSR_TRY(launch_fwd_tc(A, ctx->num_sms, st));  // fills the stash of the batch
-        for (int l = nL - 1; l >= 0; --l) {
-            A.l = l;
-            A.gx_in = w.gx[(l + 1) & 1];
-            A.gx_out = w.gx[l & 1];
-            A.gy = w.gy[l & 1];
-            A.gy_up = w.gy[(l + 1) & 1];
-            PSR_TRY(launch_bwd_tc_layer(A, ctx->num_sms, st));
-        }
-    }
-    return PSR_OK;
-}
-
-// ------------------------------------------------ FP32 gradients by layers
-// The layer-by-layer FP32 gradients hold every layer's arrays of a batch of
+// ------------------------------------------------ gradients by layers
+// The layer-by-layer gradients hold every layer's arrays of a batch of
 // samples; batches are sized to kGradBudget bytes of them.  A sample that
 // needs more by itself goes to the chunk-recompute kernel of its model, which
 // keeps only chunk carries.
@@ -413,6 +329,20 @@ inline int64_t grad_batch(size_t per, int64_t sites, int64_t n) {
     const int64_t most = ((int64_t)1 << 30) / sites;
     if (B > most) B = most;
     return B < n ? B : n;
+}
+
+// How the products of a gradient run.  FP32 sums over samples: three-part split
+// operands on the tensor cores from width 64 on (error against FP64 no larger
+// than with FP32 multiply-adds; the chain at hidden 64, 256 sites, 400 samples:
+// 0.9e-6 against 1.5e-6).  FP32 O_k rows: CUDA cores, because a single row
+// shows the tensor cores' rounding toward zero (4.4e-7 against 2.5e-7), which
+// cancels in a sum.  BF16 O_k rows: two-part split.
+inline gemm::Engine grad_engine(const psr_context *ctx, int H, bool sum, bool bf16_rows = false) {
+    return gemm::Engine{bf16_rows ? 2 : sum && H >= 64 ? 3 : 0, ctx->num_sms, ctx->status};
+}
+
+inline bool grad_bf16_rows(const psr_params *p, const float *dout) {
+    return p->precision == PSR_BF16 && p->hidden == 128 && dout == nullptr;
 }
 
 inline bool aligned16p(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -446,10 +376,10 @@ inline void grad_f32_carve(Carver &c, int nL, int H, int L, int64_t B, bool sum,
 
 // Enqueues the gradient of n samples of L sites (bit-packed, W words a row) in
 // batches of B through the arrays in A: O_k rows (dout == NULL) or the
-// dout-weighted sum into out.
+// dout-weighted sum into out.  bf16_rows: O_k rows of the BF16 path.
 inline int enqueue_grad_f32(psr_context *ctx, int nL, int H, int u1, const float *theta, const float *pk,
                             const uint64_t *bits, int64_t n, int L, int W, const float *dout, float *out,
-                            int64_t B, GradF32Args A) {
+                            int64_t B, GradF32Args A, bool bf16_rows) {
     cudaStream_t st = ctx->stream;
     A.tl = theta_layout(nL, H);
     A.fl = f32_layout(nL, H);
@@ -465,6 +395,7 @@ inline int enqueue_grad_f32(psr_context *ctx, int nL, int H, int u1, const float
     A.nL = nL;
     A.H = H;
     A.pk = pk;
+    A.en = grad_engine(ctx, H, dout != nullptr, bf16_rows);
     if (dout) {
         A.sm = GradSmall{0, 2 * H, 3 * H, 5 * H, 6 * H, 8 * H, 10 * H};
         A.small_stride = grad_f32_small_floats(H);

@@ -255,6 +255,10 @@ static int grad2d_layers(const psr_params *params, const uint8_t *spins, int64_t
     A.u1 = params->u1_mask;
     A.nL = nL;
     A.H = H;
+    A.en = grad_engine(ctx, H, dout != nullptr);
+    // weight gradients on CUDA cores: over ranges of 512 sites the tensor
+    // cores' error at hidden 256 was 8.8e-7 against 6.7e-7 (7.1e-7 before)
+    A.enw = grad_engine(ctx, H, false);
     A.tl = t2_layout(nL, H);
     A.f = f2_layout(nL, H);
     float *theta_ws = nullptr, *dout_ws = nullptr, *g_ws = nullptr, *pk = nullptr;
@@ -1008,6 +1012,7 @@ static int lru_grad_layers(const psr_params *params, const uint8_t *spins, int64
     A.u1 = params->u1_mask;
     A.nL = nL;
     A.H = H;
+    A.en = grad_engine(ctx, H, dout != nullptr);
     A.tl = tlru_layout(nL, H);
     A.f = lru_layout(nL, H);
     int64_t small_floats = 0;

@@ -13,16 +13,18 @@
 //             scan along the path, dz and dc; then gx of the layer below =
 //             W_z^T dz + W_hx^T dc + D^T gy for all
 //   weights   sums over patches of dz u^T, dc u^T, dc h(above)^T, gy h^T, gy u^T
-// The products are the FP32 tiles of psr_gemm.cuh.  What bounds it: the FP32
-// rate (72 H^2 operations a patch); the products of one patch row (n Lx / 2
-// sites) are the only ones that wait for each other.  Measured, hidden 256,
-// 1600 samples of 10 x 10, weighted sum: 5.3 ms with log psi of the samples
-// (the row-recompute kernel, psr_bwd2d.cu, a CTA per sample: 37.7 ms and a
-// forward of 4.3 ms, and 4.3 ms for log psi).
+// The products run on the engine the caller picks (psr_gemm_tc.cuh, split BF16
+// operands on the tensor cores; psr_gemm.cuh, FP32 multiply-adds), the weight
+// gradients on CUDA cores.  What bounds it: the weight gradients' FP32 rate (52
+// TFLOP/s); the products of one patch row (n Lx / 2 sites) are the only ones
+// that wait for each other.  Measured, hidden 256, 1600 samples of 10 x 10,
+// weighted sum with log psi of the samples: 3.3 ms (5.3 ms with FP32
+// multiply-adds throughout; the row-recompute kernel, psr_bwd2d.cu, a CTA per
+// sample: 37.7 ms and two forwards of 4.3 ms).
 #include <cuda_runtime.h>
 
 #include "psr_device.cuh"
-#include "psr_gemm.cuh"
+#include "psr_gemm_tc.cuh"
 #include "psr_internal.cuh"
 
 namespace psr {
@@ -120,6 +122,22 @@ struct EpiGyOf {
     int H;
     __device__ In load(int m, int j) const { return {ld4(dy + (size_t)m * H + j)}; }
     __device__ void store(int m, int j, float4 v, In in) const { st4(gy + (size_t)m * H + j, mul4(v, in.dy)); }
+};
+
+struct EpiGyAcc {  // gy = (gy + product) GELU'(y): the last of several products
+    struct In {
+        float4 gy, dy;
+    };
+    const float *dy;
+    float *gy;
+    int H;
+    __device__ In load(int m, int j) const {
+        const size_t i = (size_t)m * H + j;
+        return {ld4(gy + i), ld4(dy + i)};
+    }
+    __device__ void store(int m, int j, float4 v, In in) const {
+        st4(gy + (size_t)m * H + j, mul4(add4(in.gy, v), in.dy));
+    }
 };
 
 constexpr int kStep = 8;  // patches in flight per thread
@@ -281,21 +299,21 @@ cudaError_t launch_grad2d_fwd(const Grad2dArgs &A, float *logpsi, cudaStream_t s
         const int din = l ? H : 32, ldh = din + H;
         const float *u = l ? A.x[l - 1] : A.u0;
         const Args g1{M, H, 1, {{u, A.theta + tl.Wz[l], A.theta + tl.Wh[l], din, din, din, ldh}}};
-        if ((e = launch<true>(g1, EpiZC{A.theta + tl.bz[l], A.theta + tl.bh[l], A.a[l], A.c[l], H}, st))) return e;
+        if ((e = launch<true>(g1, EpiZC{A.theta + tl.bz[l], A.theta + tl.bh[l], A.a[l], A.c[l], H}, A.en, st))) return e;
         for (int j = 0; j < Py; ++j) {
             if (j > 0) {
                 const Args gv{R, H, 1, {{A.h[l] + (size_t)(j - 1) * R * H, A.theta + tl.Wh[l] + din, nullptr, H, H, ldh, 0}}};
-                if ((e = launch<false>(gv, EpiAdd{A.c[l] + (size_t)j * R * H, H}, st))) return e;
+                if ((e = launch<false>(gv, EpiAdd{A.c[l] + (size_t)j * R * H, H}, A.en, st))) return e;
             }
             scan_row_fwd_kernel<<<scan_blocks, 128, 0, st>>>(A, l, j);
             if ((e = cudaGetLastError())) return e;
         }
         const Args gy{M, H, 2,
                       {{A.h[l], A.theta + tl.C[l], nullptr, H, H, H, 0}, {u, A.theta + tl.D[l], nullptr, din, din, din, 0}}};
-        if ((e = launch<false>(gy, EpiX{l >= 2 ? A.h[l - 1] : nullptr, A.dy[l], A.x[l], H}, st))) return e;
+        if ((e = launch<false>(gy, EpiX{l >= 2 ? A.h[l - 1] : nullptr, A.dy[l], A.x[l], H}, A.en, st))) return e;
     }
     const Args go{M, 32, 1, {{A.x[nL - 1], A.wo32, nullptr, H, H, H, 0}}};
-    if ((e = launch<false>(go, EpiStore{A.logits, 32}, st))) return e;
+    if ((e = launch<false>(go, EpiStore{A.logits, 32}, A.en, st))) return e;
     if (logpsi) {
         softmax2d_kernel<<<(unsigned)((M + 127) / 128), 128, 0, st>>>(A, A.logp, false);
         sum_logp_kernel<<<(unsigned)((A.n + 7) / 8), 256, 0, st>>>(A.logp, A.n, Px, Py, logpsi);
@@ -328,9 +346,9 @@ cudaError_t launch_grad2d_bwd(const Grad2dArgs &A, cudaStream_t st) {
         WgArgs w = w0;
         w.n_pair = 1;
         w.p[0] = Pair{A.g, A.x[top], 32, H, 32, H, 16, M, tl.Wo, H, tl.bo};
-        if ((e = launch_wgrad(w, st))) return e;
+        if ((e = launch_wgrad(w, A.enw, st))) return e;
         const Args gx{M, H, 1, {{A.g, A.wo32t, nullptr, 32, 32, 32, 0}}};
-        if ((e = launch<false>(gx, EpiGyOf{A.dy[top], A.gy[top & 1], H}, st))) return e;
+        if ((e = launch<false>(gx, EpiGyOf{A.dy[top], A.gy[top & 1], H}, A.en, st))) return e;
     }
     for (int l = top; l >= 0; --l) {
         const int din = l ? H : 32, ldh = din + H;
@@ -338,11 +356,11 @@ cudaError_t launch_grad2d_bwd(const Grad2dArgs &A, cudaStream_t st) {
         float *gy = A.gy[l & 1];
         const bool resid = l + 1 < nL && l + 1 >= 2;
         const Args gc{M, H, 1, {{gy, A.pk + A.f.CT[l], nullptr, H, H, H, 0}}};
-        if ((e = launch<false>(gc, EpiStore{A.gh, H}, st))) return e;
+        if ((e = launch<false>(gc, EpiStore{A.gh, H}, A.en, st))) return e;
         for (int j = Py - 1; j >= 0; --j) {
             if (j + 1 < Py) {
                 const Args gv{R, H, 1, {{A.dc + (size_t)(j + 1) * R * H, A.pk + A.f.WhvT[l], nullptr, H, H, H, 0}}};
-                if ((e = launch<false>(gv, EpiAdd{A.gh + (size_t)j * R * H, H}, st))) return e;
+                if ((e = launch<false>(gv, EpiAdd{A.gh + (size_t)j * R * H, H}, A.en, st))) return e;
             }
             if (resid) scan_row_bwd_kernel<true><<<scan_blocks, 128, 0, st>>>(A, l, j);
             else scan_row_bwd_kernel<false><<<scan_blocks, 128, 0, st>>>(A, l, j);
@@ -361,16 +379,25 @@ cudaError_t launch_grad2d_bwd(const Grad2dArgs &A, cudaStream_t st) {
         v.p[1] = Pair{A.dc + (size_t)R * H, A.h[l], H, H, H, H, H, M - R, tl.Wh[l] + din, ldh, -1};
         if (l) {
             for (int q = 0; q < 2; ++q) w.p[w.n_pair++] = v.p[q];
-        } else if ((e = launch_wgrad(v, st))) {
+        } else if ((e = launch_wgrad(v, A.enw, st))) {
             return e;
         }
-        if ((e = launch_wgrad(w, st))) return e;
+        if ((e = launch_wgrad(w, A.enw, st))) return e;
         if (l) {
-            const Args gx{M, H, 3,
-                          {{A.gh, A.pk + A.f.WzT[l], nullptr, H, H, H, 0},
-                           {A.dc, A.pk + A.f.WhxT[l], nullptr, H, H, H, 0},
-                           {gy, A.pk + A.f.DT[l], nullptr, H, H, H, 0}}};
-            if ((e = launch<false>(gx, EpiGyOf{A.dy[l - 1], A.gy[(l - 1) & 1], H}, st))) return e;
+            const Seg seg[3] = {{A.gh, A.pk + A.f.WzT[l], nullptr, H, H, H, 0},
+                                {A.dc, A.pk + A.f.WhxT[l], nullptr, H, H, H, 0},
+                                {gy, A.pk + A.f.DT[l], nullptr, H, H, H, 0}};
+            float *to = A.gy[(l - 1) & 1];
+            if (A.en.split) {
+                // one product each, added in FP32: a tensor-core sum over 3 H
+                // terms would round (toward zero) three times as often
+                if ((e = launch<false>(Args{M, H, 1, {seg[0]}}, EpiStore{to, H}, A.en, st))) return e;
+                if ((e = launch<false>(Args{M, H, 1, {seg[1]}}, EpiAdd{to, H}, A.en, st))) return e;
+                if ((e = launch<false>(Args{M, H, 1, {seg[2]}}, EpiGyAcc{A.dy[l - 1], to, H}, A.en, st))) return e;
+            } else {
+                const Args gx{M, H, 3, {seg[0], seg[1], seg[2]}};
+                if ((e = launch<false>(gx, EpiGyOf{A.dy[l - 1], to, H}, A.en, st))) return e;
+            }
         }
     }
     if (!A.sum_out) return cudaSuccess;

@@ -25,8 +25,9 @@ struct ReadoutArgs {
 };
 
 // Readout adjoint g_t = 1/2 (s_t - P(1 | s_<t)) dout and, through `top`, the
-// adjoint of x: top(index, g wd).  One warp per kSites sites, E = H / 32 units
-// a lane; the sites' rows are in flight together (bound by reading x).
+// adjoint of x: top.store(index, g wd, top.load(index)).  One warp per kSites
+// sites, E = H / 32 units a lane; all the sites' rows are in flight together
+// (bound by the arrays' bytes).
 template <int E, class Top>
 __global__ void __launch_bounds__(256) grad_readout_kernel(const __grid_constant__ ReadoutArgs A,
                                                            const __grid_constant__ Top top) {
@@ -36,13 +37,17 @@ __global__ void __launch_bounds__(256) grad_readout_kernel(const __grid_constant
     if (m0 >= M) return;
     constexpr int H = 32 * E;
     float wd[E], x[kSites][E], d[kSites];
+    typename Top::In in[kSites][E];
 #pragma unroll
     for (int e = 0; e < E; ++e) wd[e] = A.wd[32 * e + lane];
 #pragma unroll
     for (int i = 0; i < kSites; ++i) {
         const float *p = A.x + (size_t)min(m0 + i, M - 1) * H + lane;
 #pragma unroll
-        for (int e = 0; e < E; ++e) x[i][e] = p[32 * e];
+        for (int e = 0; e < E; ++e) {
+            x[i][e] = p[32 * e];
+            in[i][e] = top.load((size_t)min(m0 + i, M - 1) * H + 32 * e + lane);
+        }
     }
 #pragma unroll
     for (int i = 0; i < kSites; ++i) {
@@ -71,7 +76,7 @@ __global__ void __launch_bounds__(256) grad_readout_kernel(const __grid_constant
         if (A.dout) g *= A.dout[s];
         if (lane == 0) A.g[m] = g;
 #pragma unroll
-        for (int e = 0; e < E; ++e) top((size_t)m * H + 32 * e + lane, g * wd[e]);
+        for (int e = 0; e < E; ++e) top.store((size_t)m * H + 32 * e + lane, g * wd[e], in[i][e]);
     }
 }
 

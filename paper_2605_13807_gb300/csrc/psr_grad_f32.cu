@@ -1,4 +1,4 @@
-// Reverse-mode gradient d log psi / d theta of the chain minGRU in FP32
+// Reverse-mode gradient d log psi / d theta of the chain minGRU
 // (derivative of Eq. minGRU and of the output map, Sec. II.F-G; the
 // energy-gradient estimates of Sec. III.B), layer by layer over a whole batch
 // of samples in site-major arrays [sample][site][unit]:
@@ -11,19 +11,21 @@
 //             dz = lambda (h_{t-1} - c) a (1 - a),  dc = lambda (1 - a);
 //             gx of layer l-1 = W_z^T dz + W_h^T dc + D^T gy
 //   weights   dC = sum gy h^T, dD = sum gy u^T, dW_z = sum dz u^T, dW_h = sum dc u^T
-// The products are the FP32 tiles of psr_gemm.cuh; the scans are one thread
-// per (sample, unit), coalesced over units.
+// The products run on the engine the caller picks (psr_gemm_tc.cuh: split BF16
+// operands on the tensor cores; psr_gemm.cuh: FP32 multiply-adds); the scans are
+// one thread per (sample, unit), coalesced over units.
 //
-// What bounds it: the FP32 rate in the products (54 H^2 operations a site) and
-// HBM for the arrays between them (about 75 arrays of 4 H bytes a site): at
-// hidden 64, 4096 samples of 100 sites (weighted sum) 2.1 ms of the 2.9 ms are
-// products at 33 to 46 TFLOP/s, the rest streams.  The chunk-recompute kernel
-// (psr_bwd.cu: a CTA per sample, a thread per unit, the sum by reductions in
-// L2 every 16 sites) takes 11.3 ms there.
+// What bounds it: HBM, for the arrays between the products (about 75 arrays of
+// 4 H bytes a site; the products run at 0.5 to 0.8 of the measured rate for
+// their bytes, the weight gradients at 0.4).  Measured, per-sample kernels of
+// a CTA each with reductions in L2 (psr_bwd.cu) / FP32 multiply-adds / split
+// operands: weighted sum, hidden 64, 4096 samples of 100 sites 11.3 / 2.9 / 2.1
+// ms; O_k rows at BF16, hidden 128, 2048 samples of 100 sites 2.0 ms (two-part
+// split; 5.7 ms in unit-major arrays with unpipelined products before).
 #include <cuda_runtime.h>
 
 #include "psr_device.cuh"
-#include "psr_gemm.cuh"
+#include "psr_gemm_tc.cuh"
 #include "psr_grad_common.cuh"
 #include "psr_internal.cuh"
 
@@ -140,9 +142,11 @@ __global__ void __launch_bounds__(128) grad_scan_fwd_kernel(const __grid_constan
 }
 
 struct TopGy {  // gy of the top layer from gx = g wd
+    using In = float;
     const float *dy;
     float *gy;
-    __device__ void operator()(size_t i, float gx) const { gy[i] = gx * dy[i]; }
+    __device__ float load(size_t i) const { return dy[i]; }
+    __device__ void store(size_t i, float gx, float d) const { gy[i] = gx * d; }
 };
 
 // reverse scan of a layer l >= 1: dz (in place of gh) and dc
@@ -295,14 +299,14 @@ cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t st) {
     for (int l = 0; l < nL; ++l) {
         if (l > 0) {
             Args g{M, H, 1, {{A.u[l - 1], A.theta + tl.Wz[l], A.theta + tl.Wh[l], H, H, H, H}}};
-            if ((e = launch<true>(g, EpiProj{A.pk + A.fl.bz[l], A.pk + A.fl.bh[l], A.a[l], A.c[l], H}, st))) return e;
+            if ((e = launch<true>(g, EpiProj{A.pk + A.fl.bz[l], A.pk + A.fl.bh[l], A.a[l], A.c[l], H}, A.en, st))) return e;
         }
         grad_scan_fwd_kernel<<<scan_blocks, 128, 0, st>>>(A, l);
         if ((e = cudaGetLastError())) return e;
         Args g{M, H, l ? 2 : 1, {{A.h[l], A.theta + tl.C[l], nullptr, H, H, H, H}, {}}};
         if (l) g.seg[1] = Seg{A.u[l - 1], A.theta + tl.D[l], nullptr, H, H, H, H};
         const EpiOut eo{l ? nullptr : A.pk + A.fl.DU0, l >= 2 ? A.h[l - 1] : nullptr, A.bits, A.dy[l], A.u[l], H, A.N, A.W};
-        if ((e = launch<false>(g, eo, st))) return e;
+        if ((e = launch<false>(g, eo, A.en, st))) return e;
     }
     const ReadoutArgs ro{A.n, A.N, H, A.W, A.u1, A.bits, A.u[nL - 1], A.pk + A.fl.wd, A.pk + A.fl.bd, A.dout, A.g,
                          A.small + A.sm.Wo, A.small + A.sm.bo, A.small_stride};
@@ -312,7 +316,7 @@ cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t st) {
     for (int l = nL - 1; l >= 0; --l) {
         float *gy = A.gy[l & 1];
         Args gc{M, H, 1, {{gy, A.pk + A.fl.CT[l], nullptr, H, H, H, H}}};
-        if ((e = launch<false>(gc, EpiStore{A.gh, H}, st))) return e;
+        if ((e = launch<false>(gc, EpiStore{A.gh, H}, A.en, st))) return e;
         if (l == 0) grad_scan_bwd0_kernel<<<scan_blocks, 128, 0, st>>>(A);
         else if (l + 1 < nL) grad_scan_bwd_kernel<true><<<scan_blocks, 128, 0, st>>>(A, l);
         else grad_scan_bwd_kernel<false><<<scan_blocks, 128, 0, st>>>(A, l);
@@ -332,14 +336,14 @@ cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t st) {
         w.seg_stride = range;
         w.out = A.rows;
         w.out_stride = tl.total;
-        if ((e = launch_wgrad(w, st))) return e;
+        if ((e = launch_wgrad(w, A.en, st))) return e;
         if (l > 0) {
             // W^T as [input unit][output unit] rows: the packed transposes
             Args gx{M, H, 3,
                     {{A.gh, A.pk + A.fl.WzT[l], nullptr, H, H, H, H},
                      {A.dc, A.pk + A.fl.WhT[l], nullptr, H, H, H, H},
                      {gy, A.pk + A.fl.DT[l], nullptr, H, H, H, H}}};
-            if ((e = launch<false>(gx, EpiGy{A.dy[l - 1], A.gy[(l - 1) & 1], H}, st))) return e;
+            if ((e = launch<false>(gx, EpiGy{A.dy[l - 1], A.gy[(l - 1) & 1], H}, A.en, st))) return e;
         }
     }
     if (!A.sum_out) return cudaSuccess;

@@ -12,15 +12,15 @@
 //             B_im^T d(Bu)_im + D dy + gx (residual)
 //   weights   sums over sites of da y^T, dg y^T, dy h^T, d(Bu) u^T; lambda,
 //             gamma, D and the one-hot columns of layer 0 in the reverse scan
-// The products are the FP32 tiles of psr_gemm.cuh.  What bounds it: the FP32
-// rate (80 H^2 operations a site) and HBM for about 110 arrays of 4 H bytes a
-// site.  Measured, hidden 64, 1024 samples of 256 sites, weighted sum: 3.28 ms
-// (2.4 ms of it products, at 38 to 47 TFLOP/s); the chunk-recompute kernel
-// (psr_bwd_lru.cu, a CTA per sample) with its forward takes 10.65 ms.
+// The products run on the engine the caller picks (psr_gemm_tc.cuh, split BF16
+// operands on the tensor cores; psr_gemm.cuh, FP32 multiply-adds).  What bounds
+// it: HBM for about 110 arrays of 4 H bytes a site.  Measured, hidden 64, 1024
+// samples of 256 sites, weighted sum: 2.3 ms (3.3 ms with FP32 multiply-adds;
+// 10.7 ms for the chunk-recompute kernel, psr_bwd_lru.cu, and its forward).
 #include <cuda_runtime.h>
 
 #include "psr_device.cuh"
-#include "psr_gemm.cuh"
+#include "psr_gemm_tc.cuh"
 #include "psr_grad_common.cuh"
 #include "psr_internal.cuh"
 
@@ -93,12 +93,16 @@ struct EpiDh {
 
 // gx of a block's output turned into the adjoints of its GLU
 struct TopGlu {
+    struct In {
+        float p1, p2;
+    };
     const float *p1, *p2;
     float *gx, *da, *dg;
-    __device__ void operator()(size_t i, float v) const {
+    __device__ In load(size_t i) const { return {p1[i], p2[i]}; }
+    __device__ void store(size_t i, float v, In in) const {
         gx[i] = v;
-        da[i] = v * p1[i];
-        dg[i] = v * p2[i];
+        da[i] = v * in.p1;
+        dg[i] = v * in.p2;
     }
 };
 
@@ -340,15 +344,15 @@ cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t st) {
         const float *u = l ? A.x[l - 1] : nullptr;
         if (l) {
             const Args g{M, H, 1, {{u, A.theta + tl.Bre[l], A.theta + tl.Bim[l], H, H, H, H}}};
-            if ((e = launch<true>(g, EpiBu{A.br[l], A.bi[l], H}, st))) return e;
+            if ((e = launch<true>(g, EpiBu{A.br[l], A.bi[l], H}, A.en, st))) return e;
         }
         lru_scan_fwd_kernel<<<scan_blocks, 128, 0, st>>>(A, l);
         if ((e = cudaGetLastError())) return e;
         const Args gy{M, H, 2,
                       {{A.hr[l], A.theta + tl.Cre[l], nullptr, H, H, H, H}, {A.hn[l], A.theta + tl.Cim[l], nullptr, H, H, H, H}}};
-        if ((e = launch<false>(gy, EpiY{A.pk + A.f.D[l], u, A.bits, A.y[l], H, A.N, A.W}, st))) return e;
+        if ((e = launch<false>(gy, EpiY{A.pk + A.f.D[l], u, A.bits, A.y[l], H, A.N, A.W}, A.en, st))) return e;
         const Args gg{M, H, 1, {{A.y[l], A.theta + tl.Wa[l], A.theta + tl.Wg[l], H, H, H, H}}};
-        if ((e = launch<true>(gg, EpiGlu{A.pk + A.f.ba[l], A.pk + A.f.bg[l], u, A.p1[l], A.p2[l], A.x[l], H}, st))) return e;
+        if ((e = launch<true>(gg, EpiGlu{A.pk + A.f.ba[l], A.pk + A.f.bg[l], u, A.p1[l], A.p2[l], A.x[l], H}, A.en, st))) return e;
     }
     const int top = nL - 1;
     const ReadoutArgs ro{A.n, A.N, H, A.W, A.u1, A.bits, A.x[top], A.pk + A.f.wd, A.pk + A.f.bd, A.dout, A.g,
@@ -361,9 +365,9 @@ cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t st) {
         const float *u = l ? A.x[l - 1] : nullptr;
         const Args gy{M, H, 2,
                       {{A.da, A.pk + A.f.WaT[l], nullptr, H, H, H, H}, {A.dg, A.pk + A.f.WgT[l], nullptr, H, H, H, H}}};
-        if ((e = launch<false>(gy, EpiStore{A.dy, H}, st))) return e;
+        if ((e = launch<false>(gy, EpiStore{A.dy, H}, A.en, st))) return e;
         const Args gh{M, H, 1, {{A.dy, A.pk + A.f.CreT[l], A.pk + A.f.CimT[l], H, H, H, H}}};
-        if ((e = launch<true>(gh, EpiDh{A.dhr, A.dhi, H}, st))) return e;
+        if ((e = launch<true>(gh, EpiDh{A.dhr, A.dhi, H}, A.en, st))) return e;
         if (l) lru_scan_bwd_kernel<false><<<scan_blocks, 128, 0, st>>>(A, l);
         else lru_scan_bwd_kernel<true><<<scan_blocks, 128, 0, st>>>(A, l);
         if ((e = cudaGetLastError())) return e;
@@ -381,12 +385,12 @@ cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t st) {
         w.len = w.step = w.seg_len = w.seg_stride = range;
         w.out = A.rows;
         w.out_stride = tl.total;
-        if ((e = launch_wgrad(w, st))) return e;
+        if ((e = launch_wgrad(w, A.en, st))) return e;
         if (l) {
             const Args gx{M, H, 2,
                           {{A.dhr, A.pk + A.f.BreT[l], nullptr, H, H, H, H}, {A.dhi, A.pk + A.f.BimT[l], nullptr, H, H, H, H}}};
             const EpiGx ex{A.pk + A.f.D[l], A.dy, A.p1[l - 1], A.p2[l - 1], A.gx, A.da, A.dg, H};
-            if ((e = launch<false>(gx, ex, st))) return e;
+            if ((e = launch<false>(gx, ex, A.en, st))) return e;
         }
     }
     if (!A.sum_out) return cudaSuccess;

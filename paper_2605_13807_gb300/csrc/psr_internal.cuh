@@ -70,19 +70,6 @@ struct FwdGroup {
     float *carries_out;          // mode 0, optional: [n][nch][nL][H]
 };
 
-// Stash of one sample for the tensor-core backward, written by its own
-// forward (launch_fwd_tc): for layer l and quantity q (kStashA: gate a, kStashC:
-// candidate c = W_h u + b_h, kStashH: state h, kStashY: output-map
-// pre-activation y, residual included) a [H][Npad] block at
-// ((l * kStashQ + q) * H) * Npad, then the readout adjoint g [Npad] at
-// nL * kStashQ * H * Npad, g_t = 1/2 (s_t - P(1 | s_<t)) (0 where the
-// zero-magnetisation mask forces s_t).  Npad = N rounded up to 64; every
-// value at t >= N is 0.
-enum { kStashA = 0, kStashC = 1, kStashH = 2, kStashY = 3, kStashQ = 4 };
-__host__ __device__ inline int stash_npad(int N) { return (N + 63) & ~63; }
-__host__ __device__ inline size_t stash_floats_per_sample(int nL, int H, int N) {
-    return ((size_t)nL * kStashQ * H + 1) * (size_t)stash_npad(N);
-}
 struct FwdJobs {
     int mode;
     int n_groups;
@@ -410,11 +397,20 @@ cudaError_t launch_adam(const float *theta, const float *grad, int64_t P, float 
 // tensors' places in theta (sum_out == NULL), or partial rows
 // [ceil(n N / grad_f32_range)][P] and per-sample entries small
 // [n][grad_f32_small_floats], summed into sum_out [P] (added to it if add).
+namespace gemm {
+// How the products of a gradient run: split 0 on CUDA cores, 2 or 3 on the
+// tensor cores (psr_gemm_tc.cuh).
+struct Engine {
+    int split, num_sms;
+    int *status;
+};
+}  // namespace gemm
 struct GradSmall {
     int64_t Wz0, bz0, Wh0, bh0, D0, Wo, bo;
 };
 struct GradF32Args {
     int n, N, W, u1, nL, H;
+    gemm::Engine en;
     const float *theta;  // 16-byte aligned
     ThetaLayout tl;
     const float *pk;
@@ -443,6 +439,7 @@ struct GradLruSmall {
 };
 struct GradLruArgs {
     int n, N, W, u1, nL, H;
+    gemm::Engine en;
     const float *theta;  // 16-byte aligned
     TLruLayout tl;
     const float *pk;
@@ -472,6 +469,7 @@ cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t stream);
 // launch_grad2d_bwd only.
 struct Grad2dArgs {
     int n, Lx, Ly, W, u1, nL, H;
+    gemm::Engine en, enw;  // products; weight gradients
     const float *theta;
     T2Layout tl;
     const float *pk;
@@ -506,40 +504,6 @@ struct BwdJobs {
     int64_t first[kMaxGroups + 1];
     BwdGroup g[kMaxGroups];
 };
-// Tensor-core backward (hidden 128; psr_bwd_tc.cu): one layer at a time over
-// the samples of a batch, from the FP32 forward's stash.  Arrays [n][H][Np]
-// FP32 (unit-major, Np = stash_npad(N)).
-struct BwdTcArgs {
-    int n, N, Np, W, nL, l;
-    int64_t P;
-    ThetaLayout tl;
-    const float *stash;      // batch stash, stash_stride floats per sample
-    int64_t stash_stride;
-    const float *wd;         // readout logit-difference weights [H]
-    const uint8_t *images;   // launch_pack_bwd_tc output
-    const uint64_t *bits;    // [n][W] bit-packed spins of the batch
-    const float *gx_in;      // gradient w.r.t. this layer's output x^{l+1} (l < nL - 1)
-    float *gx_out;           // gradient w.r.t. its input x^l (l >= 1)
-    float *gy;               // gx_in (.) GELU'(y) of this layer
-    const float *gy_up;      // gy of layer l + 1 (its residual input is h^l)
-    float *gh;               // C^T gy
-    float *dz, *dc;          // gate and candidate adjoints
-    float *rows;             // [n][P] O_k rows of the batch
-    const float *pk;         // packed FP32 weights (layer-0 tables, biases, readout)
-    F32Layout fl;
-    int u1;
-    int *status;
-};
-// The forward that fills the stash of a batch (all layers and the readout
-// adjoint) with the same split-BF16 tensor-core products.
-cudaError_t launch_fwd_tc(const BwdTcArgs &A, int num_sms, cudaStream_t stream);
-size_t bwd_tc_image_bytes(int nL);
-cudaError_t launch_pack_bwd_tc(const float *theta, const ThetaLayout &tl, void *images, cudaStream_t stream);
-cudaError_t launch_bwd_tc_layer(const BwdTcArgs &A, int num_sms, cudaStream_t stream);
-// Sets the tensor-core backward kernels' shared-memory attributes (once per
-// device; call before a stream capture that will contain their launches).
-cudaError_t prepare_bwd_tc();
-
 // Sets the backward kernel's shared-memory attribute (done by every launch;
 // call it before a stream capture that will contain a launch).
 cudaError_t prepare_bwd_f32(int H, int nL);
