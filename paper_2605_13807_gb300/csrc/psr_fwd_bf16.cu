@@ -92,6 +92,31 @@ constexpr size_t PK_TOTAL = PK_TMEM + (size_t)kTmemMats * kMatBytes;
 using namespace tc;
 using namespace bf16m;
 
+// Chunk boundaries are counted from the end of the sequence, as far as whole
+// groups of 8 sites allow: chunk c holds sites 32 c - off .. 32 c - off + 31, and
+// the first off sites of chunk 0 lie before the sequence (their values are
+// computed and dropped; the scans start from zero at group off / 8).  A
+// connected configuration resumes at the chunk of its first flipped site and
+// runs to the last one, so empty sites at the end cost every configuration
+// and empty sites at the start almost none: 94 evaluated sites of 100-site
+// configurations with chunks from site 0, 70 so (E_loc of 2048 samples of
+// 10 x 10: 12.05 against 9.74 ms).  The start in mid-chunk costs the kernel 2 %,
+// so an offset under 2 % of the sites (a gain under 4 %) is left at zero.
+__host__ __device__ __forceinline__ int chunk_offset(int N) {
+    const int off = ((N + CH - 1) / CH * CH - N) & ~7;
+    return off * 50 >= N ? off : 0;
+}
+
+// The 32 spins from site t0 (a multiple of 8, at least -24); sites outside the
+// sequence read as 0.
+__device__ __forceinline__ uint32_t chunk_spins(const uint64_t *row, int t0) {
+    if (t0 < 0) return (uint32_t)row[0] << -t0;
+    const int sh = t0 & 63;
+    uint64_t v = row[t0 >> 6] >> sh;
+    if (sh > 32) v |= row[(t0 >> 6) + 1] << (64 - sh);  // rows end with a zero word
+    return (uint32_t)v;
+}
+
 // B operand: an activation tile, MN-major (kN sites = kRowBytes per K row),
 // 64-byte (kN = 32) or 128-byte (kN = 64) swizzle; 8-row groups of kAtom
 // bytes along K.  The kN sites are one swizzle atom wide, so only the
@@ -227,12 +252,13 @@ __device__ __forceinline__ void issue(int s, uint32_t sbase) {
 // accumulators: a = sigmoid(z + b_z), h_t = a_t h_{t-1} + (1 - a_t)(h~_t + b_h).
 // The sites go to chunks 2 hh, 2 hh + 1 of this sequence's part (cbase) of
 // the tile row.
-template <int L, class SH>
+template <int L, class SH, bool kOff>
 __device__ __forceinline__ void gates_scan16(const uint32_t (&rz)[16], const uint32_t (&rc)[16], int hh,
                                              float2 hbz2, float2 bh2, float &h, float (&h1)[32],
-                                             uint8_t *tileH, int j, int cbase) {
+                                             uint8_t *tileH, int j, int cbase, int rg) {
 #pragma unroll
     for (int gg = 0; gg < 2; ++gg) {
+        if (kOff && 2 * hh + gg == rg) h = 0.0f;  // the sequence starts here
         float hv[8];
 #pragma unroll
         for (int i = 0; i < 8; i += 2) {
@@ -256,13 +282,14 @@ __device__ __forceinline__ void gates_scan16(const uint32_t (&rz)[16], const uin
 // One dense layer (l = 1 or 2) of one stream's step, from the projection
 // MMAs to the output epilogue.  act: this warpgroup's sequence has a chunk in
 // this step (an idle warpgroup keeps the stream's barriers and waits but
-// computes nothing).  h1: layer 1 writes its FP32 h there (the residual of
+// computes nothing).  rg: the group of 8 sites the sequence starts with, if it
+// starts in this chunk, else -1 (kOff; not used otherwise).  h1: layer 1 writes its FP32 h there (the residual of
 // layer 2); layer 2 adds it and overwrites it with the layer output x3.
-template <int L, class SH, class WaitF, class PubF>
+template <int L, class SH, bool kOff, class WaitF, class PubF>
 __device__ __forceinline__ void dense_layer(bool act, float hbz, float bh, uint8_t *tileX, uint8_t *tileH,
                                             uint32_t sbase, int s, uint32_t accZ, uint32_t accC,
-                                            bool issuer, int j, int cbase, float &carry, float (&h1)[32],
-                                            WaitF &sync_wait, PubF &publish) {
+                                            bool issuer, int j, int cbase, int rg, float &carry,
+                                            float (&h1)[32], WaitF &sync_wait, PubF &publish) {
     if (issuer) issue<L == 1 ? 1 : 3, SH>(s, sbase);
     sync_wait();
     if (act) {
@@ -276,9 +303,9 @@ __device__ __forceinline__ void dense_layer(bool act, float hbz, float bh, uint8
             tmem_wait_ld16x2(z0, c0);
             tmem_ld16(accZ + 16, z1);
             tmem_ld16(accC + 16, c1);
-            gates_scan16<L, SH>(z0, c0, 0, hbz2, bh2, h, h1, tileH, j, cbase);
+            gates_scan16<L, SH, kOff>(z0, c0, 0, hbz2, bh2, h, h1, tileH, j, cbase, rg);
             tmem_wait_ld16x2(z1, c1);
-            gates_scan16<L, SH>(z1, c1, 1, hbz2, bh2, h, h1, tileH, j, cbase);
+            gates_scan16<L, SH, kOff>(z1, c1, 1, hbz2, bh2, h, h1, tileH, j, cbase, rg);
         } else {
             // layer 2 keeps the residual h1 live: one half at a time
 #pragma unroll
@@ -287,7 +314,7 @@ __device__ __forceinline__ void dense_layer(bool act, float hbz, float bh, uint8
                 tmem_ld16(accZ + 16 * hh, z);
                 tmem_ld16(accC + 16 * hh, cc);
                 tmem_wait_ld16x2(z, cc);
-                gates_scan16<L, SH>(z, cc, hh, hbz2, bh2, h, h1, tileH, j, cbase);
+                gates_scan16<L, SH, kOff>(z, cc, hh, hbz2, bh2, h, h1, tileH, j, cbase, rg);
             }
         }
         carry = h;
@@ -325,6 +352,8 @@ __device__ __forceinline__ void dense_layer(bool act, float hbz, float bh, uint8
 // each; thread j of a stream's warpgroup owns hidden unit j (TMEM lane j) for
 // the 32 sites of the chunk.  Each stream walks the chunks of one job at a
 // time (its own job loop, no step-synchronous bookkeeping).
+// kOff: some sequence starts in mid-chunk (chunk_offset).
+template <bool kOff>
 __global__ void __launch_bounds__(kThreads, 1)
 fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ pkb,
                  const float *__restrict__ pk, F32Layout fl) {
@@ -465,8 +494,9 @@ fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__
             sample = e[0];
             p = e[1];
             q = e[2];
-            c0 = p / CH;
+            c0 = (p + (kOff ? chunk_offset(N) : 0)) / CH;
         }
+        const int off = kOff ? chunk_offset(N) : 0;
         const uint64_t *row = G.bits + (int64_t)sample * G.W;
         float cr[NL] = {0.0f, 0.0f, 0.0f};  // scan carries
         if (c0 > 0) {
@@ -475,7 +505,7 @@ fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__
             cr[1] = cin[H];
             cr[2] = cin[2 * H];
         }
-        int n_up = G.u1 ? count_up_before(row, c0 * CH) : 0;
+        int n_up = G.u1 ? count_up_before(row, max(c0 * CH - off, 0)) : 0;
         float acc = 0.0f;
         // the 64-bit word holding the current chunk's 32 spins; the spin
         // before the chunk (s_{t0-1}) of the unflipped sample
@@ -513,7 +543,7 @@ fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__
                 const float d = bd + red[lane] + red[32 + lane] + red[64 + lane] + red[96 + lane];
                 const int tt = rd_t0 + lane;
                 float sv = 0.0f;
-                if (tt < N) {
+                if ((!kOff || tt >= 0) && tt < N) {
                     const int sbit = (int)((rd_cur >> lane) & 1u);
                     const int nu = n_up + __popc(rd_cur & ((1u << lane) - 1u));
                     const float lp = site_logp_fast(d, sbit, u1_forced(G.u1, N, tt, nu));
@@ -527,26 +557,30 @@ fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__
             n_up += __popc(rd_cur);
             if (M.abort_flag[s]) aborted = true;  // uniform: read after the barrier
         };
-        uint64_t word = row[c0 >> 1];
-        uint32_t next_prev =
-            (c0 == 0) ? 0u : (uint32_t)(((c0 & 1) ? (word >> 31) : (row[(c0 >> 1) - 1] >> 63)) & 1ull);
+        uint64_t word = kOff ? 0 : row[c0 >> 1];
+        uint32_t next_cur = kOff ? chunk_spins(row, c0 * CH - off) : 0u;  // kOff: the chunk's spins themselves
+        uint32_t next_prev = (c0 == 0) ? 0u
+                             : kOff    ? chunk_spins(row, (c0 - 1) * CH - off) >> 31
+                                       : (uint32_t)(((c0 & 1) ? (word >> 31) : (row[(c0 >> 1) - 1] >> 63)) & 1ull);
 
         for (int c = c0; c < nch && !aborted; ++c) {
-            const int t0 = c * CH;
+            const int t0 = c * CH - off;
+            const int rg = (c == 0) ? off >> 3 : -1;  // group of 8 sites the sequence starts with
             if (G.carries_out) {
                 float *co = G.carries_out + (((int64_t)sample * nch + c) * NL) * H + j;
                 co[0] = cr[0];
                 co[H] = cr[1];
                 co[2 * H] = cr[2];
             }
-            uint32_t cur = (uint32_t)(word >> (32 * (c & 1)));
+            uint32_t cur = kOff ? next_cur : (uint32_t)(word >> (32 * (c & 1)));
             uint32_t prev = next_prev;
             next_prev = cur >> 31;
             // the next word of spins and this chunk's reference log P are
             // fetched now, long before they are needed
-            if ((c & 1) && c + 1 < nch) word = row[(c + 1) >> 1];
+            if (kOff && c + 1 < nch) next_cur = chunk_spins(row, t0 + CH);
+            if (!kOff && (c & 1) && c + 1 < nch) word = row[(c + 1) >> 1];
             float lp_ref = 0.0f;
-            if (jb.mode == 1 && (warp & 3) == 0 && t0 + lane < N)
+            if (jb.mode == 1 && (warp & 3) == 0 && (!kOff || t0 + lane >= 0) && t0 + lane < N)
                 lp_ref = G.logp_ref[(int64_t)sample * N + t0 + lane];
 #pragma unroll
             for (int f = 0; f < 2; ++f) {
@@ -569,11 +603,12 @@ fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__
                 for (int g = 0; g < 4; ++g) {
                     float hv[8];
                     uint32_t du[8];
+                    if (kOff && g == rg) h = 0.0f;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const bool sb = (inbits >> (8 * g + i)) & 1u;
                         float a = sb ? a0_2 : a0_1, b = sb ? b0_2 : b0_1, dd = sb ? d0_2 : d0_1;
-                        if (g == 0 && i == 0 && seq_start) { a = a0_0; b = b0_0; dd = d0_0; }
+                        if (i == 0 && (kOff ? g == rg : (g == 0 && seq_start))) { a = a0_0; b = b0_0; dd = d0_0; }
                         h = fmaf(a, h, b);
                         hv[i] = h;
                         du[i] = __float_as_uint(dd);
@@ -609,10 +644,10 @@ fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__
             publish();
 
             // ---------------- layers 1 and 2
-            dense_layer<1, SH>(true, hbz1, bh1, tileX, tileH, sbase, s, accZ, accC, issuer, j, 0, cr[1], h1,
-                               sync_wait, publish);
-            dense_layer<2, SH>(true, hbz2, bh2, tileX, tileH, sbase, s, accZ, accC, issuer, j, 0, cr[2], h1,
-                               sync_wait, publish);
+            dense_layer<1, SH, kOff>(true, hbz1, bh1, tileX, tileH, sbase, s, accZ, accC, issuer, j, 0, rg,
+                                     cr[1], h1, sync_wait, publish);
+            dense_layer<2, SH, kOff>(true, hbz2, bh2, tileX, tileH, sbase, s, accZ, accC, issuer, j, 0, rg,
+                                     cr[2], h1, sync_wait, publish);
             // x3 (in h1) is read out while the next chunk's layer-0 MMAs run
             rd_cur = cur;
             rd_t0 = t0;
@@ -778,12 +813,11 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
     enum { kNeed = 0, kActive = 1, kDone = 2 };
     int state = kNeed;
     int slot = 1;             // RdInfo slot of the current job
-    int N = 0, nch = 0, c = 0, p = -1, q = -1, n_up = 0;
+    int N = 0, nch = 0, c = 0, p = -1, q = -1, n_up = 0, off = 0;
     const uint64_t *row = nullptr;
     const float *lpref_row = nullptr;  // mode 1: log P of the sample, per site
     float *co_row = nullptr;           // mode 0: chunk carries out of this sample
-    uint64_t word = 0;
-    uint32_t next_prev = 0;
+    uint32_t next_cur = 0, next_prev = 0;
     float cr[NL] = {0.0f, 0.0f, 0.0f};  // scan carries
     float h1[32];  // FP32 h of layer 1 (residual of layer 2), then the layer-2 output x3
 
@@ -826,7 +860,7 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
                             *red_addr(96 + lane);
             const int tt = rd_t0 + lane;
             float sv = 0.0f;
-            if (tt < ri.N) {
+            if (tt >= 0 && tt < ri.N) {
                 const int sbit = (int)((rd_cur >> lane) & 1u);
                 const int nu = rd_nup + __popc(rd_cur & ((1u << lane) - 1u));
                 const float lp = site_logp_fast(d, sbit, u1_forced(ri.u1, ri.N, tt, nu));
@@ -863,6 +897,7 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
                 const long long lj = job - M.base[gi];
                 N = G.N;
                 nch = (N + CH - 1) / CH;
+                off = chunk_offset(N);
                 int sample, c0 = 0;
                 p = -1;
                 q = -1;
@@ -873,7 +908,7 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
                     sample = e[0];
                     p = e[1];
                     q = e[2];
-                    c0 = p / CH;
+                    c0 = (p + off) / CH;
                 }
                 row = G.bits + (int64_t)sample * G.W;
                 cr[0] = cr[1] = cr[2] = 0.0f;
@@ -883,13 +918,12 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
                     cr[1] = cin[H];
                     cr[2] = cin[2 * H];
                 }
-                n_up = G.u1 ? count_up_before(row, c0 * CH) : 0;
+                n_up = G.u1 ? count_up_before(row, max(c0 * CH - off, 0)) : 0;
                 lpref_row = (jb.mode == 1) ? G.logp_ref + (int64_t)sample * N : nullptr;
                 co_row = (jb.mode == 0 && G.carries_out) ? G.carries_out + (int64_t)sample * nch * NL * H + j
                                                          : nullptr;
-                word = row[c0 >> 1];
-                next_prev = (c0 == 0) ? 0u
-                                      : (uint32_t)(((c0 & 1) ? (word >> 31) : (row[(c0 >> 1) - 1] >> 63)) & 1ull);
+                next_cur = chunk_spins(row, c0 * CH - off);
+                next_prev = (c0 == 0) ? 0u : chunk_spins(row, (c0 - 1) * CH - off) >> 31;
                 c = c0;
                 slot ^= 1;
                 if (leader) {
@@ -908,7 +942,8 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
         // ---------------- layer 0: lookup gates, scan -> tile H; the one-hot
         // input's output term D0 u -> this sequence's accumulator columns,
         // which the layer-0 MMAs then add C0 h to
-        const int t0 = c * CH;
+        const int t0 = c * CH - off;
+        const int rg = (c == 0) ? off >> 3 : -1;  // group of 8 sites the sequence starts with
         uint32_t cur = 0u;
         float lp_ref = 0.0f;
         if (act) {
@@ -918,13 +953,13 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
                 co[H] = cr[1];
                 co[2 * H] = cr[2];
             }
-            cur = (uint32_t)(word >> (32 * (c & 1)));
+            cur = next_cur;
             uint32_t prev = next_prev;
             next_prev = cur >> 31;
-            // the next word of spins and this chunk's reference log P are
+            // the next chunk's spins and this chunk's reference log P are
             // fetched now, long before they are needed
-            if ((c & 1) && c + 1 < nch) word = row[(c + 1) >> 1];
-            if (lpref_row && (warp & 3) == 0 && t0 + lane < N) lp_ref = lpref_row[t0 + lane];
+            if (c + 1 < nch) next_cur = chunk_spins(row, t0 + CH);
+            if (lpref_row && (warp & 3) == 0 && t0 + lane >= 0 && t0 + lane < N) lp_ref = lpref_row[t0 + lane];
 #pragma unroll
             for (int f = 0; f < 2; ++f) {
                 const int x = f ? q : p;
@@ -935,17 +970,17 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
             if (nvalid < 32) cur &= (1u << nvalid) - 1u;
             // bit i = s_{t-1} for site t = t0 + i
             const uint32_t inbits = (cur << 1) | prev;
-            const bool seq_start = (t0 == 0);  // site 0 has no predecessor
             float h = cr[0];
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
                 float hv[8];
                 uint32_t du[8];
+                if (g == rg) h = 0.0f;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
                     const bool sb = (inbits >> (8 * g + i)) & 1u;
                     float a = sb ? a0_2 : a0_1, b = sb ? b0_2 : b0_1, dd = sb ? d0_2 : d0_1;
-                    if (g == 0 && i == 0 && seq_start) { a = a0_0; b = b0_0; dd = d0_0; }
+                    if (i == 0 && g == rg) { a = a0_0; b = b0_0; dd = d0_0; }  // no predecessor
                     h = fmaf(a, h, b);
                     hv[i] = h;
                     du[i] = __float_as_uint(dd);
@@ -994,10 +1029,10 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
         publish();
 
         // ---------------- layers 1 and 2
-        dense_layer<1, SH>(act, hbz1, bh1, tileX, tileH, sbase, s, accZ, accC, issuer, j, cbase, cr[1], h1,
-                           sync_wait, publish);
-        dense_layer<2, SH>(act, hbz2, bh2, tileX, tileH, sbase, s, accZ, accC, issuer, j, cbase, cr[2], h1,
-                           sync_wait, publish);
+        dense_layer<1, SH, true>(act, hbz1, bh1, tileX, tileH, sbase, s, accZ, accC, issuer, j, cbase, rg,
+                                 cr[1], h1, sync_wait, publish);
+        dense_layer<2, SH, true>(act, hbz2, bh2, tileX, tileH, sbase, s, accZ, accC, issuer, j, cbase, rg,
+                                 cr[2], h1, sync_wait, publish);
         // x3 (in h1) is read out while the next step's layer-0 MMAs run
         if (act) {
             rd_valid = true;
@@ -1030,8 +1065,11 @@ cudaError_t prepare_fwd_bf16() {
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64 && done[dev]) return cudaSuccess;
-    e = cudaFuncSetAttribute(fwd_bf16_kernel1, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(fwd_bf16_kernel1<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kSmemBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fwd_bf16_kernel1<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)kSmemBytes);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(fwd_bf16_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kSmemBytes);
@@ -1050,8 +1088,12 @@ cudaError_t launch_fwd_bf16(const FwdJobs &jobs, const void *packed_bf16, const 
     if (grid > max_jobs_ctas) grid = max_jobs_ctas;
     if (grid < 1) grid = 1;
     const uint8_t *pb = static_cast<const uint8_t *>(packed_bf16);
-    if (seqs_per_stream == 1)
-        fwd_bf16_kernel1<<<(int)grid, kThreads, kSmemBytes, stream>>>(jobs, pb, packed_f32, fl);
+    bool mid = false;  // some sequence starts in mid-chunk
+    for (int i = 0; i < jobs.n_groups; ++i) mid = mid || chunk_offset(jobs.g[i].N) > 0;
+    if (seqs_per_stream == 1 && mid)
+        fwd_bf16_kernel1<true><<<(int)grid, kThreads, kSmemBytes, stream>>>(jobs, pb, packed_f32, fl);
+    else if (seqs_per_stream == 1)
+        fwd_bf16_kernel1<false><<<(int)grid, kThreads, kSmemBytes, stream>>>(jobs, pb, packed_f32, fl);
     else
         fwd_bf16_kernel<2><<<(int)grid, kThreads, kSmemBytes, stream>>>(jobs, pb, packed_f32, fl);
     return cudaGetLastError();
