@@ -23,15 +23,18 @@
 // (128 rows x 64 BF16, 128-byte swizzle) and streamed through a ring of
 // slices by bulk copies, from L2, where every CTA's stream hits.
 //
-// Roles: H epilogue threads (thread j = hidden unit j: its tensor-memory lane
-// holds unit j's accumulators for all 128 columns), one producer thread (the
-// weight stream) and one MMA thread.  Per row step and layer:
+// Roles: 512 epilogue threads (a thread's tensor-memory lane holds one hidden
+// unit's accumulators for all 128 columns), one producer thread (the weight
+// stream), one MMA thread and one image warp (the h_V images: up to S H / 64
+// bulk copies per layer each way, two a lane; issued by single threads of the
+// MMA and epilogue roles they held up every other thread, 20 % of a row step
+// at 16 slots).  Per row step and layer:
 //   MMA  z, c (needs x, then h_V)  ->  epilogue: gates and scan, h -> smem
 //   MMA  y = D x + C h             ->  epilogue: GELU(y + residual) -> x
 // then the readout MMA and the masked 16-way softmax of every patch.
 // The next row's h_V is this row's h, path-reversed (consecutive rows run in
-// opposite directions); the scan writes it to global memory as a BF16 image
-// in the tile layout, and the next row bulk-copies it into the h tile.  In
+// opposite directions); the image warp writes it to global memory as a 16-bit
+// image in the tile layout, and the next row bulk-copies it into the h tile.  In
 // mode 0 these images are the row checkpoints that mode 1 (connected
 // configurations, resumed at the patch row of the first flipped spin) reads.
 #include <cuda_bf16.h>
@@ -71,7 +74,8 @@ __device__ __forceinline__ uint64_t kdesc(uint32_t addr) {
 }
 __device__ __forceinline__ uint64_t kstep(int kk) { return (uint64_t)((kk * 32) >> 4); }
 
-constexpr int kEpi = 512;  // epilogue threads: 512 / H per hidden unit
+constexpr int kEpi = 512;             // epilogue threads: 512 / H per hidden unit
+constexpr int kThreads2 = kEpi + 96;  // + producer, MMA and image warps
 
 struct Slot2 {
     int job;              // -1: needs a job, -2: none left (a launch holds < 2^31 jobs)
@@ -85,11 +89,13 @@ struct Slot2 {
 
 struct Misc2 {
     uint64_t full[kMaxRing], empty[kMaxRing];
-    uint64_t e2m[2], m2e[2], hv, imgw, go[2];  // e2m, m2e: per unit half
+    uint64_t e2m[2], m2e[2], go[2];  // e2m, m2e: per unit half
+    // image warp: a row step's slots are set, the h tile is written (MMA thread),
+    // its last reader is done (MMA commit), h_V has landed in it
+    uint64_t slots, hset, hfree, hv;
     uint32_t tmem_base;
     int abort_flag;
     int go_flag[2];
-    uint32_t hv_armed;                           // h_V image loads issued
     Slot2 slot[kMaxSlots];
 };
 
@@ -155,24 +161,18 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 // largest finite FP16 saturate to it) or BF16.
 template <bool F16>
 __device__ __forceinline__ uint16_t op_bits(float x) {
-    if (F16) return __half_as_ushort(__float2half_rn(fminf(fmaxf(x, -65504.0f), 65504.0f)));
-    const __nv_bfloat16 b = __float2bfloat16_rn(x);
-    return *reinterpret_cast<const uint16_t *>(&b);
+    uint16_t h;
+    if (F16) asm("cvt.rn.satfinite.f16.f32 %0, %1;" : "=h"(h) : "f"(x));
+    else asm("cvt.rn.bf16.f32 %0, %1;" : "=h"(h) : "f"(x));
+    return h;
 }
 template <bool F16>
 __device__ __forceinline__ uint32_t op_pack(float lo, float hi) {
     return (uint32_t)op_bits<F16>(lo) | ((uint32_t)op_bits<F16>(hi) << 16);
 }
 
-// 16 columns (two 8-column TMEM loads) of this thread's lane, columns beyond
-// `nc8` chunks left untouched.
-__device__ __forceinline__ void tmem_ld_cols16(uint32_t taddr, int nc8, uint32_t (&r)[16]) {
-    tmem_ld8(taddr, r[0], r[1], r[2], r[3], r[4], r[5], r[6], r[7]);
-    if (nc8 > 1) tmem_ld8(taddr + 8, r[8], r[9], r[10], r[11], r[12], r[13], r[14], r[15]);
-}
-
 template <int H, bool F16>
-__global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_constant__ Fwd2TcArgs A) {
+__global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_constant__ Fwd2TcArgs A) {
     constexpr int NH = H / 128;     // unit halves (M tiles)
     constexpr int KC = H / 64;      // K chunks of a hidden-size input
     constexpr int CG = kEpi / H;    // epilogue threads per unit (column groups)
@@ -223,9 +223,10 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
             mbar_init(smem_u32(&M.e2m[g]), 1);
             mbar_init(smem_u32(&M.m2e[g]), 1);
         }
-        M.hv_armed = 0;
+        mbar_init(smem_u32(&M.slots), 1);
+        mbar_init(smem_u32(&M.hset), 1);
+        mbar_init(smem_u32(&M.hfree), 1);
         mbar_init(smem_u32(&M.hv), 1);
-        mbar_init(smem_u32(&M.imgw), 1);
         mbar_init(smem_u32(&M.go[0]), 1);
         mbar_init(smem_u32(&M.go[1]), 1);
         M.abort_flag = 0;
@@ -248,7 +249,7 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
     if (tid == 0) mbar_arrive(smem_u32(&M.go[0]));  // row step 0 runs
     __syncthreads();
     const long long njobs = A.mode == 1 ? (long long)*A.n_jobs_dev : (long long)A.n_jobs;
-    const uint32_t hvb = smem_u32(&M.hv), imgw = smem_u32(&M.imgw);
+    const uint32_t hvb = smem_u32(&M.hv);
 
     if (warp == NW) {
         // ------------------------------------------------ producer: weight stream
@@ -283,15 +284,16 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
             if (*ab) set_status(A.status, PSR_ETIMEOUT);
         }
     } else if (warp == NW + 1) {
-        // ------------------------------------------------ MMA issue, h_V image stores
+        // ------------------------------------------------ MMA issue
         if (lane == 0 && !M.abort_flag) {
             // slices consumed; ring slot and the full barriers' phase; e2m and
             // h_V barrier phases
             uint32_t q = 0, slot = 0, fph = 0, pe0 = 0, pe1 = 0, ph = 0;
             const uint32_t e2m0 = smem_u32(&M.e2m[0]), e2m1 = smem_u32(&M.e2m[1]), m2e0 = smem_u32(&M.m2e[0]),
                            m2e1 = smem_u32(&M.m2e[1]);
-            const uint32_t ha = smem_u32(ht), fb = smem_u32(&M.full[0]), ebar = smem_u32(&M.empty[0]);
-            const uint64_t xd = kdesc(smem_u32(xt)), hd = kdesc(ha), rd = kdesc(smem_u32(ring));
+            const uint32_t hset = smem_u32(&M.hset), hfree = smem_u32(&M.hfree);
+            const uint32_t fb = smem_u32(&M.full[0]), ebar = smem_u32(&M.empty[0]);
+            const uint64_t xd = kdesc(smem_u32(xt)), hd = kdesc(smem_u32(ht)), rd = kdesc(smem_u32(ring));
             bool ok = true;
             for (uint32_t row = 0; ok; ++row) {
                 if (!wait_ab(smem_u32(&M.go[row & 1]), (row >> 1) & 1, ab)) {
@@ -304,9 +306,10 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
                     if (op & 0x00FF0000u) {
                         const uint32_t fl = (op >> 16) & 0xFFu;
                         if (fl & (kSchedC0 | kSchedC1)) {
-                            bulk_wait_read();  // the h tile may be overwritten once this commit lands
                             if (fl & kSchedC0) mma_commit(m2e0);
                             if (fl & kSchedC1) mma_commit(m2e1);
+                            // the layer's last MMAs on the h tile
+                            if (fl & kSchedWaitHv) mma_commit(hfree);
                         }
                         if (fl & kSchedW0) {
                             if (!wait_ab(e2m0, pe0, ab)) { ok = false; break; }
@@ -318,20 +321,7 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
                             pe1 ^= 1u;
                             tc_after();
                         }
-                        if (fl & kSchedStoreH) {
-                            // the scan has written h: it is the next row's h_V of layer l
-                            const int l = (int)((op >> 24) & 0xFu);
-                            for (int s = 0; s < S; ++s) {
-                                const Slot2 &st = M.slot[s];
-                                if (st.job < 0) continue;
-                                uint8_t *dst = img_dst(st, s, l);
-                                if (!dst) continue;
-                                for (int c = 0; c < KC; ++c)
-                                    bulk_s2g(dst + (size_t)c * W * 128, ha + c * 16384 + s * W * 128,
-                                             (uint32_t)W * 128u);
-                            }
-                            bulk_commit();
-                        }
+                        if (fl & kSchedStoreH) mbar_arrive(hset);
                         if (fl & kSchedWaitHv) {
                             if (!wait_ab(hvb, ph, ab)) { ok = false; break; }
                             ph ^= 1u;
@@ -354,13 +344,9 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
                     }
                 }
                 if (!ok) break;
-                // the row's image stores are complete before its successor reads them
-                bulk_wait_all();
-                mbar_arrive(imgw);
                 mma_commit(m2e0);  // logits of the row
                 if (NH == 2) mma_commit(m2e1);
             }
-            bulk_wait_all();
             // the MMAs of the last slices complete before the CTA may exit
             const uint32_t last = q < (uint32_t)R ? q : (uint32_t)R;
             for (uint32_t t = 0; t < last; ++t) {
@@ -372,6 +358,77 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
                 set_status(A.status, PSR_ETIMEOUT);
             }
         }
+    } else if (warp == NW + 2) {
+        // ------------------------------------------------ h_V images
+        // Lane pairs (slot, K chunk): loads of the row's h_V of each layer, then
+        // stores of the layer's h as the next row's h_V.
+        if (!M.abort_flag) {
+            static_assert(kMaxSlots * KC <= 64, "two (slot, K chunk) pairs a lane");
+            const uint32_t ha = smem_u32(ht), piece = (uint32_t)W * 128u;
+            uint32_t armed = 0, nh = 0, nf = 0;  // loads, hset and hfree phases so far
+            auto wait_w = [&](uint32_t bar, uint32_t parity) {
+                bool w = false;
+                if (lane == 0) w = wait_ab(bar, parity, ab);
+                w = __shfl_sync(0xffffffffu, w ? 1 : 0, 0) != 0;
+                __syncwarp();
+                return w;
+            };
+            for (uint32_t row = 0;; ++row) {
+                if (!wait_w(smem_u32(&M.go[row & 1]), (row >> 1) & 1)) break;
+                if (!*(volatile int *)&M.go_flag[row & 1]) break;
+                if (!wait_w(smem_u32(&M.slots), row & 1)) break;
+                const uint8_t *src[2] = {nullptr, nullptr};
+                uint8_t *dst[2] = {nullptr, nullptr};
+                uint32_t sstep[2] = {0, 0}, at[2] = {0, 0}, bytes = 0;
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    const int id = lane + 32 * k, s = id / KC, kc = id - s * KC;
+                    if (s >= S || M.slot[s].job < 0) continue;
+                    const Slot2 &st = M.slot[s];
+                    const size_t o = (size_t)kc * piece;
+                    src[k] = img_src(st, s, 0) + o;
+                    sstep[k] = (st.row == 0) ? 0u : img_bytes;  // one zero image for all layers
+                    dst[k] = img_dst(st, s, 0);
+                    if (dst[k]) dst[k] += o;
+                    at[k] = ha + (uint32_t)kc * 16384u + (uint32_t)s * piece;
+                    bytes += piece;
+                }
+                bytes = __reduce_add_sync(0xffffffffu, bytes);
+                auto load = [&](int l) {
+                    if (lane == 0) mbar_arrive_tx(hvb, bytes);
+                    ++armed;
+                    __syncwarp();
+#pragma unroll
+                    for (int k = 0; k < 2; ++k)
+                        if (src[k]) bulk_g2s(at[k], src[k] + (size_t)l * sstep[k], piece, hvb);
+                };
+                load(0);
+                bool ok = true;
+                for (int l = 0; l < nL && ok; ++l) {
+                    // the scan has written h: it is the next row's h_V of layer l
+                    ok = wait_w(smem_u32(&M.hset), nh++ & 1);
+                    if (!ok) break;
+#pragma unroll
+                    for (int k = 0; k < 2; ++k)
+                        if (dst[k]) bulk_s2g(dst[k] + (size_t)l * img_bytes, at[k], piece);
+                    bulk_commit();
+                    if (l + 1 < nL) {
+                        // h_V of layer l + 1 lands in the h tile once the stores and
+                        // the output map's MMAs have read it
+                        bulk_wait_read();
+                        ok = wait_w(smem_u32(&M.hfree), nf++ & 1);
+                        if (ok) load(l + 1);
+                    }
+                }
+                // the row's image stores are complete before its successor reads them
+                bulk_wait_all();
+                __syncwarp();
+                if (!ok) break;
+            }
+            bulk_wait_all();
+            // loads still in flight land before the CTA may exit
+            if (lane == 0 && armed > 0 && !mbar_wait(hvb, (armed - 1) & 1)) set_status(A.status, PSR_ETIMEOUT);
+        }
     } else {
         // ------------------------------------------------ epilogue
         // warp w reads tensor-memory lanes 32 (w & 3) ..; warpgroup w >> 2
@@ -382,17 +439,15 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
         const uint32_t tz = tmem + lane_off + 128u * g;          // z, then y
         const uint32_t tcc = tmem + lane_off + 128u * (NH + g);  // c
         const uint32_t tlg = tmem + lane_off + 128u * NH;        // logits (lanes 32 q4 + 0..15)
-        // unit j's place in a K-major tile row
-        const uint32_t kreg = (uint32_t)(j >> 6) * 16384u;
-        const int ch = (j & 63) >> 3;
-        const uint32_t eb = (uint32_t)(j & 7) * 2u;
-        // unit j's element of tile row nb + k, nb a multiple of 8 (so the
-        // 16-byte chunk's swizzle phase is k & 7)
-        const uint32_t eoff = kreg + eb, sw = (uint32_t)ch << 4;
-        auto tile_st = [&](uint8_t *tile, int nb, int k, uint16_t v) {
-            *reinterpret_cast<uint16_t *>(tile + eoff + (uint32_t)nb * 128u + (sw ^ ((uint32_t)(k & 7) << 4)) +
-                                          (uint32_t)k * 128u) = v;
-        };
+        // unit j's element of row k (mod 8) of a K-major tile, 128-byte swizzle
+        // (16-byte group c of row k at c ^ (k & 7)); rows n .. n + 7 of a tile, n a
+        // multiple of 8, are at tile + 128 n + koff[0 .. 7]
+        uint32_t koff[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            koff[k] = (uint32_t)(j >> 6) * 16384u + 128u * k + ((uint32_t)(((j & 63) >> 3) ^ k) << 4) + (uint32_t)(j & 7) * 2u;
+        const uint32_t hta = smem_u32(ht), xta = smem_u32(xt);
+        auto st16 = [&](uint32_t a, uint16_t v) { asm volatile("st.shared.b16 [%0], %1;" ::"r"(a), "h"(v)); };
         float *res = A.res + (size_t)blockIdx.x * 2 * kCols * H;
         uint32_t pm = 0;  // m2e phase of this thread's unit half
         bool ok = !M.abort_flag;
@@ -401,22 +456,6 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
         const uint32_t hbar = 2u + (uint32_t)g, hcount = (uint32_t)(kEpi / NH);
         const bool leader = tid == 128 * g;
 
-        // thread 0: bulk copies of every active slot's h_V image of layer l
-        auto issue_hv = [&](int l) {
-            uint32_t bytes = 0;
-            for (int s = 0; s < S; ++s)
-                if (M.slot[s].job >= 0) bytes += img_bytes;
-            mbar_arrive_tx(hvb, bytes);
-            for (int s = 0; s < S; ++s) {
-                const Slot2 &st = M.slot[s];
-                if (st.job < 0) continue;
-                const uint8_t *src = img_src(st, s, l);
-                for (int kc = 0; kc < KC; ++kc)
-                    bulk_g2s(smem_u32(ht + kc * 16384 + s * W * 128), src + (size_t)kc * W * 128, (uint32_t)W * 128u,
-                             hvb);
-            }
-            ++M.hv_armed;
-        };
         // One thread polls the MMA thread's barrier and a named barrier
         // releases the others (hundreds of pollers would contend for the
         // shared memory the tensor core reads its operands from); the
@@ -438,6 +477,44 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
             tc_before();
             named_bar(hbar, hcount);
             if (leader) mbar_arrive(e2m);
+        };
+        // Runs go(v, s, cc, n) for the 8-column chunks (columns n .. n + 7, chunk cc
+        // in path order of slot s) of this thread's active slots, with the next
+        // chunk's loads ld(v, n) in flight: a chunk's loads, gates and serial scan
+        // are a chain of latencies that four warps per scheduler do not cover.
+        // Columns past P_x are computed like the others: a column's values reach
+        // no other column but through the scan, which starts after them.
+        auto chunks = [&](auto &&ld, auto &&go) {
+            auto next = [&](int &s, int &cc) {
+                if (++cc == nch) {
+                    cc = 0;
+                    s += CG;
+                    while (s < S && M.slot[s].job < 0) s += CG;
+                }
+                return s < S;
+            };
+            auto col = [&](int s, int cc) { return s * W + 8 * ((M.slot[s].row & 1) ? nch - 1 - cc : cc); };
+            auto wait = [&](uint32_t(&v)[16]) { asm volatile("tcgen05.wait::ld.sync.aligned;" : PSR_P16(v, 0)::"memory"); };
+            uint32_t va[16], vb[16];
+            int s = cg - CG, cc = nch - 1;
+            bool more = next(s, cc);
+            if (more) ld(va, col(s, cc));
+            while (more) {
+                int s2 = s, c2 = cc;
+                more = next(s2, c2);
+                wait(va);
+                if (more) ld(vb, col(s2, c2));
+                go(va, s, cc, col(s, cc));
+                if (!more) break;
+                s = s2;
+                cc = c2;
+                more = next(s2, c2);
+                wait(vb);
+                if (more) ld(va, col(s2, c2));
+                go(vb, s, cc, col(s, cc));
+                s = s2;
+                cc = c2;
+            }
         };
         // the previous row's readout sums into the job's total (fixed order),
         // and the job's log psi after its last row (slot s, its warp)
@@ -530,13 +607,7 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
                 if (!more) more = (long long)atomicAdd(A.job_counter, 0ull) < njobs;
                 M.go_flag[(row_it + 1) & 1] = more ? 1 : 0;
                 mbar_arrive(smem_u32(&M.go[(row_it + 1) & 1]));
-                // the previous row's image stores are complete
-                if (row_it > 0 && !wait_ab(imgw, (row_it - 1) & 1, ab)) {
-                    ok = false;
-                    M.abort_flag = 1;
-                    set_status(A.status, PSR_ETIMEOUT);
-                }
-                if (ok) issue_hv(0);
+                mbar_arrive(smem_u32(&M.slots));
             }
             // ---- layer-0 input: one-hot (v_H, v_V) of every column, K chunk 0
             {
@@ -575,92 +646,75 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
                     const float2 hbz2 = make_float2(hbz, hbz), bh2 = make_float2(bh, bh);
                     const bool keep_res = (l >= 1) && (l + 1 < nL);
                     float *resw = res + (size_t)(l & 1) * kCols * H;
-                    for (int s = cg; s < S; s += CG) {
-                        const Slot2 &st = M.slot[s];
-                        if (st.job < 0) continue;
-                        const int n0 = s * W;
-                        const bool odd = st.row & 1;
-                        float h = 0.0f;  // the row starts from h_H = 0
-                        // two 16-column halves, in path order
-                        for (int hh = 0; hh < 2; ++hh) {
-                            const int half = odd ? 1 - hh : hh;
-                            const int c0 = 16 * half;
-                            if (c0 >= Px) continue;
-                            const int nc8 = nch - 2 * half;
-                            uint32_t zr[16], cr[16];
-                            tmem_ld_cols16(tz + n0 + c0, nc8, zr);
-                            tmem_ld_cols16(tcc + n0 + c0, nc8, cr);
-                            tmem_wait_ld16x2(zr, cr);
-                            float av[16], bv[16];
+                    float h = 0.0f;
+                    chunks(
+                        [&](uint32_t(&v)[16], int n) {
+                            tmem_ld8(tz + n, v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]);
+                            tmem_ld8(tcc + n, v[8], v[9], v[10], v[11], v[12], v[13], v[14], v[15]);
+                        },
+                        [&](uint32_t(&v)[16], int s, int cc, int n) {
+                            float av[8], bv[8];
 #pragma unroll
-                            for (int k = 0; k < 16; k += 2) {
+                            for (int k = 0; k < 8; k += 2) {
                                 float2 a2, b2;
-                                gates2(make_float2(__uint_as_float(zr[k]), __uint_as_float(zr[k + 1])),
-                                       make_float2(__uint_as_float(cr[k]), __uint_as_float(cr[k + 1])), hbz2, bh2, a2,
+                                gates2(make_float2(__uint_as_float(v[k]), __uint_as_float(v[k + 1])),
+                                       make_float2(__uint_as_float(v[8 + k]), __uint_as_float(v[9 + k])), hbz2, bh2, a2,
                                        b2);
                                 av[k] = a2.x;
                                 av[k + 1] = a2.y;
                                 bv[k] = b2.x;
                                 bv[k + 1] = b2.y;
                             }
-                            if (!odd) {
+                            if (cc == 0) h = 0.0f;  // the row starts from h_H = 0
+                            const uint32_t a = hta + 128u * n;
+                            if (M.slot[s].row & 1) {
+                                const int k0 = Px - 1 - (n - s * W);  // the path's first column, if in this chunk
 #pragma unroll
-                                for (int k = 0; k < 16; ++k) {
-                                    if (c0 + k < Px) {
-                                        h = fmaf(av[k], h, bv[k]);
-                                        tile_st(ht, n0 + c0, k, op_bits<F16>(h));
-                                        if (keep_res) resw[(size_t)(n0 + c0 + k) * H + j] = h;
-                                    }
+                                for (int k = 7; k >= 0; --k) {
+                                    if (k == k0) h = 0.0f;
+                                    h = fmaf(av[k], h, bv[k]);
+                                    bv[k] = h;
+                                    st16(a + koff[k], op_bits<F16>(h));
                                 }
                             } else {
 #pragma unroll
-                                for (int k = 15; k >= 0; --k) {
-                                    if (c0 + k < Px) {
-                                        h = fmaf(av[k], h, bv[k]);
-                                        tile_st(ht, n0 + c0, k, op_bits<F16>(h));
-                                        if (keep_res) resw[(size_t)(n0 + c0 + k) * H + j] = h;
-                                    }
+                                for (int k = 0; k < 8; ++k) {
+                                    h = fmaf(av[k], h, bv[k]);
+                                    bv[k] = h;
+                                    st16(a + koff[k], op_bits<F16>(h));
                                 }
                             }
-                        }
-                    }
+                            if (keep_res) {
+#pragma unroll
+                                for (int k = 0; k < 8; ++k) resw[(size_t)(n + k) * H + j] = bv[k];
+                            }
+                        });
                 }
                 arrive_e2m();
 
                 // ---- output map: x = GELU(y + residual)
                 wait_m2e();
-                // the last half's output map is committed: every MMA reading
-                // the h tile is complete, the next layer's h_V may land in it
-                if (leader && g == NH - 1 && l + 1 < nL && ok) issue_hv(l + 1);
                 {
                     const bool use_res = (l >= 2);
                     const float *resr = res + (size_t)((l - 1) & 1) * kCols * H;
-                    for (int s = cg; s < S; s += CG) {
-                        const Slot2 &st = M.slot[s];
-                        if (st.job < 0) continue;
-                        const int n0 = s * W;
-                        for (int half = 0; half < 2; ++half) {
-                            const int c0 = 16 * half;
-                            if (c0 >= Px) continue;
-                            uint32_t yr[16];
-                            tmem_ld_cols16(tz + n0 + c0, nch - 2 * half, yr);
-                            float rv[16];
+                    chunks(
+                        [&](uint32_t(&v)[16], int n) {
+                            tmem_ld8(tz + n, v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7]);
 #pragma unroll
-                            for (int k = 0; k < 16; ++k)
-                                rv[k] = (use_res && c0 + k < Px) ? resr[(size_t)(n0 + c0 + k) * H + j] : 0.0f;
-                            asm volatile("tcgen05.wait::ld.sync.aligned;" : PSR_P16(yr, 0)::"memory");
+                            for (int k = 0; k < 8; ++k)
+                                v[8 + k] = use_res ? __float_as_uint(resr[(size_t)(n + k) * H + j]) : 0u;
+                        },
+                        [&](uint32_t(&v)[16], int, int, int n) {
+                            const uint32_t a = xta + 128u * n;
 #pragma unroll
-                            for (int k = 0; k < 16; k += 2) {
-                                if (c0 + k < Px) {
-                                    const float2 x = gelu_bf16out2(make_float2(__uint_as_float(yr[k]) + rv[k],
-                                                                               __uint_as_float(yr[k + 1]) + rv[k + 1]));
-                                    tile_st(xt, n0 + c0, k, op_bits<F16>(x.x));
-                                    if (c0 + k + 1 < Px)
-                                        tile_st(xt, n0 + c0, k + 1, op_bits<F16>(x.y));
-                                }
+                            for (int k = 0; k < 8; k += 2) {
+                                const float2 x = gelu_bf16out2(
+                                    __fadd2_rn(make_float2(__uint_as_float(v[k]), __uint_as_float(v[k + 1])),
+                                               make_float2(__uint_as_float(v[8 + k]), __uint_as_float(v[9 + k]))));
+                                st16(a + koff[k], op_bits<F16>(x.x));
+                                st16(a + koff[k + 1], op_bits<F16>(x.y));
                             }
-                        }
-                    }
+                        });
                 }
                 arrive_e2m();
             }
@@ -699,29 +753,39 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
                     asm volatile("tcgen05.wait::ld.sync.aligned;"
                                  : "+r"(lr[0]), "+r"(lr[1]), "+r"(lr[2]), "+r"(lr[3]), "+r"(lr[4]), "+r"(lr[5]),
                                    "+r"(lr[6]), "+r"(lr[7])::"memory");
+                    // the eight columns side by side (a column's two reductions are a
+                    // chain of eight shuffles); columns past P_x are not summed
+                    float lg[8], m[8], ex[8];
+                    uint32_t allowed = 0;  // bit e: this lane's value in column e
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int i = i0 + e, k = odd ? Px - 1 - i : i;
+                        const int up = st.n_up + __shfl_sync(0xffffffffu, upx, k);
+                        const int down = 2 * r * Lx + 4 * k - up;
+                        if (!A.u1 || (up + pc_lane <= N / 2 && down + 4 - pc_lane <= N / 2)) allowed |= 1u << e;
+                        lg[e] = __uint_as_float(lr[e]) + bo;
+                        m[e] = (allowed >> e) & 1u ? lg[e] : -INFINITY;
+                    }
+#pragma unroll
+                    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) m[e] = fmaxf(m[e], __shfl_xor_sync(0xffffffffu, m[e], o, 16));
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) ex[e] = (allowed >> e) & 1u ? __expf(lg[e] - m[e]) : 0.0f;
+#pragma unroll
+                    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) ex[e] += __shfl_xor_sync(0xffffffffu, ex[e], o, 16);
                     float rsum = 0.0f;
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
-                        const int i = i0 + e;
-                        if (i >= Px) break;
-                        const int k = odd ? Px - 1 - i : i, v = st.v[i];
-                        const int up = st.n_up + __shfl_sync(0xffffffffu, upx, k);
-                        const int down = 2 * r * Lx + 4 * k - up;
-                        const bool allowed = !A.u1 || (up + pc_lane <= N / 2 && down + 4 - pc_lane <= N / 2);
-                        const float lg = __uint_as_float(lr[e]) + bo;
-                        float m = allowed ? lg : -INFINITY;
-#pragma unroll
-                        for (int o = 8; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o, 16));
-                        float ex = allowed ? __expf(lg - m) : 0.0f;
-#pragma unroll
-                        for (int o = 8; o > 0; o >>= 1) ex += __shfl_xor_sync(0xffffffffu, ex, o, 16);
-                        float lp = allowed ? lg - m - __logf(ex) : -INFINITY;
-                        lp = __shfl_sync(0xffffffffu, lp, v);
+                        const int i = i0 + e, k = odd ? Px - 1 - i : i;
+                        float lp = (allowed >> e) & 1u ? lg[e] - m[e] - __logf(ex[e]) : -INFINITY;
+                        lp = __shfl_sync(0xffffffffu, lp, st.v[i]);
                         const float rf = __shfl_sync(0xffffffffu, ref, e);
-                        float d = lp;
-                        if (A.mode == 1) d = lp - rf;
-                        else if (A.logp_out && lane == 0) A.logp_out[(size_t)st.sample * Np + r * Px + k] = lp;
-                        rsum += d;
+                        if (i >= Px) continue;
+                        if (A.mode != 1 && A.logp_out && lane == 0) A.logp_out[(size_t)st.sample * Np + r * Px + k] = lp;
+                        rsum += A.mode == 1 ? lp - rf : lp;
                     }
                     if (lane == 0) st.part[c8] = rsum;
                 }
@@ -740,7 +804,6 @@ __global__ void __launch_bounds__(kEpi + 64, 1) fwd2d_tc_kernel(const __grid_con
             M.abort_flag = 1;
             set_status(A.status, PSR_ETIMEOUT);
         }
-        if (tid == 0 && M.hv_armed > 0 && !mbar_wait(hvb, (M.hv_armed - 1) & 1)) set_status(A.status, PSR_ETIMEOUT);
     }
     tc_before();
     __syncthreads();
@@ -761,7 +824,7 @@ cudaError_t launch_h(const Fwd2TcArgs &a, int grid, cudaStream_t stream) {
     cudaError_t e =
         cudaFuncSetAttribute(fwd2d_tc_kernel<H, F16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    fwd2d_tc_kernel<H, F16><<<grid, kEpi + 64, smem, stream>>>(a);
+    fwd2d_tc_kernel<H, F16><<<grid, kThreads2, smem, stream>>>(a);
     return cudaGetLastError();
 }
 
