@@ -285,67 +285,112 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
         }
     } else if (warp == NW + 1) {
         // ------------------------------------------------ MMA issue
-        if (lane == 0 && !M.abort_flag) {
+        if (!M.abort_flag) {
+            // Issuing a slice's four MMAs (256 cycles of the tensor core) must not
+            // take longer than they do.  So the order of the slices
+            // (fwd2d_tc_schedule) is in loops, and the whole warp walks them with
+            // every value uniform, electing a lane for the MMAs and commits only:
+            // descriptors then stay in uniform registers, where the MMA takes them.
+            // E_loc of the 16 x 16 model: 9.31 ms with one thread reading a list of
+            // operations from the kernel's parameters (730 cycles a slice), 8.60 with
+            // one thread in loops, 7.79 so.
+            auto wait_u = [&](uint32_t bar, uint32_t parity) {
+                return __all_sync(0xffffffffu, wait_ab(bar, parity, ab)) != 0;
+            };
             // slices consumed; ring slot and the full barriers' phase; e2m and
             // h_V barrier phases
-            uint32_t q = 0, slot = 0, fph = 0, pe0 = 0, pe1 = 0, ph = 0;
-            const uint32_t e2m0 = smem_u32(&M.e2m[0]), e2m1 = smem_u32(&M.e2m[1]), m2e0 = smem_u32(&M.m2e[0]),
-                           m2e1 = smem_u32(&M.m2e[1]);
+            uint32_t q = 0, slot = 0, fph = 0, pe = 0, ph = 0;
+            const uint32_t e2m = smem_u32(&M.e2m[0]), m2e = smem_u32(&M.m2e[0]);
             const uint32_t hset = smem_u32(&M.hset), hfree = smem_u32(&M.hfree);
             const uint32_t fb = smem_u32(&M.full[0]), ebar = smem_u32(&M.empty[0]);
             const uint64_t xd = kdesc(smem_u32(xt)), hd = kdesc(smem_u32(ht)), rd = kdesc(smem_u32(ring));
+            constexpr int HL = NH - 1;  // last unit half
             bool ok = true;
-            for (uint32_t row = 0; ok; ++row) {
-                if (!wait_ab(smem_u32(&M.go[row & 1]), (row >> 1) & 1, ab)) {
-                    ok = false;
-                    break;
-                }
-                if (!*(volatile int *)&M.go_flag[row & 1]) break;
-                for (int i = 0; i < A.n_slices; ++i, ++q) {
-                    const uint32_t op = A.sched.op[i];
-                    if (op & 0x00FF0000u) {
-                        const uint32_t fl = (op >> 16) & 0xFFu;
-                        if (fl & (kSchedC0 | kSchedC1)) {
-                            if (fl & kSchedC0) mma_commit(m2e0);
-                            if (fl & kSchedC1) mma_commit(m2e1);
-                            // the layer's last MMAs on the h tile
-                            if (fl & kSchedWaitHv) mma_commit(hfree);
-                        }
-                        if (fl & kSchedW0) {
-                            if (!wait_ab(e2m0, pe0, ab)) { ok = false; break; }
-                            pe0 ^= 1u;
-                            tc_after();
-                        }
-                        if (fl & kSchedW1) {
-                            if (!wait_ab(e2m1, pe1, ab)) { ok = false; break; }
-                            pe1 ^= 1u;
-                            tc_after();
-                        }
-                        if (fl & kSchedStoreH) mbar_arrive(hset);
-                        if (fl & kSchedWaitHv) {
-                            if (!wait_ab(hvb, ph, ab)) { ok = false; break; }
-                            ph ^= 1u;
-                            tc_after();
-                        }
-                    }
+            // the next nk slices: accumulator columns d, K chunks of tile b, added to
+            // the accumulator from the first K step if acc
+            auto run = [&](uint32_t d, uint64_t b, int nk, uint32_t acc) {
+#pragma unroll 1
+                for (int kc = 0; kc < nk && ok; ++kc) {
                     // the weight slice has landed (bulk-copy transactions)
-                    if (!wait_ab(fb + 8 * slot, fph, ab)) { ok = false; break; }
+                    if (!wait_u(fb + 8 * slot, fph)) { ok = false; break; }
                     const uint64_t ad = rd + (uint64_t)(slot * (kSlice >> 4));
-                    const uint64_t bd = ((op & (1u << 10)) ? hd : xd) + (uint64_t)(((op >> 12) & 3u) * (16384u >> 4));
-                    const uint32_t d = tmem + (op & 0x3FFu);
-                    mma_ss<idesc2<F16>()>(d, ad, bd, (op >> 11) & 1u);
-                    mma_ss<idesc2<F16>()>(d, ad + kstep(1), bd + kstep(1), 1u);
-                    mma_ss<idesc2<F16>()>(d, ad + kstep(2), bd + kstep(2), 1u);
-                    mma_ss<idesc2<F16>()>(d, ad + kstep(3), bd + kstep(3), 1u);
-                    mma_commit(ebar + 8 * slot);
+                    if (elect1()) {
+                        mma_ss<idesc2<F16>()>(d, ad, b, acc);
+                        mma_ss<idesc2<F16>()>(d, ad + kstep(1), b + kstep(1), 1u);
+                        mma_ss<idesc2<F16>()>(d, ad + kstep(2), b + kstep(2), 1u);
+                        mma_ss<idesc2<F16>()>(d, ad + kstep(3), b + kstep(3), 1u);
+                        mma_commit(ebar + 8 * slot);
+                    }
+                    __syncwarp();
+                    acc = 1u;
+                    b += 16384u >> 4;
+                    ++q;
                     if (++slot == (uint32_t)R) {
                         slot = 0;
                         fph ^= 1u;
                     }
                 }
-                if (!ok) break;
-                mma_commit(m2e0);  // logits of the row
-                if (NH == 2) mma_commit(m2e1);
+            };
+            // half g's epilogue has arrived
+            auto wait_e = [&](int g) {
+                ok = ok && wait_u(e2m + 8 * g, (pe >> g) & 1u);
+                pe ^= 1u << g;
+                tc_after();
+            };
+            auto commit = [&](int g) {
+                if (ok && elect1()) mma_commit(m2e + 8 * g);
+                __syncwarp();
+            };
+            for (uint32_t row = 0; ok; ++row) {
+                if (!wait_u(smem_u32(&M.go[row & 1]), (row >> 1) & 1)) {
+                    ok = false;
+                    break;
+                }
+                if (!*(volatile int *)&M.go_flag[row & 1]) break;
+#pragma unroll 1
+                for (int l = 0; l < nL && ok; ++l) {
+                    const int kin = l == 0 ? 1 : KC;
+                    // W_hv h_V needs only the h_V image of the layer: above layer 0 it
+                    // runs while the epilogue computes the layer input
+                    if (l > 0) {
+                        commit(HL);         // the last half's output map of layer l - 1
+                        if (elect1()) mma_commit(hfree);  // and the last MMAs on the h tile
+                    }
+                    ok = ok && wait_u(hvb, ph);
+                    ph ^= 1u;
+                    tc_after();
+#pragma unroll 1
+                    for (int g = 0; g < NH; ++g) run(tmem + 128u * (NH + g), hd, KC, 0u);
+                    // W_z x, W_hx x once x is complete; half g's projections are
+                    // committed (its scan may start) before half g + 1's are issued
+                    for (int g = 0; g < NH; ++g) wait_e(g);
+#pragma unroll 1
+                    for (int g = 0; g < NH; ++g) {
+                        if (g > 0) commit(g - 1);
+                        run(tmem + 128u * g, xd, kin, 0u);
+                        run(tmem + 128u * (NH + g), xd, kin, 1u);
+                    }
+                    commit(HL);
+                    // D x of half g once half g's scan has consumed z; C h once every
+                    // half's scan has written h (then h is also stored as the next
+                    // row's h_V); half g's output map committed before half g + 1's C
+#pragma unroll 1
+                    for (int g = 0; g < NH; ++g) {
+                        wait_e(g);
+                        if (g == HL && ok && lane == 0) mbar_arrive(hset);
+                        run(tmem + 128u * g, xd, kin, 0u);
+                    }
+#pragma unroll 1
+                    for (int g = 0; g < NH; ++g) {
+                        if (g > 0) commit(g - 1);
+                        run(tmem + 128u * g, hd, KC, 1u);
+                    }
+                }
+                // readout once both halves' layer input of the readout (x) is complete
+                commit(HL);
+                for (int g = 0; g < NH; ++g) wait_e(g);
+                run(tmem + 128u * NH, xd, KC, 0u);
+                for (int g = 0; g < NH; ++g) commit(g);  // logits of the row
             }
             // the MMAs of the last slices complete before the CTA may exit
             const uint32_t last = q < (uint32_t)R ? q : (uint32_t)R;
@@ -353,7 +398,7 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
                 const uint32_t qq = q - 1 - t;
                 if (!mbar_wait(smem_u32(&M.empty[qq % R]), (qq / R) & 1)) set_status(A.status, PSR_ETIMEOUT);
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 M.abort_flag = 1;
                 set_status(A.status, PSR_ETIMEOUT);
             }
@@ -869,71 +914,30 @@ __global__ void pack2d_tc_kernel(const float *__restrict__ theta, T2Layout tl, S
 
 }  // namespace
 
-// Slices of one row step, in the order the MMA thread consumes them, with
-// the synchronisation each needs first.
+// Slices of one row step, in the order the MMA thread consumes them.
 Sched2 fwd2d_tc_schedule(int nL, int H) {
     Sched2 sc{};
     const int NH = H / 128, KC = H / 64;
     int n = 0;
-    auto add = [&](int ty, int l, int g, int kc, int fl) {
-        sc.type[n] = (uint8_t)ty;
-        sc.l[n] = (uint8_t)l;
-        sc.g[n] = (uint8_t)g;
-        sc.kc[n] = (uint8_t)kc;
-        sc.flags[n] = (uint8_t)fl;
-        // accumulator column (z / y of half g: 128 g; c: 128 (NH + g); logits:
-        // 128 NH), B tile, accumulate flag
-        uint32_t dcol = 0, from_h = 0, acc = 0;
-        switch (ty) {
-            case kMtWz: dcol = 128u * g; acc = kc > 0; break;
-            case kMtWhx: dcol = 128u * (NH + g); acc = 1; break;
-            case kMtWhv: dcol = 128u * (NH + g); from_h = 1; acc = kc > 0; break;
-            case kMtD: dcol = 128u * g; acc = kc > 0; break;
-            case kMtC: dcol = 128u * g; from_h = 1; acc = 1; break;
-            default: dcol = 128u * NH; acc = kc > 0; break;
+    auto add = [&](int ty, int l, int g, int nk) {
+        for (int kc = 0; kc < nk; ++kc, ++n) {
+            sc.type[n] = (uint8_t)ty;
+            sc.l[n] = (uint8_t)l;
+            sc.g[n] = (uint8_t)g;
+            sc.kc[n] = (uint8_t)kc;
         }
-        sc.op[n] = dcol | (from_h << 10) | (acc << 11) | ((uint32_t)kc << 12) | ((uint32_t)fl << 16) |
-                   ((uint32_t)l << 24);
-        ++n;
     };
-    const int HL = NH - 1;                                       // last unit half
-    const int kC[2] = {kSchedC0, kSchedC1}, kW[2] = {kSchedW0, kSchedW1};
-    const int wall = NH == 2 ? (kSchedW0 | kSchedW1) : kSchedW0;  // both halves' epilogues
     for (int l = 0; l < nL; ++l) {
         const int kin = l == 0 ? 1 : KC;
-        // W_hv h_V needs only the h_V image of the layer: above layer 0 it
-        // runs while the epilogue computes the layer input (after the last
-        // half's output map of layer l - 1 has been committed)
-        for (int g = 0; g < NH; ++g)
-            for (int kc = 0; kc < KC; ++kc) {
-                int fl = 0;
-                if (g == 0 && kc == 0) fl = kSchedWaitHv | (l > 0 ? kC[HL] : 0);
-                add(kMtWhv, l, g, kc, fl);
-            }
-        // W_z x, W_hx x once x is complete; half g's projections are
-        // committed (its scan may start) before half g + 1's are issued
+        for (int g = 0; g < NH; ++g) add(kMtWhv, l, g, KC);
         for (int g = 0; g < NH; ++g) {
-            for (int kc = 0; kc < kin; ++kc) {
-                int fl = 0;
-                if (kc == 0) fl = (g == 0) ? wall : kC[g - 1];
-                add(kMtWz, l, g, kc, fl);
-            }
-            for (int kc = 0; kc < kin; ++kc) add(kMtWhx, l, g, kc, 0);
+            add(kMtWz, l, g, kin);
+            add(kMtWhx, l, g, kin);
         }
-        // D x of half g once half g's scan has consumed z; C h once every
-        // half's scan has written h (then h is also stored as the next row's
-        // h_V); half g's output map committed before half g + 1's C
-        for (int g = 0; g < NH; ++g)
-            for (int kc = 0; kc < kin; ++kc) {
-                int fl = 0;
-                if (kc == 0) fl = (g == 0 ? kC[HL] : 0) | kW[g] | (g == HL ? kSchedStoreH : 0);
-                add(kMtD, l, g, kc, fl);
-            }
-        for (int g = 0; g < NH; ++g)
-            for (int kc = 0; kc < KC; ++kc) add(kMtC, l, g, kc, (kc == 0 && g > 0) ? kC[g - 1] : 0);
+        for (int g = 0; g < NH; ++g) add(kMtD, l, g, kin);
+        for (int g = 0; g < NH; ++g) add(kMtC, l, g, KC);
     }
-    // readout once both halves' layer input of the readout (x) is complete
-    for (int kc = 0; kc < KC; ++kc) add(kMtWo, 0, 0, kc, kc == 0 ? (kC[HL] | wall) : 0);
+    add(kMtWo, 0, 0, KC);
     sc.n = n;
     return sc;
 }
@@ -988,8 +992,7 @@ cudaError_t launch_fwd2d_tc(Fwd2TcArgs a, int grid, cudaStream_t stream) {
     if (e != cudaSuccess) return e;
     const int H = a.tl.H;
     fwd2d_tc_geometry(a.Lx, &a.W, &a.S);
-    a.sched = fwd2d_tc_schedule(a.tl.nL, H);
-    a.n_slices = a.sched.n;
+    a.n_slices = fwd2d_tc_schedule(a.tl.nL, H).n;
     const size_t base = (H == 256) ? fwd2d_tc_smem<256>(0) : fwd2d_tc_smem<128>(0);
     if ((size_t)optin < base + 2 * kSlice) return cudaErrorInvalidConfiguration;
     int R = (int)(((size_t)optin - base) / kSlice);

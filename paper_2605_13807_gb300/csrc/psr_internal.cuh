@@ -218,20 +218,12 @@ T2Layout t2_layout(int nL, int H);
 // FP16 or BF16 operands, FP32 accumulation, gates, scan, GELU and softmax; hidden
 // 128 or 256, Lx <= 64.  The weights are streamed as 16 KB slices in MMA
 // order (launch_pack2d_tc writes them); Sched2 lists, per slice, the matrix,
-// layer, unit half, K chunk and the synchronisation before it.
+// layer, unit half and K chunk.
 enum { kMtWz = 0, kMtWhx = 1, kMtWhv = 2, kMtC = 3, kMtD = 4, kMtWo = 5 };
-// Synchronisation before a slice, in this order: commit the MMAs so far to
-// unit half 0's / 1's epilogue, wait for half 0's / 1's epilogue, store the
-// h tile as the next row's h_V images, wait for the h_V image of the layer.
-enum { kSchedC0 = 1, kSchedC1 = 2, kSchedW0 = 4, kSchedW1 = 8, kSchedStoreH = 16, kSchedWaitHv = 32 };
 constexpr int kSchedMax = 320;
-// op[i], what the MMA thread needs of slice i: bits 0-9 accumulator column,
-// bit 10 B operand from the h tile (else x), bit 11 accumulate from the
-// first K step, bits 12-13 K chunk, bits 16-23 flags, bits 24-27 layer.
 struct Sched2 {
     int n;
-    uint8_t type[kSchedMax], l[kSchedMax], g[kSchedMax], kc[kSchedMax], flags[kSchedMax];
-    uint32_t op[kSchedMax];
+    uint8_t type[kSchedMax], l[kSchedMax], g[kSchedMax], kc[kSchedMax];
 };
 Sched2 fwd2d_tc_schedule(int nL, int H);
 // Jobs as in Fwd2Group; the row checkpoints are 16-bit h_V images:
@@ -260,7 +252,6 @@ struct Fwd2TcArgs {
     int *status;
     // set by launch_fwd2d_tc
     int W, S, R, n_slices;
-    Sched2 sched;
 };
 bool fwd2d_tc_supported(int nL, int H, int Lx);
 void fwd2d_tc_geometry(int Lx, int *W, int *S);

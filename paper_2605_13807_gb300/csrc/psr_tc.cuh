@@ -103,6 +103,18 @@ __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint3
         : "memory");
 }
 
+// True in one lane of a full warp, always the same one.  MMAs and commits are
+// issued under elect1() by a warp that reaches them with warp-uniform values
+// (loop counters, kernel parameters, a warp index broadcast by a shuffle), not
+// by a branch on a thread's own index: the descriptors then live in uniform
+// registers, where the instruction wants them, and an MMA is issued in about the
+// time the tensor core takes for it instead of twice that.
+__device__ __forceinline__ bool elect1() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 template <uint32_t IDESC>
 __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t acc) {
     asm volatile(
