@@ -221,6 +221,8 @@ __device__ __forceinline__ uint64_t boff(int kk) { return (uint64_t)((kk * 16 * 
 
 template <int WHAT, class SH>
 __device__ __forceinline__ void issue(int s, uint32_t sbase) {
+    __syncwarp();
+    if (!elect1()) return;
     constexpr uint32_t ID = SH::kIdesc;
     const uint32_t tX = sbase + OFF_TILES + (uint32_t)(2 * s) * SH::kTileBytes;
     const uint64_t bX = bdesc<SH>(tX), bH = bdesc<SH>(tX + SH::kTileBytes);
@@ -288,9 +290,9 @@ __device__ __forceinline__ void gates_scan16(const uint32_t (&rz)[16], const uin
 template <int L, class SH, bool kOff, class WaitF, class PubF>
 __device__ __forceinline__ void dense_layer(bool act, float hbz, float bh, uint8_t *tileX, uint8_t *tileH,
                                             uint32_t sbase, int s, uint32_t accZ, uint32_t accC,
-                                            bool issuer, int j, int cbase, int rg, float &carry,
+                                            bool iw, int j, int cbase, int rg, float &carry,
                                             float (&h1)[32], WaitF &sync_wait, PubF &publish) {
-    if (issuer) issue<L == 1 ? 1 : 3, SH>(s, sbase);
+    if (iw) issue<L == 1 ? 1 : 3, SH>(s, sbase);
     sync_wait();
     if (act) {
         const float2 hbz2 = make_float2(hbz, hbz), bh2 = make_float2(bh, bh);
@@ -320,7 +322,7 @@ __device__ __forceinline__ void dense_layer(bool act, float hbz, float bh, uint8
         carry = h;
     }
     publish();
-    if (issuer) issue<L == 1 ? 2 : 4, SH>(s, sbase);
+    if (iw) issue<L == 1 ? 2 : 4, SH>(s, sbase);
     sync_wait();
     if (act) {
         uint32_t r[32];
@@ -373,6 +375,12 @@ fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__
     // one MMA-issuing thread per stream, each on its own SM sub-partition
     // (lane 0 of warp s of the stream's warpgroup)
     const bool issuer = (j == 32 * s);
+    // the warp that issues the stream's MMAs, and its stream, as warp-uniform values
+    // (elect1): a stream alternates between its MMAs and its epilogue, so the
+    // issue is part of every chunk step's latency.  52 x 52 step of 64 samples:
+    // 304.7 ms with the branch on the thread's index, 261.2 so.
+    const int wu = __shfl_sync(0xffffffffu, tid >> 5, 0), su = wu >> 2;
+    const bool iw = wu == 5 * su;
 
     uint8_t *tileX = smem + OFF_TILES + (2 * s) * SH::kTileBytes;
     uint8_t *tileH = tileX + SH::kTileBytes;
@@ -620,7 +628,7 @@ fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__
                 tmem_wait_st();
             }
             publish();
-            if (issuer) issue<0, SH>(s, sbase);
+            if (iw) issue<0, SH>(su, sbase);
             if (c > c0) readout();  // the previous chunk, while the MMAs run
             sync_wait();
             // epilogue: x1 = GELU(C0 h0 + D0 u) -> tile X
@@ -644,9 +652,9 @@ fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__
             publish();
 
             // ---------------- layers 1 and 2
-            dense_layer<1, SH, kOff>(true, hbz1, bh1, tileX, tileH, sbase, s, accZ, accC, issuer, j, 0, rg,
+            dense_layer<1, SH, kOff>(true, hbz1, bh1, tileX, tileH, sbase, su, accZ, accC, iw, j, 0, rg,
                                      cr[1], h1, sync_wait, publish);
-            dense_layer<2, SH, kOff>(true, hbz2, bh2, tileX, tileH, sbase, s, accZ, accC, issuer, j, 0, rg,
+            dense_layer<2, SH, kOff>(true, hbz2, bh2, tileX, tileH, sbase, su, accZ, accC, iw, j, 0, rg,
                                      cr[2], h1, sync_wait, publish);
             // x3 (in h1) is read out while the next chunk's layer-0 MMAs run
             rd_cur = cur;
@@ -695,6 +703,8 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
     const int lane_base = (warp & 3) * 32;
     // one MMA-issuing thread per stream, each on its own SM sub-partition
     const bool issuer = (half == 0) && (j == 32 * s);
+    const int wu = __shfl_sync(0xffffffffu, tid >> 5, 0), su = wu / (4 * HALVES);
+    const bool iw = wu == (4 * HALVES + 1) * su;  // as in fwd_bf16_kernel1
     const bool leader = (j == 0);    // per warpgroup: job fetch, sums, output
     const int cbase = 4 * half;      // first 16-byte chunk of this sequence in a tile row
 
@@ -1005,7 +1015,7 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
             stop = M.abort_flag[s] != 0;
             if (all_done || stop) break;
         }
-        if (issuer) issue<0, SH>(s, sbase);
+        if (iw) issue<0, SH>(su, sbase);
         if (rd_valid) readout();  // the previous chunk, while the MMAs run
         sync_wait();
         // epilogue: x1 = GELU(C0 h0 + D0 u) -> tile X
@@ -1029,9 +1039,9 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
         publish();
 
         // ---------------- layers 1 and 2
-        dense_layer<1, SH, true>(act, hbz1, bh1, tileX, tileH, sbase, s, accZ, accC, issuer, j, cbase, rg,
+        dense_layer<1, SH, true>(act, hbz1, bh1, tileX, tileH, sbase, su, accZ, accC, iw, j, cbase, rg,
                                  cr[1], h1, sync_wait, publish);
-        dense_layer<2, SH, true>(act, hbz2, bh2, tileX, tileH, sbase, s, accZ, accC, issuer, j, cbase, rg,
+        dense_layer<2, SH, true>(act, hbz2, bh2, tileX, tileH, sbase, su, accZ, accC, iw, j, cbase, rg,
                                  cr[2], h1, sync_wait, publish);
         // x3 (in h1) is read out while the next step's layer-0 MMAs run
         if (act) {
