@@ -311,7 +311,6 @@ struct LruTcArgs {
     int *status;
     // set by launch_lru_tc
     int R, n_slices;
-    uint32_t op[kLruSchedMax];
 };
 bool lru_tc_supported(int nL, int H);
 size_t lru_tc_weight_bytes(int nL);

@@ -136,11 +136,6 @@ __device__ __forceinline__ void sts16(uint32_t a, uint16_t v) {
     asm volatile("st.shared.b16 [%0], %1;" ::"r"(a), "h"(v));
 }
 
-// op word of a slice: bit 0 K chunk of the B tile, bit 1 accumulate from the
-// first K step, bit 2 last slice of its stage (commit to the epilogue).
-// Every stage starts after an epilogue arrival of the same group.
-enum { kLopKc = 1u, kLopAcc = 2u, kLopEnd = 4u };
-
 template <bool F16>
 __global__ void __launch_bounds__(kEpiL + 64, 1) lru_tc_kernel(const __grid_constant__ LruTcArgs A) {
     constexpr int NW = kEpiL / 32;
@@ -248,63 +243,82 @@ __global__ void __launch_bounds__(kEpiL + 64, 1) lru_tc_kernel(const __grid_cons
         }
     } else if (warp == NW + 1) {
         // ------------------------------------------------ MMA issue
-        // Each stage (the slices up to one marked kLopEnd) runs for group 0,
-        // then for group 1, each after that group's epilogue arrival; the
-        // stage's ring slots are released after group 1's MMAs.
-        if (lane == 0 && !M.abort_flag) {
-            uint32_t q = 0, pe0 = 0, pe1 = 0;
+        // Each stage (one or two slices, in the order of lru_tc_schedule) runs for
+        // group 0, then for group 1, each after that group's epilogue arrival; the
+        // stage's ring slots are released after group 1's MMAs.  The whole warp
+        // walks the stages with uniform values, an elected lane issues (elect1).
+        if (!M.abort_flag) {
+            uint32_t q = 0, slot = 0, fph = 0, pe = 0;
             const uint32_t fb = smem_u32(&M.full[0]), ebar = smem_u32(&M.empty[0]);
-            const uint64_t tdesc0 = kdesc_l(smem_u32(tiles)), rd = kdesc_l(smem_u32(ring));
+            const uint32_t e2m = smem_u32(&M.e2m[0]), m2e = smem_u32(&M.m2e[0]);
+            const uint64_t td = kdesc_l(smem_u32(tiles)), rd = kdesc_l(smem_u32(ring));
             bool ok = true;
+            auto wait_u = [&](uint32_t bar, uint32_t parity) {
+                return __all_sync(0xffffffffu, wait_abl(bar, parity, ab)) != 0;
+            };
+            // the next two slices (K chunks 0, 1 of the tile) or the next one
+            auto stage = [&](bool two) {
+                const bool wrap = slot + 1 == (uint32_t)R;
+                const uint32_t s1 = wrap ? 0u : slot + 1;
+#pragma unroll
+                for (int g = 0; g < kGroups; ++g) {
+                    ok = ok && wait_u(e2m + 8 * g, pe);
+                    tc_after();
+                    if (g == 0) {
+                        ok = ok && wait_u(fb + 8 * slot, fph);
+                        if (two) ok = ok && wait_u(fb + 8 * s1, fph ^ (wrap ? 1u : 0u));
+                    }
+                    if (ok && elect1()) {
+                        const uint32_t d = tmem + 128u * g;
+                        const uint64_t bd = td + (uint64_t)((g * kTileG) >> 4);
+                        auto mm4 = [&](uint64_t a, uint64_t b, uint32_t acc) {
+                            mma_ss<idesc_l<F16>()>(d, a, b, acc);
+                            mma_ss<idesc_l<F16>()>(d, a + 2, b + 2, 1u);
+                            mma_ss<idesc_l<F16>()>(d, a + 4, b + 4, 1u);
+                            mma_ss<idesc_l<F16>()>(d, a + 6, b + 6, 1u);
+                        };
+                        mm4(rd + (uint64_t)(slot * (kSliceL >> 4)), bd, 0u);
+                        if (two) mm4(rd + (uint64_t)(s1 * (kSliceL >> 4)), bd + (16384u >> 4), 1u);
+                        mma_commit(m2e + 8 * g);
+                        if (g == kGroups - 1) {
+                            mma_commit(ebar + 8 * slot);
+                            if (two) mma_commit(ebar + 8 * s1);
+                        }
+                    }
+                    __syncwarp();
+                }
+                if (!ok) return;
+                pe ^= 1u;
+                q += two ? 2u : 1u;
+                if (two) {
+                    slot = s1;
+                    fph ^= wrap ? 1u : 0u;
+                }
+                if (++slot == (uint32_t)R) {
+                    slot = 0;
+                    fph ^= 1u;
+                }
+            };
             for (uint32_t row = 0; ok; ++row) {
-                if (!wait_abl(smem_u32(&M.go[row & 1]), (row >> 1) & 1, ab)) {
+                if (!wait_u(smem_u32(&M.go[row & 1]), (row >> 1) & 1)) {
                     ok = false;
                     break;
                 }
                 if (!*(volatile int *)&M.go_flag[row & 1]) break;
-                for (int i = 0; i < A.n_slices && ok;) {
-                    int ns = 1;
-                    while (!(A.op[i + ns - 1] & kLopEnd)) ++ns;
-#pragma unroll
-                    for (int g = 0; g < kGroups; ++g) {
-                        if (!ok) break;
-                        uint32_t &pe = g ? pe1 : pe0;
-                        if (!wait_abl(smem_u32(&M.e2m[g]), pe, ab)) {
-                            ok = false;
-                            break;
-                        }
-                        pe ^= 1u;
-                        tc_after();
-                        for (int k = 0; k < ns; ++k) {
-                            const uint32_t qq = q + k, sl = qq % R;
-                            if (g == 0 && !wait_abl(fb + 8 * sl, (qq / R) & 1, ab)) {
-                                ok = false;
-                                break;
-                            }
-                            const uint32_t op = A.op[i + k];
-                            const uint64_t ad = rd + (uint64_t)(sl * (kSliceL >> 4)),
-                                           bd = tdesc0 + (uint64_t)((g * kTileG + (op & kLopKc) * 16384u) >> 4);
-                            const uint32_t d = tmem + 128u * g;
-                            mma_ss<idesc_l<F16>()>(d, ad, bd, (op & kLopAcc) ? 1u : 0u);
-                            mma_ss<idesc_l<F16>()>(d, ad + 2, bd + 2, 1u);
-                            mma_ss<idesc_l<F16>()>(d, ad + 4, bd + 4, 1u);
-                            mma_ss<idesc_l<F16>()>(d, ad + 6, bd + 6, 1u);
-                        }
-                        if (!ok) break;
-                        mma_commit(smem_u32(&M.m2e[g]));
-                    }
-                    if (!ok) break;
-                    for (int k = 0; k < ns; ++k) mma_commit(ebar + 8 * ((q + k) % R));
-                    q += ns;
-                    i += ns;
+#pragma unroll 1
+                for (int l = 0; l < nL && ok; ++l) {
+                    if (l > 0) stage(false);    // e^gamma B u
+                    if (ok) stage(true);        // Re(C h): h_re, h_im
+                    if (ok) stage(false);       // [W_a; W_g] y
                 }
+                if (ok) stage(false);  // readout
             }
             const uint32_t last = q < (uint32_t)R ? q : (uint32_t)R;
             for (uint32_t t = 0; t < last; ++t) {
                 const uint32_t qq = q - 1 - t;
                 if (!mbar_wait(smem_u32(&M.empty[qq % R]), (qq / R) & 1)) set_status(A.status, PSR_ETIMEOUT);
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 M.abort_flag = 1;
                 set_status(A.status, PSR_ETIMEOUT);
             }
@@ -756,22 +770,18 @@ __global__ void pack_lru_tc_kernel(const float *__restrict__ pk, LruLayout f, Lr
 
 }  // namespace
 
-// Slices of one chunk step and the MMA thread's op words (kLopKc, kLopAcc,
-// kLopEnd); kind[i] = matrix type << 4 | layer.
-int lru_tc_schedule(int nL, uint8_t *kind, uint32_t *op) {
+// Slices of one chunk step, in the order the MMA warp consumes them; kind[i] =
+// matrix type << 4 | layer.
+int lru_tc_schedule(int nL, uint8_t *kind) {
     int n = 0;
-    auto add = [&](int ty, int l, uint32_t fl) {
-        kind[n] = (uint8_t)(ty << 4 | l);
-        op[n] = fl;
-        ++n;
-    };
+    auto add = [&](int ty, int l) { kind[n++] = (uint8_t)(ty << 4 | l); };
     for (int l = 0; l < nL; ++l) {
-        if (l > 0) add(0, l, kLopEnd);  // e^gamma B u: after the previous GLU (x ready)
-        add(1, l, 0);                   // Re(C h), K chunk 0 (h_re): after the scan
-        add(2, l, kLopKc | kLopAcc | kLopEnd);
-        add(3, l, kLopEnd);             // [W_a; W_g] y: y ready
+        if (l > 0) add(0, l);  // e^gamma B u: after the previous GLU (x ready)
+        add(1, l);             // Re(C h), K chunk 0 (h_re): after the scan
+        add(2, l);             // K chunk 1 (h_im)
+        add(3, l);             // [W_a; W_g] y: y ready
     }
-    add(4, 0, kLopEnd);  // readout: x of the last layer ready
+    add(4, 0);  // readout: x of the last layer ready
     return n;
 }
 
@@ -781,8 +791,7 @@ size_t lru_tc_weight_bytes(int nL) { return (size_t)(4 * nL) * kSliceL; }
 
 cudaError_t launch_pack_lru_tc(const float *pk, const LruLayout &f, bool f16, uint8_t *wimg, cudaStream_t stream) {
     LruKinds kd{};
-    uint32_t op[kLruSchedMax];
-    kd.n = lru_tc_schedule(f.nL, kd.kind, op);
+    kd.n = lru_tc_schedule(f.nL, kd.kind);
     const int blocks = (int)(((int64_t)kd.n * 1024 + 255) / 256);
     if (f16) pack_lru_tc_kernel<true><<<blocks, 256, 0, stream>>>(pk, f, kd, wimg);
     else pack_lru_tc_kernel<false><<<blocks, 256, 0, stream>>>(pk, f, kd, wimg);
@@ -796,7 +805,7 @@ cudaError_t launch_lru_tc(LruTcArgs a, int grid, cudaStream_t stream) {
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     uint8_t kind[kLruSchedMax];
-    a.n_slices = lru_tc_schedule(a.nL, kind, a.op);
+    a.n_slices = lru_tc_schedule(a.nL, kind);
     const size_t base = sizeof(MiscL) + 1024 + kTilesBytes + (size_t)a.nL * kCst * kH * sizeof(float) +
                         (size_t)kGroups * kSl * kMaxLL * 2 * kH * sizeof(float);
     if ((size_t)optin < base + 2 * kSliceL) return cudaErrorInvalidConfiguration;

@@ -175,7 +175,8 @@ __global__ void __launch_bounds__(kEpiS + 32, 1)
 
     if (warp == NW) {
         // ------------------------------------------------ MMA issue
-        if (lane == 0 && !M.abort_flag) {
+        // the whole warp, with uniform values; an elected lane issues (elect1)
+        if (!M.abort_flag) {
             const uint32_t e2m = smem_u32(&M.e2m), m2e = smem_u32(&M.m2e);
             const uint64_t wd0 = kdesc_s(smem_u32(wts)), td = kdesc_s(smem_u32(tile)), wdd = kdesc_s(smem_u32(wdb));
             uint32_t pe = 0;
@@ -183,18 +184,21 @@ __global__ void __launch_bounds__(kEpiS + 32, 1)
             // one stage: wait for the epilogue, MMAs over the slices
             // [i0, i0 + ns) (K chunk kc of the tile for the i-th), commit
             auto stage = [&](int i0, int ns) -> bool {
-                if (!wait_abs(e2m, pe, ab)) return false;
+                if (!__all_sync(0xffffffffu, wait_abs(e2m, pe, ab))) return false;
                 pe ^= 1u;
                 tc_after();
-                for (int k = 0; k < ns; ++k) {
-                    const uint64_t ad = wd0 + (uint64_t)((i0 + k) * (kSliceS >> 4)),
-                                   bd = td + (uint64_t)((k * 16384u) >> 4);
-                    mma_ss<idesc_s<F16, kBs>()>(tmem, ad, bd, k > 0 ? 1u : 0u);
-                    mma_ss<idesc_s<F16, kBs>()>(tmem, ad + 2, bd + 2, 1u);
-                    mma_ss<idesc_s<F16, kBs>()>(tmem, ad + 4, bd + 4, 1u);
-                    mma_ss<idesc_s<F16, kBs>()>(tmem, ad + 6, bd + 6, 1u);
+                if (elect1()) {
+                    for (int k = 0; k < ns; ++k) {
+                        const uint64_t ad = wd0 + (uint64_t)((i0 + k) * (kSliceS >> 4)),
+                                       bd = td + (uint64_t)((k * 16384u) >> 4);
+                        mma_ss<idesc_s<F16, kBs>()>(tmem, ad, bd, k > 0 ? 1u : 0u);
+                        mma_ss<idesc_s<F16, kBs>()>(tmem, ad + 2, bd + 2, 1u);
+                        mma_ss<idesc_s<F16, kBs>()>(tmem, ad + 4, bd + 4, 1u);
+                        mma_ss<idesc_s<F16, kBs>()>(tmem, ad + 6, bd + 6, 1u);
+                    }
+                    mma_commit(m2e);
                 }
-                mma_commit(m2e);
+                __syncwarp();
                 return true;
             };
             for (int64_t blk = blockIdx.x; blk < nblk && ok; blk += gridDim.x) {
@@ -212,20 +216,23 @@ __global__ void __launch_bounds__(kEpiS + 32, 1)
                     }
                     if (!ok) break;
                     // readout: A = the x tile (samples in rows 0..31), B = w_d
-                    if (!wait_abs(e2m, pe, ab)) {
+                    if (!__all_sync(0xffffffffu, wait_abs(e2m, pe, ab))) {
                         ok = false;
                         break;
                     }
                     pe ^= 1u;
                     tc_after();
-                    mma_ss<idesc_s<F16, 16>()>(tmem, td, wdd, 0u);
-                    mma_ss<idesc_s<F16, 16>()>(tmem, td + 2, wdd + 2, 1u);
-                    mma_ss<idesc_s<F16, 16>()>(tmem, td + 4, wdd + 4, 1u);
-                    mma_ss<idesc_s<F16, 16>()>(tmem, td + 6, wdd + 6, 1u);
-                    mma_commit(m2e);
+                    if (elect1()) {
+                        mma_ss<idesc_s<F16, 16>()>(tmem, td, wdd, 0u);
+                        mma_ss<idesc_s<F16, 16>()>(tmem, td + 2, wdd + 2, 1u);
+                        mma_ss<idesc_s<F16, 16>()>(tmem, td + 4, wdd + 4, 1u);
+                        mma_ss<idesc_s<F16, 16>()>(tmem, td + 6, wdd + 6, 1u);
+                        mma_commit(m2e);
+                    }
+                    __syncwarp();
                 }
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 M.abort_flag = 1;
                 set_status(status, PSR_ETIMEOUT);
             }

@@ -179,7 +179,8 @@ __global__ void __launch_bounds__(kEpiC + 32, 1)
 
     if (warp == NW) {
         // ------------------------------------------------ MMA issue
-        if (lane == 0 && !M.abort_flag) {
+        // the whole warp, with uniform values; an elected lane issues (elect1)
+        if (!M.abort_flag) {
             const uint32_t e2m = smem_u32(&M.e2m), m2e = smem_u32(&M.m2e);
             const uint64_t bx = kdesc_c(smem_u32(tileX)), bh = kdesc_c(smem_u32(tileH)),
                            ad0 = kdesc_c(smem_u32(wd));
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(kEpiC + 32, 1)
             // K step kk (16 inputs) of a B tile: chunk kk / 4 (4 KB apart), 32 bytes per step
             auto bk = [](uint64_t b, int kk) { return b + (uint64_t)(((kk >> 2) * 4096 + (kk & 3) * 32) >> 4); };
             auto wait_e = [&]() -> bool {
-                if (!wait_abc(e2m, pe, ab)) return false;
+                if (!__all_sync(0xffffffffu, wait_abc(e2m, pe, ab))) return false;
                 pe ^= 1u;
                 tc_after();
                 return true;
@@ -208,30 +209,38 @@ __global__ void __launch_bounds__(kEpiC + 32, 1)
                     mma_ss<idesc_c<kBc>()>(tmem + dc, a, bk(b, kk), 1u);
                 }
             };
-            for (int64_t blk = blockIdx.x; blk < nblk && ok; blk += gridDim.x) {
-                for (int t = 0; t < N && ok; ++t) {
-                    if (!(ok = wait_e())) break;  // h0
-                    mm_t(kTmZ, kWC0, bh, false);
-                    mma_commit(m2e);
-                    if (!(ok = wait_e())) break;  // x1
-                    mm_t(kTmZ, kWWz1, bx, false);
-                    mm_t(kTmH, kWWh1, bx, false);
-                    mma_commit(m2e);
-                    if (!(ok = wait_e())) break;  // h1
-                    mm_t(kTmZ, kWC1, bh, false);
-                    mm_s(kTmZ, 0, bx);
-                    mma_commit(m2e);
-                    if (!(ok = wait_e())) break;  // x2
-                    mm_t(kTmZ, kWWz2, bx, false);
-                    mm_t(kTmH, kWWh2, bx, false);
-                    mma_commit(m2e);
-                    if (!(ok = wait_e())) break;  // h2
-                    mm_t(kTmZ, kWC2, bh, false);
-                    mm_s(kTmZ, 1, bx);
+            // one stage: the epilogue's arrival, the MMAs, their commit
+            auto stage = [&](auto &&mmas) -> bool {
+                if (!wait_e()) return false;
+                if (elect1()) {
+                    mmas();
                     mma_commit(m2e);
                 }
+                __syncwarp();
+                return true;
+            };
+            for (int64_t blk = blockIdx.x; blk < nblk && ok; blk += gridDim.x) {
+                for (int t = 0; t < N && ok; ++t) {
+                    // h0; x1; h1; x2; h2
+                    ok = stage([&] { mm_t(kTmZ, kWC0, bh, false); }) && stage([&] {
+                             mm_t(kTmZ, kWWz1, bx, false);
+                             mm_t(kTmH, kWWh1, bx, false);
+                         }) &&
+                         stage([&] {
+                             mm_t(kTmZ, kWC1, bh, false);
+                             mm_s(kTmZ, 0, bx);
+                         }) &&
+                         stage([&] {
+                             mm_t(kTmZ, kWWz2, bx, false);
+                             mm_t(kTmH, kWWh2, bx, false);
+                         }) &&
+                         stage([&] {
+                             mm_t(kTmZ, kWC2, bh, false);
+                             mm_s(kTmZ, 1, bx);
+                         });
+                }
             }
-            if (!ok) {
+            if (!ok && lane == 0) {
                 M.abort_flag = 1;
                 set_status(status, PSR_ETIMEOUT);
             }
