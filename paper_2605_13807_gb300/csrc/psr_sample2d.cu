@@ -24,6 +24,45 @@ namespace {
 
 __device__ __forceinline__ int pos2(int Lx, int i, int j) { return j * Lx + ((j & 1) ? Lx - 1 - i : i); }
 
+// acc[w][b] += sum over m of W_w[m][j] v[b][m], in order of m, for NW weight
+// matrices (p[w] points at column j).  A CTA reads every weight from L2 for each
+// patch and layer with H threads, so the loads in flight set its pace: the next
+// 16 rows of every matrix are loaded while 16 are used.
+template <int H, int B, int NW>
+__device__ __forceinline__ void matvecs(const float *const (&p)[NW], const float *v, float (&acc)[NW][B]) {
+    constexpr int U = 16;
+    float w0[NW][U], w1[NW][U];
+    auto load = [&](float(&w)[NW][U], int m0) {
+#pragma unroll
+        for (int i = 0; i < NW; ++i)
+#pragma unroll
+            for (int u = 0; u < U; ++u) w[i][u] = p[i][(m0 + u) * H];
+    };
+    auto use = [&](const float(&w)[NW][U], int m0) {
+#pragma unroll
+        for (int q = 0; q < U; q += 4)
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const float4 x = *reinterpret_cast<const float4 *>(v + b * H + m0 + q);
+#pragma unroll
+                for (int i = 0; i < NW; ++i) {
+                    acc[i][b] = fmaf(w[i][q], x.x, acc[i][b]);
+                    acc[i][b] = fmaf(w[i][q + 1], x.y, acc[i][b]);
+                    acc[i][b] = fmaf(w[i][q + 2], x.z, acc[i][b]);
+                    acc[i][b] = fmaf(w[i][q + 3], x.w, acc[i][b]);
+                }
+            }
+    };
+    load(w0, 0);
+#pragma unroll 1
+    for (int m0 = 0; m0 < H; m0 += 2 * U) {
+        load(w1, m0 + U);
+        use(w0, m0);
+        if (m0 + 2 * U < H) load(w0, m0 + 2 * U);
+        use(w1, m0 + U);
+    }
+}
+
 template <int H, int B>
 __global__ void __launch_bounds__(H) sample2d_kernel(const float *__restrict__ pk, F2Layout f,
                                                      const float *__restrict__ unif, int64_t n,
@@ -36,7 +75,7 @@ __global__ void __launch_bounds__(H) sample2d_kernel(const float *__restrict__ p
     const int Px = Lx >> 1, Py = Ly >> 1, N = Lx * Ly, Np = Px * Py;
     float *buf = smem;                          // [B][nL][H][Px] states by column
     float *xs = buf + (size_t)B * nL * H * Px;  // [B][H] layer input / output of the patch
-    float *hs = xs + B * H;                     // [B][H] states of the patch's current layer
+    float *hs = xs + B * H;                     // [B][H] h_V of the patch's current layer, then its states
     float *lg = hs + B * H;                     // [B][16] logits
     __shared__ int s_vprev[B][32];              // previous row's values by column (updated in place)
     __shared__ int s_vlast[B];                  // value of the previous patch on the path
@@ -59,11 +98,13 @@ __global__ void __launch_bounds__(H) sample2d_kernel(const float *__restrict__ p
         const int pj = t / Px, k = t - pj * Px;
         const int pi = (pj & 1) ? Px - 1 - k : k;
         const int pprev = (pj & 1) ? pi + 1 : pi - 1;  // column of the previous patch in the row
+        const int pn = k + 1 == Px ? pi : (pj & 1) ? pi - 1 : pi + 1;  // column of the next patch
         float hres[B];
 #pragma unroll
         for (int b = 0; b < B; ++b) hres[b] = 0.0f;
         for (int l = 0; l < nL; ++l) {
-            float z[B], c[B], y[B];
+            float acc[3][B];  // z, c, y
+            float(&z)[B] = acc[0], (&c)[B] = acc[1], (&y)[B] = acc[2];
             const float bz = pk[f.bz[l] + j], bh = pk[f.bh[l] + j];
             if (l == 0) {
                 const float *WzT = pk + f.WzT[0], *WhxT = pk + f.WhxT[0], *DT = pk + f.DT[0];
@@ -76,31 +117,23 @@ __global__ void __launch_bounds__(H) sample2d_kernel(const float *__restrict__ p
                     y[b] = (vh >= 0 ? DT[vh * H + j] : 0.0f) + (vv >= 0 ? DT[(16 + vv) * H + j] : 0.0f);
                 }
             } else {
-                const float *WzT = pk + f.WzT[l], *WhxT = pk + f.WhxT[l];
 #pragma unroll
                 for (int b = 0; b < B; ++b) {
                     z[b] = bz;
                     c[b] = bh;
+                    y[b] = (l >= 2) ? hres[b] : 0.0f;
                 }
-#pragma unroll 4
-                for (int m = 0; m < H; ++m) {
-                    const float wz = WzT[m * H + j], wh = WhxT[m * H + j];
-#pragma unroll
-                    for (int b = 0; b < B; ++b) {
-                        const float xv = xs[b * H + m];
-                        z[b] += wz * xv;
-                        c[b] += wh * xv;
-                    }
-                }
+                const float *const p[3] = {pk + f.WzT[l] + j, pk + f.WhxT[l] + j, pk + f.DT[l] + j};
+                matvecs<H, B, 3>(p, xs, acc);
             }
             if (pj > 0) {
-                const float *Wv = pk + f.WhvT[l];
-#pragma unroll 4
-                for (int m = 0; m < H; ++m) {
-                    const float w = Wv[m * H + j];
+                const float *const p[1] = {pk + f.WhvT[l] + j};
+                float a1[1][B];
 #pragma unroll
-                    for (int b = 0; b < B; ++b) c[b] += w * buf[(((size_t)b * nL + l) * H + m) * Px + pi];
-                }
+                for (int b = 0; b < B; ++b) a1[0][b] = c[b];
+                matvecs<H, B, 1>(p, hs, a1);
+#pragma unroll
+                for (int b = 0; b < B; ++b) c[b] = a1[0][b];
             }
             float h[B];
 #pragma unroll
@@ -110,38 +143,30 @@ __global__ void __launch_bounds__(H) sample2d_kernel(const float *__restrict__ p
                 // explicit rounding order: identical for every samples-per-CTA instance
                 h[b] = fmaf(a, hH, __fmul_rn(1.0f - a, c[b]));
             }
-            __syncthreads();  // every read of column pi (h_V) is done
+            __syncthreads();  // every read of hs (h_V) is done
 #pragma unroll
             for (int b = 0; b < B; ++b) {
                 buf[(((size_t)b * nL + l) * H + j) * Px + pi] = h[b];
                 hs[b * H + j] = h[b];
             }
             __syncthreads();
-            if (l >= 1) {
-#pragma unroll
-                for (int b = 0; b < B; ++b) y[b] = (l >= 2) ? hres[b] : 0.0f;
-                const float *DT = pk + f.DT[l];
-#pragma unroll 4
-                for (int m = 0; m < H; ++m) {
-                    const float wd = DT[m * H + j];
-#pragma unroll
-                    for (int b = 0; b < B; ++b) y[b] += wd * xs[b * H + m];
-                }
-            }
             {
-                const float *Ct = pk + f.CT[l];
-#pragma unroll 4
-                for (int m = 0; m < H; ++m) {
-                    const float w = Ct[m * H + j];
+                const float *const p[1] = {pk + f.CT[l] + j};
+                float a1[1][B];
 #pragma unroll
-                    for (int b = 0; b < B; ++b) y[b] += w * hs[b * H + m];
-                }
+                for (int b = 0; b < B; ++b) a1[0][b] = y[b];
+                matvecs<H, B, 1>(p, hs, a1);
+#pragma unroll
+                for (int b = 0; b < B; ++b) y[b] = a1[0][b];
             }
             __syncthreads();  // every read of xs and hs is done
 #pragma unroll
             for (int b = 0; b < B; ++b) {
                 xs[b * H + j] = gelu_f(y[b]);
                 hres[b] = h[b];
+                // h_V of the next layer, or of layer 0 at the next patch's column
+                // (unit j's states are this thread's own)
+                hs[b * H + j] = buf[(((size_t)b * nL + (l + 1 < nL ? l + 1 : 0)) * H + j) * Px + (l + 1 < nL ? pi : pn)];
             }
             __syncthreads();
         }
@@ -150,7 +175,8 @@ __global__ void __launch_bounds__(H) sample2d_kernel(const float *__restrict__ p
             const int b = j >> 4, o = j & 15;
             const float *Wo = pk + f.Wo;
             float v = Wo[16 * H + o];
-            for (int m = 0; m < H; ++m) v += Wo[o * H + m] * xs[b * H + m];
+#pragma unroll 16
+            for (int m = 0; m < H; ++m) v = fmaf(Wo[o * H + m], xs[b * H + m], v);
             lg[b * 16 + o] = v;
         }
         __syncthreads();
