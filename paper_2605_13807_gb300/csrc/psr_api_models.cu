@@ -45,9 +45,10 @@ cudaError_t tc2_prepare(const float *theta, const T2Layout &tl, int Lx, bool f16
 }
 
 // The jobs of `jb` on the tensor cores; row checkpoints as 16-bit images
-// (img_out written in mode 0 when set, img_in read in mode 1).
+// (img_out written in mode 0 when set, img_in read in mode 1).  images > 1: the
+// connected configurations of that many sample sets in one launch (Fwd2TcArgs).
 cudaError_t tc2_run(psr_context *ctx, const Fwd2Jobs &jb, bool f16, const float *theta, const T2Layout &tl,
-                    const Tc2 &t, const uint8_t *img_in, uint8_t *img_out) {
+                    const Tc2 &t, const uint8_t *img_in, uint8_t *img_out, int images = 1, int64_t n_samples = 0) {
     Fwd2TcArgs a{};
     a.mode = jb.mode;
     a.f16 = f16 ? 1 : 0;
@@ -56,6 +57,8 @@ cudaError_t tc2_run(psr_context *ctx, const Fwd2Jobs &jb, bool f16, const float 
     a.u1 = jb.g.u1;
     a.n_jobs = jb.g.n_jobs;
     a.n_jobs_dev = jb.g.n_jobs_dev;
+    a.images = images;
+    a.n_samples = n_samples;
     a.spins = jb.g.spins;
     a.entries = jb.g.entries;
     a.img_in = img_in;
@@ -74,7 +77,7 @@ cudaError_t tc2_run(psr_context *ctx, const Fwd2Jobs &jb, bool f16, const float 
     if (jb.g.n_jobs >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;  // job indices are 32-bit
     int W, S;
     fwd2d_tc_geometry(a.Lx, &W, &S);
-    int64_t grid = (jb.g.n_jobs + S - 1) / S;
+    int64_t grid = (images * jb.g.n_jobs + S - 1) / S;
     if (grid > ctx->num_sms) grid = ctx->num_sms;
     if (grid < 1) grid = 1;
     return launch_fwd2d_tc(a, (int)grid, ctx->stream);
@@ -665,7 +668,11 @@ int sym2d_run(const psr_params *params, const uint8_t *samples, int64_t n, int32
     }
     if (eloc && cap > 0) {
         StageScope sc(ctx, PSR_STAGE_FWD_CONNECTED);
-        for (int g = 0; g < 8; ++g) {
+        // On the tensor cores the images' configurations are one launch: each launch
+        // ends with CTAs that wait for the last rows of others (eight launches of 24
+        // row steps each at 200 samples of 10 x 10).
+        const int sets = tc && 8 * cap < ((int64_t)1 << 31) ? 8 : 1;  // job indices are 32-bit
+        for (int g = 0; g < 8; g += sets) {
             Fwd2Jobs jc = js;
             jc.mode = 1;
             jc.g.n_jobs = cap;
@@ -678,7 +685,7 @@ int sym2d_run(const psr_params *params, const uint8_t *samples, int64_t n, int32
             jc.g.logp_out = nullptr;
             jc.g.carries_out = nullptr;
             jc.job_counter = counters + 1 + g;
-            if (tc) PSR_TRY(tc2_run(ctx, jc, f16, theta, tl, t2, ckimg8 + (size_t)g * n * ckpt_img, nullptr));
+            if (tc) PSR_TRY(tc2_run(ctx, jc, f16, theta, tl, t2, ckimg8 + (size_t)g * n * ckpt_img, nullptr, sets, n));
             else PSR_TRY(launch_fwd2d_f32(jc, pk, f, ctx->num_sms, st));
         }
         PSR_TRY(launch_sym_delta(b.entries, b.offsets + n, cap, lp8, n, delta8, dsym, st));

@@ -78,7 +78,8 @@ constexpr int kEpi = 512;             // epilogue threads: 512 / H per hidden un
 constexpr int kThreads2 = kEpi + 96;  // + producer, MMA and image warps
 
 struct Slot2 {
-    int job;              // -1: needs a job, -2: none left (a launch holds < 2^31 jobs)
+    int job;              // -1: needs a job, -2: none left, else a job is running
+    int64_t out;          // its place in A.out
     int sample, p, q;     // configuration (p, q: flipped sites or -1)
     int row, r0, n_up;    // current patch row, first row, up spins before it
     float acc;            // sum of log P (mode 0) or of its differences (mode 1)
@@ -248,7 +249,8 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
     }
     if (tid == 0) mbar_arrive(smem_u32(&M.go[0]));  // row step 0 runs
     __syncthreads();
-    const long long njobs = A.mode == 1 ? (long long)*A.n_jobs_dev : (long long)A.n_jobs;
+    const long long per_set = A.mode == 1 ? (long long)*A.n_jobs_dev : (long long)A.n_jobs;
+    const long long njobs = A.images > 1 ? per_set * A.images : per_set;
     const uint32_t hvb = smem_u32(&M.hv);
 
     if (warp == NW) {
@@ -569,7 +571,7 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
                 float a = st.acc;
                 for (int c = 0; c < nch; ++c) a += st.part[c];
                 st.acc = a;
-                if (st.row + 1 >= Py) A.out[st.job] = 0.5f * a;
+                if (st.row + 1 >= Py) A.out[st.out] = 0.5f * a;
             }
             __syncwarp();
         };
@@ -594,9 +596,12 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
                         continue;
                     }
                     int sample = (int)nj, p = -1, qq = -1, r0 = 0;
+                    int64_t place = (int64_t)nj;
                     if (A.mode == 1) {
-                        const int32_t *e = A.entries + 3 * nj;
-                        sample = e[0];
+                        const int64_t set = A.images > 1 ? (uint32_t)nj / (uint32_t)per_set : 0u;
+                        place += set * (A.n_jobs - per_set);
+                        const int32_t *e = A.entries + 3 * place;
+                        sample = (int)(set * A.n_samples) + e[0];
                         p = e[1];
                         qq = e[2];
                         r0 = (p / Lx) >> 1;
@@ -611,7 +616,8 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
                         st.v[lane] = (uint8_t)patch_value(sp, Lx, lane, r0, p, qq);
                     }
                     if (lane == 0) {
-                        st.job = (int)nj;
+                        st.job = 0;
+                        st.out = place;
                         st.sample = sample;
                         st.p = p;
                         st.q = qq;

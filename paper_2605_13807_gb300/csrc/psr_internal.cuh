@@ -235,6 +235,11 @@ struct Fwd2TcArgs {
     int f16;            // operands FP16 (1) or BF16 (0)
     int64_t n_jobs;
     const int64_t *n_jobs_dev;
+    // mode 1: the jobs of `images` sample sets (0: one), set g with its samples at
+    // g n_samples of spins, img_in and logp_ref and its jobs at g n_jobs of
+    // entries and out; n_jobs_dev counts the jobs of one set
+    int images;
+    int64_t n_samples;
     const uint8_t *spins;
     const int32_t *entries;
     const uint8_t *img_in;

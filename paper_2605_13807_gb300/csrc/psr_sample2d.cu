@@ -27,7 +27,8 @@ __device__ __forceinline__ int pos2(int Lx, int i, int j) { return j * Lx + ((j 
 // acc[w][b] += sum over m of W_w[m][j] v[b][m], in order of m, for NW weight
 // matrices (p[w] points at column j).  A CTA reads every weight from L2 for each
 // patch and layer with H threads, so the loads in flight set its pace: the next
-// 16 rows of every matrix are loaded while 16 are used.
+// 16 rows of every matrix are loaded while 16 are used (200 samples of 10 x 10,
+// three layers of 256: 3.86 -> 1.3 ms; before, four rows of one matrix at a time).
 template <int H, int B, int NW>
 __device__ __forceinline__ void matvecs(const float *const (&p)[NW], const float *v, float (&acc)[NW][B]) {
     constexpr int U = 16;
