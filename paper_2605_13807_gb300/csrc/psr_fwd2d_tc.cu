@@ -82,8 +82,12 @@ struct Slot2 {
     int64_t out;          // its place in A.out
     int sample, p, q;     // configuration (p, q: flipped sites or -1)
     int row, r0, n_up;    // current patch row, first row, up spins before it
-    float acc;            // sum of log P (mode 0) or of its differences (mode 1)
-    float part[4];        // the row's readout sums, per 8-column chunk
+    // sum of log P (mode 0) or of its differences (mode 1) over the rows before the
+    // one whose sums (part, per 8-column chunk) are still to be added: its job's
+    // last row or not, and that job's place in A.out
+    float acc, part[4];
+    int pend, pend_last;
+    int64_t pend_out;
     uint8_t v[32];        // patch values of the current row, by column
     uint8_t vprev[32];    // previous row's values, by column
 };
@@ -238,6 +242,7 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
     for (int s = tid; s < kMaxSlots; s += blockDim.x) {
         M.slot[s].job = -1;
         M.slot[s].acc = 0.0f;
+        M.slot[s].pend = 0;
     }
     tc_before();
     __syncthreads();
@@ -391,7 +396,7 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
                 // readout once both halves' layer input of the readout (x) is complete
                 commit(HL);
                 for (int g = 0; g < NH; ++g) wait_e(g);
-                run(tmem + 128u * NH, xd, KC, 0u);
+                run(tmem, xd, KC, 0u);
                 for (int g = 0; g < NH; ++g) commit(g);  // logits of the row
             }
             // the MMAs of the last slices complete before the CTA may exit
@@ -485,7 +490,7 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
         const uint32_t lane_off = (uint32_t)(q4 * 32) << 16;
         const uint32_t tz = tmem + lane_off + 128u * g;          // z, then y
         const uint32_t tcc = tmem + lane_off + 128u * (NH + g);  // c
-        const uint32_t tlg = tmem + lane_off + 128u * NH;        // logits (lanes 32 q4 + 0..15)
+        const uint32_t tlg = tmem + lane_off;                     // logits (lanes 32 q4 + 0..15)
         // unit j's element of row k (mod 8) of a K-major tile, 128-byte swizzle
         // (16-byte group c of row k at c ^ (k & 7)); rows n .. n + 7 of a tile, n a
         // multiple of 8, are at tile + 128 n + koff[0 .. 7]
@@ -563,25 +568,31 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
                 cc = c2;
             }
         };
-        // the previous row's readout sums into the job's total (fixed order),
-        // and the job's log psi after its last row (slot s, its warp)
+        // Adds the pending row's readout sums to its job's total (fixed order), and
+        // stores the job's result if that was its last row; then the current row is
+        // the pending one (slot s, its warp).
         auto fold = [&](int s) {
             Slot2 &st = M.slot[s];
-            if (lane == 0 && st.job >= 0) {
-                float a = st.acc;
-                for (int c = 0; c < nch; ++c) a += st.part[c];
-                st.acc = a;
-                if (st.row + 1 >= Py) A.out[st.out] = 0.5f * a;
+            if (lane == 0) {
+                if (st.pend) {
+                    float a = st.acc;
+                    for (int c = 0; c < nch; ++c) a += st.part[c];
+                    if (st.pend_last) A.out[st.pend_out] = 0.5f * a;
+                    st.acc = st.pend_last ? 0.0f : a;
+                }
+                st.pend = st.job >= 0;
+                st.pend_last = st.row + 1 >= Py;
+                st.pend_out = st.out;
             }
             __syncwarp();
         };
 
-        for (uint32_t row_it = 0; ok; ++row_it) {
-            // ---- slot update (warp s for slot s): finished or empty slots
-            // take the next job, the others advance one patch row
+        // slot update (warp s for slot s): finished or empty slots take the next
+        // job, the others advance one patch row
+        auto update = [&]() {
             for (int s = warp; s < S; s += NW) {
                 Slot2 &st = M.slot[s];
-                if (row_it > 0) fold(s);
+                fold(s);
                 const int job = st.job;
                 if (job == -2) continue;
                 const uint8_t *sp;
@@ -624,7 +635,6 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
                         st.row = r0;
                         st.r0 = r0;
                         st.n_up = up;
-                        st.acc = 0.0f;
                     }
                     r = r0;
                 } else {
@@ -646,20 +656,104 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
                 }
                 __syncwarp();
             }
-            if (epi_bar_or(!ok || *ab)) {
-                ok = false;
-                break;
-            }
+        };
+        // the slots of row step `row` are set: does a row step follow it?
+        auto signal = [&](uint32_t row) {
             if (tid == 0) {
-                // does a row step follow this one?
                 bool more = false;
                 for (int s = 0; s < S; ++s)
                     if (M.slot[s].job >= 0 && M.slot[s].row + 1 < Py) more = true;
                 if (!more) more = (long long)atomicAdd(A.job_counter, 0ull) < njobs;
-                M.go_flag[(row_it + 1) & 1] = more ? 1 : 0;
-                mbar_arrive(smem_u32(&M.go[(row_it + 1) & 1]));
+                M.go_flag[(row + 1) & 1] = more ? 1 : 0;
+                mbar_arrive(smem_u32(&M.go[(row + 1) & 1]));
                 mbar_arrive(smem_u32(&M.slots));
             }
+        };
+        // Readout: masked 16-way softmax of every patch of a row; warp w takes
+        // columns 8 w .. 8 w + 7 (slot w / nch, chunk w % nch).  prepare() takes what
+        // it needs of the row from the slot, softmax() runs once the next row's input
+        // is written, while that row's first MMAs run (E_loc of the 16 x 16 model:
+        // 7.82 ms with the readout and the slot update in line, 7.45 so).
+        bool ro = false;                  // this warp has a row to read out
+        uint32_t lr[8], allowed = 0, vals = 0;  // logits; bit e: this lane's value allowed in column e; 4-bit values
+        int ncol = 0, dirn = 1;
+        int64_t pos = 0;                  // place of column 0 in logp_out
+        float ref = 0.0f;
+        auto prepare = [&]() {
+            const int s = warp / nch, i0 = 8 * (warp - s * nch);
+            ro = warp < S * nch && M.slot[s].job >= 0;
+            // (all set anew: none of them lives through the layers)
+            allowed = vals = 0;
+            ncol = 0;
+            dirn = 1;
+            pos = 0;
+            ref = 0.0f;
+            if (!ro) return;
+            const Slot2 &st = M.slot[s];
+            const int r = st.row;
+            const bool odd = r & 1;
+            const int pc_lane = __popc(lane & 15);
+            ncol = min(8, Px - i0);
+            dirn = odd ? -1 : 1;
+            const int k0 = odd ? Px - 1 - i0 : i0;  // path position of column i0
+            pos = (int64_t)st.sample * Np + r * Px + k0;
+            ref = (A.mode == 1 && lane < ncol) ? A.logp_ref[pos + dirn * lane] : 0.0f;
+            // up spins of the row's patches before path position `lane`
+            const int c = odd ? Px - 1 - lane : lane;  // column at path position lane
+            const int pc = lane < Px ? __popc(st.v[c]) : 0;
+            int incl = pc;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += t;
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int k = k0 + dirn * e;
+                const int up = st.n_up + __shfl_sync(0xffffffffu, incl - pc, k);
+                const int down = 2 * r * Lx + 4 * k - up;
+                if (!A.u1 || (up + pc_lane <= N / 2 && down + 4 - pc_lane <= N / 2)) allowed |= 1u << e;
+                vals |= (uint32_t)(st.v[i0 + e] & 15) << (4 * e);
+            }
+        };
+        auto softmax = [&]() {
+            if (!ro) return;
+            // the eight columns side by side (a column's two reductions are a
+            // chain of eight shuffles); columns past P_x are not summed
+            const float bo = A.theta[A.tl.bo + (lane & 15)];
+            float lg[8], m[8], ex[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                lg[e] = __uint_as_float(lr[e]) + bo;
+                m[e] = (allowed >> e) & 1u ? lg[e] : -INFINITY;
+            }
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) m[e] = fmaxf(m[e], __shfl_xor_sync(0xffffffffu, m[e], o, 16));
+#pragma unroll
+            for (int e = 0; e < 8; ++e) ex[e] = (allowed >> e) & 1u ? __expf(lg[e] - m[e]) : 0.0f;
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) ex[e] += __shfl_xor_sync(0xffffffffu, ex[e], o, 16);
+            float rsum = 0.0f;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                float lp = (allowed >> e) & 1u ? lg[e] - m[e] - __logf(ex[e]) : -INFINITY;
+                lp = __shfl_sync(0xffffffffu, lp, (vals >> (4 * e)) & 15u);
+                const float rf = __shfl_sync(0xffffffffu, ref, e);
+                if (e >= ncol) continue;
+                if (A.mode != 1 && A.logp_out && lane == 0) A.logp_out[pos + dirn * e] = lp;
+                rsum += A.mode == 1 ? lp - rf : lp;
+            }
+            if (lane == 0) M.slot[warp / nch].part[warp % nch] = rsum;
+        };
+
+        if (ok) update();
+        if (epi_bar_or(!ok || *ab)) ok = false;
+        if (ok) signal(0);
+        for (uint32_t row_it = 0; ok; ++row_it) {
             // ---- layer-0 input: one-hot (v_H, v_V) of every column, K chunk 0
             {
                 constexpr uint32_t kOne = F16 ? 0x3C00u : 0x3F80u;  // 1.0
@@ -688,6 +782,7 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
                 }
             }
             arrive_e2m();
+            if (row_it > 0 && ok) softmax();  // of the row before
 
             for (int l = 0; l < nL; ++l) {
                 // ---- gates and scan along each slot's row (path order)
@@ -770,83 +865,37 @@ __global__ void __launch_bounds__(kThreads2, 1) fwd2d_tc_kernel(const __grid_con
                 arrive_e2m();
             }
 
-            // ---- readout: masked 16-way softmax of every patch of the row;
-            // warp w takes 8 columns (slot w / nch, chunk w % nch)
-            wait_m2e();
-            if (ok && warp < S * nch) {
-                const int s = warp / nch, c8 = warp - s * nch;
-                Slot2 &st = M.slot[s];
-                if (st.job >= 0) {
-                    const int r = st.row, n0 = s * W, i0 = 8 * c8;
-                    const bool odd = r & 1;
-                    const float bo = A.theta[A.tl.bo + (lane & 15)];
-                    const int pc_lane = __popc(lane & 15);
-                    // up spins of the row's patches before path position `lane`
-                    int upx;
-                    {
-                        const int c = odd ? Px - 1 - lane : lane;  // column at path position lane
-                        const int pc = lane < Px ? __popc(st.v[c]) : 0;
-                        int incl = pc;
-#pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-                            if (lane >= o) incl += t;
-                        }
-                        upx = incl - pc;
-                    }
-                    float ref = 0.0f;
-                    if (A.mode == 1 && lane < 8 && i0 + lane < Px) {
-                        const int i = i0 + lane, k = odd ? Px - 1 - i : i;
-                        ref = A.logp_ref[(size_t)st.sample * Np + r * Px + k];
-                    }
-                    uint32_t lr[8];
-                    tmem_ld8(tlg + n0 + i0, lr[0], lr[1], lr[2], lr[3], lr[4], lr[5], lr[6], lr[7]);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                                 : "+r"(lr[0]), "+r"(lr[1]), "+r"(lr[2]), "+r"(lr[3]), "+r"(lr[4]), "+r"(lr[5]),
-                                   "+r"(lr[6]), "+r"(lr[7])::"memory");
-                    // the eight columns side by side (a column's two reductions are a
-                    // chain of eight shuffles); columns past P_x are not summed
-                    float lg[8], m[8], ex[8];
-                    uint32_t allowed = 0;  // bit e: this lane's value in column e
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int i = i0 + e, k = odd ? Px - 1 - i : i;
-                        const int up = st.n_up + __shfl_sync(0xffffffffu, upx, k);
-                        const int down = 2 * r * Lx + 4 * k - up;
-                        if (!A.u1 || (up + pc_lane <= N / 2 && down + 4 - pc_lane <= N / 2)) allowed |= 1u << e;
-                        lg[e] = __uint_as_float(lr[e]) + bo;
-                        m[e] = (allowed >> e) & 1u ? lg[e] : -INFINITY;
-                    }
-#pragma unroll
-                    for (int o = 8; o > 0; o >>= 1)
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) m[e] = fmaxf(m[e], __shfl_xor_sync(0xffffffffu, m[e], o, 16));
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) ex[e] = (allowed >> e) & 1u ? __expf(lg[e] - m[e]) : 0.0f;
-#pragma unroll
-                    for (int o = 8; o > 0; o >>= 1)
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) ex[e] += __shfl_xor_sync(0xffffffffu, ex[e], o, 16);
-                    float rsum = 0.0f;
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int i = i0 + e, k = odd ? Px - 1 - i : i;
-                        float lp = (allowed >> e) & 1u ? lg[e] - m[e] - __logf(ex[e]) : -INFINITY;
-                        lp = __shfl_sync(0xffffffffu, lp, st.v[i]);
-                        const float rf = __shfl_sync(0xffffffffu, ref, e);
-                        if (i >= Px) continue;
-                        if (A.mode != 1 && A.logp_out && lane == 0) A.logp_out[(size_t)st.sample * Np + r * Px + k] = lp;
-                        rsum += A.mode == 1 ? lp - rf : lp;
-                    }
-                    if (lane == 0) st.part[c8] = rsum;
-                }
+            // ---- end of the row: what its softmax needs, then the slots of the next
+            // row (the MMA and image warps start on it), then the logits
+            prepare();
+            if (epi_bar_or(!ok || *ab)) {
+                ok = false;
+                break;
             }
-            tc_before();
+            const bool last = !*(volatile int *)&M.go_flag[(row_it + 1) & 1];
+            if (!last) update();
+            else
+                for (int s = warp; s < S; s += NW) fold(s);
             if (epi_bar_or(!ok)) {
                 ok = false;
                 break;
             }
-            if (!*(volatile int *)&M.go_flag[(row_it + 1) & 1]) {
+            if (!last) signal(row_it + 1);
+            wait_m2e();
+#pragma unroll
+            for (int e = 0; e < 8; ++e) lr[e] = 0;
+            if (ro) {
+                tmem_ld8(tlg + 8 * warp, lr[0], lr[1], lr[2], lr[3], lr[4], lr[5], lr[6], lr[7]);
+                asm volatile("tcgen05.wait::ld.sync.aligned;"
+                             : "+r"(lr[0]), "+r"(lr[1]), "+r"(lr[2]), "+r"(lr[3]), "+r"(lr[4]), "+r"(lr[5]),
+                               "+r"(lr[6]), "+r"(lr[7])::"memory");
+            }
+            if (last) {
+                if (ok) softmax();
+                if (epi_bar_or(!ok)) {
+                    ok = false;
+                    break;
+                }
                 for (int s = warp; s < S; s += NW) fold(s);
                 break;
             }
