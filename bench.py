@@ -44,17 +44,16 @@ WORKLOADS = {
 
 # kernels launched per call of each entry point (BF16 precision)
 LAUNCHES = {"logpsi": 4, "local_energy": 11}
-TC_STASH_BUDGET = 16 << 30      # bytes of stash and layer arrays per gradient batch
+GRAD_BUDGET = 2 << 30           # bytes of layer arrays per gradient batch
 
 
 def grad_launches(n, L, nL=N_LAYERS, H=HIDDEN):
-    """Kernels of one tensor-core gradient call: three packing kernels, then per
-    batch 3 nL forward launches (scan and output map per layer, projections
-    above layer 0, the readout adjoint) and 4 nL - 1 backward launches."""
-    npad = (L + 63) & ~63
-    per = ((nL * 4 * H + 1) * npad + 7 * H * npad) * 4
-    B = max(1, min(n, TC_STASH_BUDGET // per))
-    return 3 + -(-n // B) * (7 * nL - 1)
+    """Kernels of one layer-by-layer gradient call (O_k rows): two packing
+    kernels, then per batch 3 nL - 1 forward launches (projections above layer
+    0, scan, output map), two of the readout and 4 nL - 1 backward launches."""
+    per = ((5 * nL + 2) * H + 1) * L * 4
+    B = max(1, min(n, GRAD_BUDGET // per))
+    return 2 + -(-n // B) * 7 * nL
 
 
 def parse():

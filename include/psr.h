@@ -54,8 +54,8 @@
  * path).  PSR_BF16: the dense projections of layers >= 1 and the output maps
  * run on the tensor cores (tcgen05) with BF16 operands and FP32
  * accumulation; the gates, scan carry, softmax, log-psi sums and every
- * reduction stay in FP32 (hidden = 128 only).  psr_grad always computes in
- * FP32.  PSR_FP16 (FP16 operands, FP32 accumulation) applies to the 2D
+ * reduction stay in FP32 (hidden = 128 only).  psr_grad keeps FP32 values and
+ * results (its products may split FP32 operands into BF16 parts).  PSR_FP16 (FP16 operands, FP32 accumulation) applies to the 2D
  * patched model's forward only (PSR_EUNSUPPORTED elsewhere).
  *
  * Errors.  Every call returns PSR_OK or an error code; nothing traps.
@@ -233,9 +233,12 @@ int psr_context_set_graphs(psr_context *ctx, int enable);
  * dout == NULL: dparams is float [n][P] with row i = O_k(s_i) = d log psi(s_i)
  *   / d theta (per-sample, e.g. for a covariance / SR solve).
  * dout != NULL (float [n]): dparams is float [P] = sum_i dout_i O_k(s_i).
- * The forward is recomputed chunk by chunk from stored chunk-boundary carries
- * and the recurrence is differentiated by a reverse scan
- * lambda_t = dL/dh_t + a_{t+1} lambda_{t+1}.  Computed in FP32. */
+ * Computed layer by layer over batches of samples (up to 2 GiB of workspace), or
+ * chunk by chunk from stored carries where one sample's layers exceed that; the
+ * recurrence is differentiated by a reverse scan
+ * lambda_t = dL/dh_t + a_{t+1} lambda_{t+1}.  FP32 values and accumulation; dense
+ * products at FP32 precision on the tensor cores (split operands: three BF16
+ * parts for sums, two for the O_k rows of the BF16 path) or on CUDA cores. */
 int psr_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_t L,
              const float *dout, float *dparams);
 
@@ -358,7 +361,7 @@ int psr_context_set_autotune(psr_context *ctx, int enable);
  * forwards of E_loc).  precision PSR_BF16: sequences per MMA stream of the
  * tcgen05 kernel, 1 (four streams per SM, MMA N = 32 sites) or 2 (two
  * streams, N = 64: each shared-memory weight slice serves twice the sites);
- * PSR_FP32: scan chunk of the SIMT kernel, 32 or 16 sites.  shape 0 returns
+ * PSR_FP32: window of the SIMT kernel, 32 or 16 sites.  shape 0 returns
  * the choice to the context (the autotuned shape, else the built-in
  * default); any other value fixes it for every later call.  PSR_EINVAL for
  * another shape.  The paper has no counterpart (a tuning choice). */
@@ -427,8 +430,9 @@ int psr2d_sample(const psr_params *params, const float *uniforms, int64_t n, int
 
 /* Gradient of log psi of the 2D model, as psr_grad for the chain model:
  * dout == NULL gives per-sample O_k rows [n][P], otherwise the dout-weighted
- * sum [P].  Rows of patches are recomputed from the forward's row
- * checkpoints and differentiated from the last row to the first, the
+ * sum [P].  Layer by layer over batches, or recomputed from the forward's row
+ * checkpoints where one sample's layers exceed 2 GiB; differentiated from the
+ * last row to the first, the
  * adjoint of each row's states reaching the row above through
  * W_h^T (the h_V columns).  FP32; every hidden size psr2d_logpsi takes. */
 int psr2d_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_t Lx, int32_t Ly,
@@ -504,9 +508,9 @@ int psr_lru_sample(const psr_params *params, const float *uniforms, int64_t n, i
 
 /* Gradient of log psi of the LRU ansatz, as psr_grad for the chain model:
  * dout == NULL gives per-sample O_k rows [n][P] (P = psr_lru_param_count),
- * otherwise the dout-weighted sum [P].  Chunks of 32 sites are recomputed
- * from the forward's complex chunk carries and differentiated from the last
- * to the first; the complex recurrence's adjoint runs backwards as
+ * otherwise the dout-weighted sum [P].  Layer by layer over batches (or chunks
+ * recomputed from the forward's complex carries where one sample's layers exceed
+ * 2 GiB), differentiated from the last site to the first; the complex recurrence's adjoint runs backwards as
  * mu_t = dL/dh_t + conj(lambda) mu_{t+1}.  FP32. */
 int psr_lru_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_t L, const float *dout,
                  float *dparams);
