@@ -436,7 +436,7 @@ int psr_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_t 
              const float *dout, float *dparams) {
     int rc = check_params(params, n, L);
     if (rc != PSR_OK && rc != PSR_EUNSUPPORTED) return rc;
-    if (!spins || !dparams) return PSR_EINVAL;
+    if (!spins || !dparams || n < 1 || L < 1) return PSR_EINVAL;  // PSR_FP16 is refused before the sizes are looked at
     const bool bf16_rows = rc == PSR_OK && grad_bf16_rows(params, dout);
     if (const int64_t B = grad_f32_batch(params->n_layers, params->hidden, L, n)) {
         rc = grad_f32_call(params, spins, n, L, dout, dparams, B, bf16_rows);
