@@ -21,6 +21,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import subprocess
 import sys
 import time
@@ -225,7 +226,8 @@ def profiled_traffic_per_unit(profile="fwd_bf16_connected_52x52.md", src_name="p
     for line in open(path):
         if line.startswith("- ") and ":" in line:
             k, v = line[2:].split(":", 1)
-            vals[k.strip()] = v.strip().strip("`")
+            quoted = re.match(r"\s*`([^`]*)`", v)  # notes may follow a quoted value
+            vals[k.strip()] = quoted.group(1) if quoted else v.strip()
     if vals.get("kernel source sha256/16") != kernel_hash(src_name):
         return None
     try:
