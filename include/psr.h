@@ -229,12 +229,30 @@ int psr_step_batch(const psr_params *params, const psr_step_item *items, int32_t
  * psr_local_energy_batch and psr_step_batch on this context. */
 int psr_context_set_graphs(psr_context *ctx, int enable);
 
+/* Bounds the device memory of this context.  workspace_bytes: the scratch
+ * workspace never exceeds it (a larger one is given back at once, after a wait
+ * for the stream); a call that needs more returns PSR_ENOMEM, gradients first
+ * take smaller batches.  Negative: no bound (the default).  grad_bytes: layer
+ * arrays that one batch of psr_grad, psr_lru_grad, psr2d_grad, the VMC steps and
+ * psr_step_batch may hold; partial sums (up to about half as much again), the
+ * call's other arrays and an eighth of reserve come on top.  A sample that needs
+ * more by itself is differentiated by recomputing chunks (0: every sample).
+ * Negative: 2 GiB (the default).  When the device has no room for a batch, it is
+ * halved until it fits, and later calls on the context start from the size that
+ * did, until this call sets the budget again.  The paper has no counterpart. */
+int psr_context_set_memory(psr_context *ctx, int64_t workspace_bytes, int64_t grad_bytes);
+
+/* Size in bytes of the context's scratch workspace, how often it has been
+ * allocated (a recorded graph is valid for one generation), and the layer arrays
+ * that a gradient's batch may hold now (psr_context_set_memory). */
+int psr_context_workspace(psr_context *ctx, int64_t *bytes, int64_t *generation, int64_t *grad_bytes);
+
 /* Gradient of log psi (Sec. III.B: stochastic energy-gradient estimates).
  * dout == NULL: dparams is float [n][P] with row i = O_k(s_i) = d log psi(s_i)
  *   / d theta (per-sample, e.g. for a covariance / SR solve).
  * dout != NULL (float [n]): dparams is float [P] = sum_i dout_i O_k(s_i).
- * Computed layer by layer over batches of samples (up to 2 GiB of workspace), or
- * chunk by chunk from stored carries where one sample's layers exceed that; the
+ * Computed layer by layer over batches of samples (psr_context_set_memory), or
+ * chunk by chunk from stored carries where one sample's layers exceed the budget; the
  * recurrence is differentiated by a reverse scan
  * lambda_t = dL/dh_t + a_{t+1} lambda_{t+1}.  FP32 values and accumulation; dense
  * products at FP32 precision on the tensor cores (split operands: three BF16
@@ -431,7 +449,7 @@ int psr2d_sample(const psr_params *params, const float *uniforms, int64_t n, int
 /* Gradient of log psi of the 2D model, as psr_grad for the chain model:
  * dout == NULL gives per-sample O_k rows [n][P], otherwise the dout-weighted
  * sum [P].  Layer by layer over batches, or recomputed from the forward's row
- * checkpoints where one sample's layers exceed 2 GiB; differentiated from the
+ * checkpoints where one sample's layers exceed the budget; differentiated from the
  * last row to the first, the
  * adjoint of each row's states reaching the row above through
  * W_h^T (the h_V columns).  FP32; every hidden size psr2d_logpsi takes. */
@@ -510,7 +528,7 @@ int psr_lru_sample(const psr_params *params, const float *uniforms, int64_t n, i
  * dout == NULL gives per-sample O_k rows [n][P] (P = psr_lru_param_count),
  * otherwise the dout-weighted sum [P].  Layer by layer over batches (or chunks
  * recomputed from the forward's complex carries where one sample's layers exceed
- * 2 GiB), differentiated from the last site to the first; the complex recurrence's adjoint runs backwards as
+ * the budget), differentiated from the last site to the first; the complex recurrence's adjoint runs backwards as
  * mu_t = dL/dh_t + conj(lambda) mu_{t+1}.  FP32. */
 int psr_lru_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_t L, const float *dout,
                  float *dparams);

@@ -71,7 +71,7 @@ EXPORTED = ("psr_context_create", "psr_context_destroy", "psr_context_sync", "ps
             "psr_sym_local_energy", "psr_vmc_step", "psr2d_sample", "psr2d_grad", "psr2d_vmc_step",
             "psr_lru_sample", "psr_lru_grad", "psr_lru_vmc_step", "psr2d_sym_logpsi",
             "psr2d_sym_local_energy", "psr_noalloc_status", "psr_step_batch",
-            "psr_context_set_fwd_shape", "psr_fwd_shape_for")
+            "psr_context_set_fwd_shape", "psr_fwd_shape_for", "psr_context_set_memory", "psr_context_workspace")
 STAGES = ("pack", "generator", "fwd_samples", "fwd_connected", "gather", "bwd", "scan", "sample")
 
 _lib = None
@@ -106,6 +106,8 @@ def lib():
                 L.psr_context_set_fwd_shape.argtypes = [vp, i32, i32]
                 L.psr_fwd_shape_for.argtypes = [vp, i32, i32, i32, C.POINTER(i64), C.POINTER(i32),
                                                 C.POINTER(i32), C.POINTER(i32)]
+                L.psr_context_set_memory.argtypes = [vp, i64, i64]
+                L.psr_context_workspace.argtypes = [vp, C.POINTER(i64), C.POINTER(i64), C.POINTER(i64)]
                 L.psr_context_set_graphs.argtypes = [vp, C.c_int]
                 L.psr_context_set_profiling.argtypes = [vp, C.c_int]
                 L.psr_context_stage_ms.argtypes = [vp, C.c_int, C.POINTER(C.c_float)]
@@ -284,6 +286,22 @@ def psr_noalloc_status(stream=None):
 
 def psr_context_set_graphs(ctx, enable=True):
     _check(lib().psr_context_set_graphs(C.c_void_p(ctx), int(bool(enable))), "psr_context_set_graphs")
+
+
+def psr_context_set_memory(ctx, workspace_bytes=-1, grad_bytes=-1):
+    """Bounds the context's workspace and the layer arrays of a gradient's
+    batch (negative: the defaults)."""
+    _check(lib().psr_context_set_memory(C.c_void_p(ctx), int(workspace_bytes), int(grad_bytes)),
+           "psr_context_set_memory")
+
+
+def psr_context_workspace(ctx):
+    """(bytes, generation) of the context's workspace, and the layer arrays that
+    a gradient's batch may hold now."""
+    b, g, a = C.c_int64(), C.c_int64(), C.c_int64()
+    _check(lib().psr_context_workspace(C.c_void_p(ctx), C.byref(b), C.byref(g), C.byref(a)),
+           "psr_context_workspace")
+    return int(b.value), int(g.value), int(a.value)
 
 
 def psr_local_energy_batch(params, items):

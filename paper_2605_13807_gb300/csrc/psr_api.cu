@@ -76,6 +76,28 @@ int psr_context_set_graphs(psr_context *ctx, int enable) {
     return PSR_OK;
 }
 
+int psr_context_set_memory(psr_context *ctx, int64_t workspace_bytes, int64_t grad_bytes) {
+    if (!ctx || ctx->capturing) return PSR_EINVAL;
+    ctx->ws_limit = workspace_bytes < 0 ? SIZE_MAX : (size_t)workspace_bytes;
+    ctx->grad_fit = grad_bytes < 0 ? kGradBudget : (size_t)grad_bytes;
+    ctx->graph_key.clear();  // a recorded step may be of the former batches
+    if (ctx->ws_size > ctx->ws_limit) {
+        PSR_TRY(cudaStreamSynchronize(ctx->stream));
+        cudaFree(ctx->ws);
+        ctx->ws = nullptr;
+        ctx->ws_size = 0;
+    }
+    return PSR_OK;
+}
+
+int psr_context_workspace(psr_context *ctx, int64_t *bytes, int64_t *generation, int64_t *grad_bytes) {
+    if (!ctx || !bytes || !generation || !grad_bytes) return PSR_EINVAL;
+    *bytes = (int64_t)ctx->ws_size;
+    *generation = (int64_t)ctx->ws_generation;
+    *grad_bytes = (int64_t)ctx->grad_fit;
+    return PSR_OK;
+}
+
 int psr_context_destroy(psr_context *ctx) {
     if (!ctx) return PSR_EINVAL;
     int rc = from_cuda(cudaStreamSynchronize(ctx->stream));
@@ -397,12 +419,14 @@ static int grad_f32_call(const psr_params *params, const uint8_t *spins, int64_t
         grad_f32_carve(c, nL, H, L, B, dout != nullptr, d_theta && !aligned16p(params->theta), A);
     };
     int rc = PSR_ENOMEM;
+    const int64_t asked = B;
     for (; B > 0; B /= 2) {
         Carver sz;
         carve(sz);
         if ((rc = ensure_ws(ctx, sz.off)) != PSR_ENOMEM) break;
     }
     if (rc != PSR_OK) return rc;
+    grad_fitted(ctx, grad_f32_floats(nL, H, L), asked, B);
     Carver cv;
     cv.base = static_cast<char *>(ctx->ws);
     carve(cv);
@@ -438,11 +462,12 @@ int psr_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_t 
     if (rc != PSR_OK && rc != PSR_EUNSUPPORTED) return rc;
     if (!spins || !dparams || n < 1 || L < 1) return PSR_EINVAL;  // PSR_FP16 is refused before the sizes are looked at
     const bool bf16_rows = rc == PSR_OK && grad_bf16_rows(params, dout);
-    if (const int64_t B = grad_f32_batch(params->n_layers, params->hidden, L, n)) {
+    psr_context *ctx = params->ctx;
+    const int64_t B = grad_f32_batch(ctx, params->n_layers, params->hidden, L, n);
+    if (B > 0) {
         rc = grad_f32_call(params, spins, n, L, dout, dparams, B, bf16_rows);
         if (rc != PSR_ENOMEM) return rc;
     }
-    psr_context *ctx = params->ctx;
     const int nL = params->n_layers, H = params->hidden;
     const ThetaLayout tl = theta_layout(nL, H);
     const F32Layout fl = f32_layout(nL, H);
@@ -486,6 +511,7 @@ int psr_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_t 
     Carver sz;
     carve(sz);
     if ((rc = ensure_ws(ctx, sz.off)) != PSR_OK) return rc;
+    if (B > 0) grad_fitted(ctx, grad_f32_floats(nL, H, L), B, 0);
     Carver cv;
     cv.base = static_cast<char *>(ctx->ws);
     carve(cv);

@@ -91,7 +91,7 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         for (int i = 0; i < n_items; ++i) {
             w[i].B = 0;
             if (!items[i].grad) continue;
-            if (layers) w[i].B = grad_f32_batch(nL, H, w[i].N, items[i].n);
+            if (layers) w[i].B = grad_f32_batch(ctx, nL, H, w[i].N, items[i].n);
             if (w[i].B == 0) {
                 n_chunk += items[i].n;
                 continue;
@@ -150,7 +150,8 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         }
     };
     // without room for the layers' arrays: smaller batches, then chunks
-    for (int shift = 0;;) {
+    int shift = 0;
+    for (;;) {
         Carver sz;
         carve(sz);
         rc = ensure_ws(ctx, sz.off);
@@ -160,6 +161,17 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
         plan_grad(smaller, ++shift);
     }
     if (rc != PSR_OK) return rc;
+    if (shift > 0) {  // later calls start from what fitted (grad_fitted)
+        size_t fit = 0, none = SIZE_MAX;
+        for (int i = 0; i < n_items; ++i) {
+            if (!items[i].grad || grad_f32_batch(ctx, nL, H, w[i].N, items[i].n) == 0) continue;
+            const size_t bytes = grad_f32_floats(nL, H, w[i].N) * sizeof(float);
+            if (w[i].B > 0 && w[i].B * bytes > fit) fit = w[i].B * bytes;
+            if (bytes - 1 < none) none = bytes - 1;
+        }
+        if (fit == 0) fit = none;
+        if (fit < ctx->grad_fit) ctx->grad_fit = fit;
+    }
     Carver cv;
     cv.base = static_cast<char *>(ctx->ws);
     carve(cv);
@@ -192,7 +204,8 @@ int step_batch_impl(const psr_params *params, const StepItem *items, int n_items
             PSR_TRY(cudaGraphLaunch(ctx->graph_exec, st));
             return PSR_OK;
         }
-        // kernel attributes are set outside the capture
+        // attributes of the persistent kernels; the layered gradients set theirs as
+        // they launch, which a capture allows
         if (bf16) PSR_TRY(prepare_fwd_bf16());
         if (by_chunk) PSR_TRY(prepare_bwd_f32(H, nL));
         PSR_TRY(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));

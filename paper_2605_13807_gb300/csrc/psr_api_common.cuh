@@ -15,6 +15,14 @@
 
 #include "psr_internal.cuh"
 
+namespace psr {
+namespace apiutil {
+// Bytes of layer arrays that a batch of a layered gradient may hold, unless
+// psr_context_set_memory says otherwise.
+constexpr size_t kGradBudget = size_t(2) << 30;
+}  // namespace apiutil
+}  // namespace psr
+
 struct psr_context {
     cudaStream_t stream = nullptr;
     int device = 0;
@@ -28,6 +36,10 @@ struct psr_context {
     cudaEvent_t ev_end[PSR_STAGE_COUNT] = {};
     bool stage_ran[PSR_STAGE_COUNT] = {};
     uint64_t ws_generation = 0;  // bumped whenever the workspace moves
+    size_t ws_limit = SIZE_MAX;  // largest workspace (psr_context_set_memory)
+    // bytes of layer arrays a gradient's batch takes: the budget, or less once
+    // the device had no room for it (grad_fitted)
+    size_t grad_fit = psr::apiutil::kGradBudget;
     bool graphs = false;
     cudaGraphExec_t graph_exec = nullptr;
     std::vector<unsigned char> graph_key;  // arguments the cached graph was built for
@@ -92,11 +104,13 @@ inline bool is_device_ptr(const void *p) {
 
 inline int ensure_ws(psr_context *ctx, size_t bytes) {
     if (bytes <= ctx->ws_size) return PSR_OK;
+    if (bytes > ctx->ws_limit) return PSR_ENOMEM;
     PSR_TRY(cudaStreamSynchronize(ctx->stream));
     if (ctx->ws) cudaFree(ctx->ws);
     ctx->ws = nullptr;
     ctx->ws_size = 0;
     size_t want = bytes + bytes / 8 + (1u << 20);
+    if (want > ctx->ws_limit) want = ctx->ws_limit;
     cudaError_t e = cudaMalloc(&ctx->ws, want);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -316,19 +330,27 @@ inline int tune_fwd_shape(psr_context *ctx, bool bf16, const FwdKey &k, Run run,
 
 // ------------------------------------------------ gradients by layers
 // The layer-by-layer gradients hold every layer's arrays of a batch of
-// samples; batches are sized to kGradBudget bytes of them.  A sample that
+// samples; batches are sized to the context's budget of them.  A sample that
 // needs more by itself goes to the chunk-recompute kernel of its model, which
 // keeps only chunk carries.
-constexpr size_t kGradBudget = size_t(2) << 30;
 
 // Samples per batch for `per` floats of arrays a sample; 0: too long.
-inline int64_t grad_batch(size_t per, int64_t sites, int64_t n) {
+inline int64_t grad_batch(const psr_context *ctx, size_t per, int64_t sites, int64_t n) {
     const size_t bytes = per * sizeof(float);
-    if (bytes > kGradBudget || sites >= (int64_t)1 << 30) return 0;
-    int64_t B = (int64_t)(kGradBudget / bytes);
+    if (bytes > ctx->grad_fit || sites >= (int64_t)1 << 30) return 0;
+    int64_t B = (int64_t)(ctx->grad_fit / bytes);
     const int64_t most = ((int64_t)1 << 30) / sites;
     if (B > most) B = most;
     return B < n ? B : n;
+}
+
+// A batch of `asked` samples found no room, one of `got` did (0: the
+// chunk-recompute kernel).  Later calls start from there: each failed attempt
+// waits for the stream, gives the workspace back and allocates it anew, which
+// also makes psr_step_batch record its graph again.
+inline void grad_fitted(psr_context *ctx, size_t per, int64_t asked, int64_t got) {
+    const size_t fit = got > 0 ? (size_t)got * per * sizeof(float) : per * sizeof(float) - 1;
+    if (got < asked && fit < ctx->grad_fit) ctx->grad_fit = fit;
 }
 
 // How the products of a gradient run.  FP32 sums over samples: three-part split
@@ -347,8 +369,10 @@ inline bool grad_bf16_rows(const psr_params *p, const float *dout) {
 
 inline bool aligned16p(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-inline int64_t grad_f32_batch(int nL, int H, int L, int64_t n) {
-    return grad_batch(grad_f32_floats_per_site(nL, H) * (size_t)L, L, n);
+inline size_t grad_f32_floats(int nL, int H, int L) { return grad_f32_floats_per_site(nL, H) * (size_t)L; }
+
+inline int64_t grad_f32_batch(const psr_context *ctx, int nL, int H, int L, int64_t n) {
+    return grad_batch(ctx, grad_f32_floats(nL, H, L), L, n);
 }
 
 // Carves the batch arrays of launch_grad_f32 into A (sum: a weighted sum over

@@ -231,10 +231,13 @@ int psr2d_sample(const psr_params *params, const float *uniforms, int64_t n, int
     return PSR_OK;
 }
 
-// Samples per batch of the layer-by-layer gradient, 0 if one does not fit.
+// Floats of layer arrays per sample, and samples per batch of the layer-by-layer
+// gradient (0 if one does not fit).
+static size_t grad2d_floats(const psr_params *params, int32_t Lx, int32_t Ly) {
+    return grad2d_floats_per_site(params->n_layers, params->hidden) * (size_t)(Lx / 2) * (size_t)(Ly / 2);
+}
 static int64_t grad2d_batch(const psr_params *params, int64_t n, int32_t Lx, int32_t Ly) {
-    const int64_t Np = (int64_t)(Lx / 2) * (Ly / 2);
-    return grad_batch(grad2d_floats_per_site(params->n_layers, params->hidden) * (size_t)Np, Np, n);
+    return grad_batch(params->ctx, grad2d_floats(params, Lx, Ly), (int64_t)(Lx / 2) * (Ly / 2), n);
 }
 
 // psr2d_grad layer by layer; PSR_ENOMEM if even a batch of one sample finds no
@@ -291,12 +294,14 @@ static int grad2d_layers(const psr_params *params, const uint8_t *spins, int64_t
     };
     if (weights && B < n) return PSR_ENOMEM;
     int rc = PSR_ENOMEM;
+    const int64_t asked = B;
     for (; B > 0; B /= 2) {
         Carver sz;
         carve(sz);
         if ((rc = ensure_ws(ctx, sz.off)) != PSR_ENOMEM || weights) break;
     }
     if (rc != PSR_OK) return rc;
+    grad_fitted(ctx, grad2d_floats(params, Lx, Ly), asked, B);
     Carver cv;
     cv.base = static_cast<char *>(ctx->ws);
     carve(cv);
@@ -345,7 +350,8 @@ int psr2d_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_
     int rc = check_params2d(params, n, Lx, Ly);
     if (rc != PSR_OK) return rc;
     if (!spins || !dparams) return PSR_EINVAL;
-    if (const int64_t B = grad2d_batch(params, n, Lx, Ly)) {
+    const int64_t B = grad2d_batch(params, n, Lx, Ly);
+    if (B > 0) {
         rc = grad2d_layers(params, spins, n, Lx, Ly, dout, dparams, B, nullptr, nullptr);
         if (rc != PSR_ENOMEM) return rc;
     }
@@ -387,6 +393,7 @@ int psr2d_grad(const psr_params *params, const uint8_t *spins, int64_t n, int32_
     Carver sz;
     carve(sz);
     if ((rc = ensure_ws(ctx, sz.off)) != PSR_OK) return rc;
+    if (B > 0) grad_fitted(ctx, grad2d_floats(params, Lx, Ly), B, 0);
     Carver cv;
     cv.base = static_cast<char *>(ctx->ws);
     carve(cv);
@@ -1062,12 +1069,14 @@ static int lru_grad_layers(const psr_params *params, const uint8_t *spins, int64
         A.small = c.get<float>(dout ? (size_t)B * small_floats : 0);
     };
     int rc = PSR_ENOMEM;
+    const int64_t asked = B;
     for (; B > 0; B /= 2) {
         Carver sz;
         carve(sz);
         if ((rc = ensure_ws(ctx, sz.off)) != PSR_ENOMEM) break;
     }
     if (rc != PSR_OK) return rc;
+    grad_fitted(ctx, grad_lru_floats_per_site(nL, H) * (size_t)N, asked, B);
     Carver cv;
     cv.base = static_cast<char *>(ctx->ws);
     carve(cv);
@@ -1115,7 +1124,8 @@ int psr_lru_grad(const psr_params *params, const uint8_t *spins, int64_t n, int3
     if (rc != PSR_OK) return rc;
     if (!spins || !dparams) return PSR_EINVAL;
     const size_t per = grad_lru_floats_per_site(params->n_layers, params->hidden) * (size_t)L;
-    if (const int64_t B = grad_batch(per, L, n)) {
+    const int64_t B = grad_batch(params->ctx, per, L, n);
+    if (B > 0) {
         rc = lru_grad_layers(params, spins, n, L, dout, dparams, B);
         if (rc != PSR_ENOMEM) return rc;
     }
@@ -1157,6 +1167,7 @@ int psr_lru_grad(const psr_params *params, const uint8_t *spins, int64_t n, int3
     Carver sz;
     carve(sz);
     if ((rc = ensure_ws(ctx, sz.off)) != PSR_OK) return rc;
+    if (B > 0) grad_fitted(ctx, per, B, 0);
     Carver cv;
     cv.base = static_cast<char *>(ctx->ws);
     carve(cv);
