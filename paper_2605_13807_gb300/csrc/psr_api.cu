@@ -440,8 +440,7 @@ static int grad_f32_call(const psr_params *params, const uint8_t *spins, int64_t
     reset_stages(ctx);
     {
         StageScope sc(ctx, PSR_STAGE_PACK);
-        PSR_TRY(launch_pack_theta_f32(theta, tl, fl, pk, st));
-        PSR_TRY(launch_bitpack(sp, n, L, W, bits, ctx->status, st));
+        PSR_TRY(launch_pack_f32_bits(theta, tl, fl, pk, sp, n, L, W, bits, ctx->status, st));
     }
     {
         StageScope sc(ctx, PSR_STAGE_BWD);  // the layers' forward and the reverse pass

@@ -393,8 +393,8 @@ inline void grad_f32_carve(Carver &c, int nL, int H, int L, int64_t B, bool sum,
     A.gh = c.get<float>(arr);
     A.dc = c.get<float>(arr);
     A.g = c.get<float>(M);
-    const size_t range = grad_f32_range(H);
-    A.rows = c.get<float>(sum ? (M + range - 1) / range * P : 0);
+    A.range = grad_f32_range(H, M);
+    A.rows = c.get<float>(sum ? (M + A.range - 1) / A.range * P : 0);
     A.small = c.get<float>(sum ? (size_t)B * grad_f32_small_floats(H) : 0);
 }
 

@@ -289,8 +289,8 @@ static int grad2d_layers(const psr_params *params, const uint8_t *spins, int64_t
         A.logp = c.get<float>(M);
         A.wo32 = c.get<float>(32 * (size_t)H);
         A.wo32t = c.get<float>(32 * (size_t)H);
-        const size_t range = grad_f32_range(H);
-        A.rows = c.get<float>(dout ? (M + range - 1) / range * P : 0);
+        A.range = grad_f32_range(H, M);
+        A.rows = c.get<float>(dout ? (M + A.range - 1) / A.range * P : 0);
     };
     if (weights && B < n) return PSR_ENOMEM;
     int rc = PSR_ENOMEM;
@@ -1064,8 +1064,8 @@ static int lru_grad_layers(const psr_params *params, const uint8_t *spins, int64
         float **adj[] = {&A.gx, &A.da, &A.dg, &A.dy, &A.dhr, &A.dhi};
         for (float **p : adj) *p = c.get<float>(arr);
         A.g = c.get<float>(M);
-        const size_t range = grad_f32_range(H);
-        A.rows = c.get<float>(dout ? (M + range - 1) / range * P : 0);
+        A.range = grad_f32_range(H, M);
+        A.rows = c.get<float>(dout ? (M + A.range - 1) / A.range * P : 0);
         A.small = c.get<float>(dout ? (size_t)B * small_floats : 0);
     };
     int rc = PSR_ENOMEM;

@@ -70,10 +70,9 @@ F32Layout f32_layout(int nL, int H) {
 // One thread per packed element, so that every read of theta is in flight at
 // once (a loop over layers and tensors paid the latency of each: 9 us at any
 // width, 3 us so).
-__global__ void __launch_bounds__(256) pack_f32_kernel(const float *__restrict__ theta, ThetaLayout tl, F32Layout fl,
-                                                       float *__restrict__ pk) {
+__device__ __forceinline__ void pack_f32_element(const float *__restrict__ theta, const ThetaLayout &tl,
+                                                 const F32Layout &fl, float *__restrict__ pk, int i) {
     const int H = tl.H;
-    const int i = blockIdx.x * 256 + threadIdx.x;
     if (i >= fl.total) return;
     // tensors of a layer in packed order; the tables and readout follow
     if (i < fl.A0) {
@@ -116,6 +115,11 @@ __global__ void __launch_bounds__(256) pack_f32_kernel(const float *__restrict__
     }
 }
 
+__global__ void __launch_bounds__(256) pack_f32_kernel(const float *__restrict__ theta, ThetaLayout tl, F32Layout fl,
+                                                       float *__restrict__ pk) {
+    pack_f32_element(theta, tl, fl, pk, blockIdx.x * 256 + threadIdx.x);
+}
+
 cudaError_t launch_pack_theta_f32(const float *theta, const ThetaLayout &tl, const F32Layout &fl,
                                   float *packed, cudaStream_t stream) {
     pack_f32_kernel<<<(unsigned)((fl.total + 255) / 256), 256, 0, stream>>>(theta, tl, fl, packed);
@@ -126,13 +130,13 @@ cudaError_t launch_pack_theta_f32(const float *theta, const ThetaLayout &tl, con
 // than 0/1 is reported as PSR_EDEVICE and treated as its lowest bit.  Words past
 // N are zero.  The first thread also zeroes n_zero counters for a kernel that
 // follows (a launch less than a memset).
-__global__ void __launch_bounds__(256) bitpack_kernel(const uint8_t *__restrict__ spins, int64_t n, int N, int W,
-                                                      uint64_t *__restrict__ bits, int *status,
-                                                      unsigned long long *zero, int n_zero) {
+__device__ __forceinline__ void bitpack_words(const uint8_t *__restrict__ spins, int64_t n, int N, int W,
+                                              uint64_t *__restrict__ bits, int *status, unsigned long long *zero,
+                                              int n_zero, int block, int blocks) {
     const int lane = threadIdx.x & 31;
-    if (blockIdx.x == 0 && threadIdx.x < n_zero) zero[threadIdx.x] = 0;
-    const int64_t total = n * W, warps = (int64_t)gridDim.x * 8;
-    for (int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); i < total; i += warps) {
+    if (block == 0 && threadIdx.x < n_zero) zero[threadIdx.x] = 0;
+    const int64_t total = n * W, warps = (int64_t)blocks * 8;
+    for (int64_t i = (int64_t)block * 8 + (threadIdx.x >> 5); i < total; i += warps) {
         const int64_t s = i / W;
         const int t = (int)(i - s * W) * 64 + lane;
         const uint8_t *row = spins + s * N;
@@ -143,11 +147,40 @@ __global__ void __launch_bounds__(256) bitpack_kernel(const uint8_t *__restrict_
     }
 }
 
+__global__ void __launch_bounds__(256) bitpack_kernel(const uint8_t *__restrict__ spins, int64_t n, int N, int W,
+                                                      uint64_t *__restrict__ bits, int *status,
+                                                      unsigned long long *zero, int n_zero) {
+    bitpack_words(spins, n, N, W, bits, status, zero, n_zero, blockIdx.x, gridDim.x);
+}
+
+static int bitpack_blocks(int64_t n, int W) {
+    const int64_t blocks = (n * W + 7) / 8;
+    return (int)(blocks > 65535 ? 65535 : blocks);
+}
+
 cudaError_t launch_bitpack(const uint8_t *spins, int64_t n, int N, int W, uint64_t *bits,
                            int *status, cudaStream_t stream, unsigned long long *zero, int n_zero) {
-    int64_t blocks = (n * W + 7) / 8;
-    if (blocks > 65535) blocks = 65535;
-    bitpack_kernel<<<(unsigned)blocks, 256, 0, stream>>>(spins, n, N, W, bits, status, zero, n_zero);
+    bitpack_kernel<<<bitpack_blocks(n, W), 256, 0, stream>>>(spins, n, N, W, bits, status, zero, n_zero);
+    return cudaGetLastError();
+}
+
+// Both packings in one launch: the first blocks take the parameters, the others
+// the spins.  A small gradient is a row of launches of about 4 us, whatever they do.
+__global__ void __launch_bounds__(256) pack_f32_bits_kernel(const float *__restrict__ theta, ThetaLayout tl,
+                                                            F32Layout fl, float *__restrict__ pk, int theta_blocks,
+                                                            const uint8_t *__restrict__ spins, int64_t n, int N, int W,
+                                                            uint64_t *__restrict__ bits, int *status) {
+    const int b = (int)blockIdx.x - theta_blocks;
+    if (b < 0) pack_f32_element(theta, tl, fl, pk, blockIdx.x * 256 + threadIdx.x);
+    else bitpack_words(spins, n, N, W, bits, status, nullptr, 0, b, gridDim.x - theta_blocks);
+}
+
+cudaError_t launch_pack_f32_bits(const float *theta, const ThetaLayout &tl, const F32Layout &fl, float *packed,
+                                 const uint8_t *spins, int64_t n, int N, int W, uint64_t *bits, int *status,
+                                 cudaStream_t stream) {
+    const int tb = (int)((fl.total + 255) / 256);
+    pack_f32_bits_kernel<<<tb + bitpack_blocks(n, W), 256, 0, stream>>>(theta, tl, fl, packed, tb, spins, n, N, W, bits,
+                                                                       status);
     return cudaGetLastError();
 }
 

@@ -220,10 +220,106 @@ inline cudaError_t launch_bn(const Args &g, const Epi &epi, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// units: 32, 64 or a multiple of 128 (32 pairs make a 64-column tile)
+// The same products on tiles of 32 sites x 32 columns (16 pairs), 2 x 4 outputs
+// a thread.  A product of few sites is one wave of tiles, and its time is one
+// tile's latency: the wide tile does 64 multiply-adds a thread for 16 floats
+// read, this one 8 for 6 (a chain of 3 x 128 inner elements: 53 us wide, 10 us
+// so).  Every output is the same chain of multiply-adds over the inner index,
+// so both give the same bits, whatever the number of sites.
+constexpr int SB = 32;       // sites and columns of a tile
+constexpr int SStages = 4;   // cp.async ring
 template <bool kPair, class Epi>
-inline cudaError_t launch(const Args &g, const Epi &epi, cudaStream_t st) {
+__global__ void __launch_bounds__(128) gemm_small_kernel(const __grid_constant__ Args g, const __grid_constant__ Epi epi) {
+    constexpr int C = kPair ? SB / 2 : SB;  // units of the tile
+    __shared__ __align__(16) float ring[SStages * 2 * SB * LDT];
+    const int tid = threadIdx.x, tx = tid & 7, ty = tid >> 3;
+    const int nblk = g.units / C;
+    const int m0 = (int)(blockIdx.x / nblk) * SB, u0 = (int)(blockIdx.x % nblk) * C;
+    const int lcol = tx * 4;
+
+    int s_next = 0, k_next = 0;  // the stage to be requested next
+    auto request = [&](int slot) {
+        if (s_next < g.n_seg) {
+            const Seg &s = g.seg[s_next];
+            float *as = ring + (size_t)slot * 2 * SB * LDT, *ws = as + SB * LDT;
+#pragma unroll
+            for (int r = ty; r < SB; r += 16) {
+                const int m = min(m0 + r, g.M - 1);  // rows past the end repeat the last (not stored)
+                cp16(as + r * LDT + lcol, s.A + (size_t)m * s.lda + k_next + lcol);
+                const float *w = !kPair || r < C ? s.W0 + (size_t)(u0 + r) * s.ldw : s.W1 + (size_t)(u0 + r - C) * s.ldw1;
+                cp16(ws + r * LDT + lcol, w + k_next + lcol);
+            }
+            k_next += BK;
+            if (k_next >= s.K) {
+                k_next = 0;
+                ++s_next;
+            }
+        }
+        cp_commit();
+    };
+    int stages = 0;
+    for (int s = 0; s < g.n_seg; ++s) stages += g.seg[s].K / BK;
+#pragma unroll
+    for (int st = 0; st < SStages - 1; ++st) request(st);
+    float acc[2][4] = {};
+    for (int st = 0; st < stages; ++st) {
+        cp_wait<SStages - 2>();
+        __syncthreads();  // this stage has landed, and the slot requested next has been read
+        request((st + SStages - 1) % SStages);
+        const float *as = ring + (size_t)(st % SStages) * 2 * SB * LDT + ty * LDT;
+        const float *ws = ring + (size_t)(st % SStages) * 2 * SB * LDT + (SB + tx) * LDT;
+#pragma unroll
+        for (int k = 0; k < BK; k += 4) {
+            float4 a[2], b[4];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) a[i] = *reinterpret_cast<const float4 *>(as + 16 * i * LDT + k);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4 *>(ws + 8 * j * LDT + k);
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
+                    acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
+                }
+        }
+    }
+    __syncthreads();  // the ring has been read: the tile goes through it, as in gemm_kernel
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ring[(ty + 16 * i) * LDT + tx + 8 * j] = acc[i][j];
+    __syncthreads();
+    constexpr int kQuads = C / 4, kStep = 128 / kQuads;
+    const int q = (tid % kQuads) * 4, u = u0 + q;
+#pragma unroll
+    for (int r = tid / kQuads; r < SB; r += kStep) {
+        const int m = m0 + r;
+        if (m >= g.M) break;
+        const typename Epi::In in = epi.load(m, u);
+        const float4 v = *reinterpret_cast<const float4 *>(ring + r * LDT + q);
+        if constexpr (kPair) epi.store(m, u, v, *reinterpret_cast<const float4 *>(ring + r * LDT + C + q), in);
+        else epi.store(m, u, v, in);
+    }
+}
+
+// units: 32, 64 or a multiple of 128 (32 pairs make a 64-column tile).
+// The small tile while the wide ones would not fill two thirds of the SMs: at
+// 32, 64 and 96 wide tiles it takes 0.42 to 0.91, 0.64 to 0.95 and 0.70 to 1.09
+// of the wide form's time (32 to 128 columns, 32 to 384 inner elements), at 128
+// tiles 0.83 to 1.17, at 256 up to 1.24.  O_k rows of 64 samples of 16 sites,
+// hidden 32 / 64 / 128: 131 / 200 / 395 us wide, 109 / 121 / 163 us small.
+template <bool kPair, class Epi>
+inline cudaError_t launch(const Args &g, const Epi &epi, int num_sms, cudaStream_t st) {
     const int cols = g.units * (kPair ? 2 : 1);
+    const int BN = cols % 128 == 0 ? 128 : cols % 64 == 0 ? 64 : 32;
+    if (cols % SB == 0 && 3 * ((int64_t)(g.M + BM - 1) / BM) * (cols / BN) <= 2 * (int64_t)num_sms) {
+        const unsigned blocks = (unsigned)((g.M + SB - 1) / SB) * (unsigned)(cols / SB);
+        gemm_small_kernel<kPair, Epi><<<blocks, 128, 0, st>>>(g, epi);
+        return cudaGetLastError();
+    }
     if (cols % 128 == 0) return launch_bn<128, kPair>(g, epi, st);
     if (cols % 64 == 0) return launch_bn<64, kPair>(g, epi, st);
     if constexpr (!kPair) {

@@ -270,7 +270,7 @@ inline cudaError_t launch(const Args &g, const Epi &epi, const Engine &en, cudaS
     if (en.split == 2 && cols % 64 == 0) return launch_tc<2, 64, kPair>(g, epi, en, st);
     if (en.split == 3 && cols % 128 == 0) return launch_tc<3, 128, kPair>(g, epi, en, st);
     if (en.split == 3 && cols % 64 == 0) return launch_tc<3, 64, kPair>(g, epi, en, st);
-    return launch<kPair>(g, epi, st);
+    return launch<kPair>(g, epi, en.num_sms, st);
 }
 
 // Weight gradients on the tensor cores: out[j][k] = sum_m A[m][j] B[m][k] over

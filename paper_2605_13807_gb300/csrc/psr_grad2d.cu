@@ -329,9 +329,8 @@ cudaError_t launch_grad2d_bwd(const Grad2dArgs &A, cudaStream_t st) {
     cudaError_t e;
     WgArgs w0{};  // ranges of the weight gradients: a sample, or a few hundred sites
     if (A.sum_out) {
-        const int range = grad_f32_range(H);
-        w0.n_range = (M + range - 1) / range;
-        w0.len = w0.step = w0.seg_len = w0.seg_stride = range;
+        w0.n_range = (M + A.range - 1) / A.range;
+        w0.len = w0.step = w0.seg_len = w0.seg_stride = A.range;
     } else {
         w0.n_range = A.n;
         w0.len = Px * Py;

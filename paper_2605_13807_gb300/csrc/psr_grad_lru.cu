@@ -359,7 +359,7 @@ cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t st) {
                          A.small + A.sm.Wo, A.small + A.sm.bo, A.small_stride};
     if ((e = launch_readout(ro, TopGlu{A.p1[top], A.p2[top], A.gx, A.da, A.dg}, st))) return e;
     // ------------------------------------------------ backward, top down
-    const int range = A.sum_out ? grad_f32_range(H) : A.N;
+    const int range = A.sum_out ? A.range : A.N;
     const int n_range = A.sum_out ? (M + range - 1) / range : A.n;
     for (int l = top; l >= 0; --l) {
         const float *u = l ? A.x[l - 1] : nullptr;

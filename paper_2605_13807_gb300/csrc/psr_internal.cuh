@@ -93,6 +93,10 @@ cudaError_t launch_pack_theta_f32(const float *theta, const ThetaLayout &tl, con
 // zero: n_zero (at most 256) counters set to 0 as well, or null.
 cudaError_t launch_bitpack(const uint8_t *spins, int64_t n, int N, int W, uint64_t *bits, int *status,
                            cudaStream_t stream, unsigned long long *zero = nullptr, int n_zero = 0);
+// launch_pack_theta_f32 and launch_bitpack in one launch.
+cudaError_t launch_pack_f32_bits(const float *theta, const ThetaLayout &tl, const F32Layout &fl, float *packed,
+                                 const uint8_t *spins, int64_t n, int N, int W, uint64_t *bits, int *status,
+                                 cudaStream_t stream);
 // chunk: sites of a window, kChunkF32 or kChunkGrad.  The carries are stored
 // every kChunkGrad sites for both, on boundaries counted from the end of the
 // sequence (align_start: from its start, as launch_bwd_f32 wants them).
@@ -390,7 +394,7 @@ cudaError_t launch_adam(const float *theta, const float *grad, int64_t P, float 
 // (turns into dz), dc; readout adjoint g [n * N].
 // rows: [n][P] O_k rows with small = rows, small_stride = P and sm the
 // tensors' places in theta (sum_out == NULL), or partial rows
-// [ceil(n N / grad_f32_range)][P] and per-sample entries small
+// [ceil(n N / range)][P] and per-sample entries small
 // [n][grad_f32_small_floats], summed into sum_out [P] (added to it if add).
 namespace gemm {
 // How the products of a gradient run: split 0 on CUDA cores, 2 or 3 on the
@@ -419,8 +423,10 @@ struct GradF32Args {
     GradSmall sm;
     float *sum_out;
     bool add;
+    int range;  // sites of a partial row
 };
-int grad_f32_range(int H);
+// Sites per partial sum of the weight gradients, for a batch of `sites`.
+int grad_f32_range(int H, int64_t sites);
 size_t grad_f32_floats_per_site(int nL, int H);
 int64_t grad_f32_small_floats(int H);
 cudaError_t launch_grad_f32(const GradF32Args &A, cudaStream_t stream);
@@ -449,6 +455,7 @@ struct GradLruArgs {
     GradLruSmall sm;
     float *sum_out;
     bool add;
+    int range;  // sites of a partial row
 };
 size_t grad_lru_floats_per_site(int nL, int H);
 GradLruSmall grad_lru_small(int nL, int H, int64_t *floats);
@@ -459,7 +466,7 @@ cudaError_t launch_grad_lru(const GradLruArgs &A, cudaStream_t stream);
 // layer gate a, candidate c, state h, GELU' dy, output x [M][H]; u0 [M][32]
 // one-hot inputs; logits, g [M][32], logp [M]; adjoints gy (two layers), gh, dc;
 // wo32, wo32t [32 H].  theta 16-byte aligned.  rows: [n][P] O_k rows, or
-// partial rows [ceil(M / grad_f32_range)][P] summed into sum_out [P] (added to
+// partial rows [ceil(M / range)][P] summed into sum_out [P] (added to
 // it if add).  launch_grad2d_fwd writes log psi [n] if asked; dout is read by
 // launch_grad2d_bwd only.
 struct Grad2dArgs {
@@ -476,6 +483,7 @@ struct Grad2dArgs {
     float *rows;
     float *sum_out;
     bool add;
+    int range;  // sites of a partial row
 };
 size_t grad2d_floats_per_site(int nL, int H);
 cudaError_t launch_grad2d_fwd(const Grad2dArgs &A, float *logpsi, cudaStream_t stream);
