@@ -15,7 +15,11 @@ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 // kernel, no chunk read twice) unless there are too few of them to keep the
 // SMs' memory pipes full AND the sequence is long: a lone warp walks about 65
 // sites per us (8 x 2704 x 32: 50 us whole, 26 us in look-back chunks of
-// 256; 64 x 700 x 64, 128 columns: 16 us whole, 38 us in chunks).  Many
+// 256; 64 x 700 x 64, 128 columns: 16 us whole, 38 us in chunks).  The lines:
+// 64 columns (16 x 2704 x 128: 49 us whole, 69 us in chunks; of 65536 sites: 1.07
+// against 1.82 ms); below them 1024 sites (4, 16 and 60 columns: 20.5 to 21.3 us
+// whole, 21 to 34 us in chunks), with up to three columns 896 (1000 sites: 20.5 us
+// whole, 19.0 to 19.6 us in chunks; 896: 18.5 us whole, 18.8 to 19.1 in chunks).  Many
 // short columns take the 128-unit block, whose rows are 512 bytes (16384 x
 // 100 x 128: 369 us against 401 us; from 256 sites on the two are equal).
 // Otherwise (H not a multiple of 32, or few long columns): the widest unit
@@ -24,7 +28,8 @@ bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) ==
 psr_scan_tile scan_default_tile(const psr_context *ctx, int64_t n, int N, int H) {
     const int64_t resident = (int64_t)ctx->num_sms * 32;  // warps at 4 CTAs of 8 warps per SM
     if (H % 128 == 0 && N < 256 && n * (H / 128) >= resident) return psr_scan_tile{128, N};
-    if (H % 32 == 0 && (n * (H / 32) >= 64 || N <= 1024)) return psr_scan_tile{32, N};
+    const int64_t whole = n * (H / 32);  // columns
+    if (H % 32 == 0 && (whole >= 64 || N <= (whole < 4 ? 896 : 1024))) return psr_scan_tile{32, N};
     int units = 4;
     const int widths[4] = {128, 32, 16, 4};
     for (int w : widths)
