@@ -243,6 +243,9 @@ __global__ void __launch_bounds__(256, 2)
         }
         __syncthreads();  // the tile is free for the next stage
     }
+    // after a wait that ran out, MMAs may still be reading the tiles: wait once
+    // more (bounded too) before the tensor memory is given back
+    if (B.abort_flag) tc::mbar_wait(bar, phase ^ 1u);
     tc::tc_before();
     __syncthreads();
     if (warp == 0) {
@@ -444,6 +447,9 @@ __global__ void __launch_bounds__(256, 2) wgrad_tc_kernel(const __grid_constant_
         }
         __syncthreads();
     }
+    // after a wait that ran out, MMAs may still be reading the tiles: wait once
+    // more (bounded too) before the tensor memory is given back
+    if (B.abort_flag) tc::mbar_wait(bar, phase ^ 1u);
     tc::tc_before();
     __syncthreads();
     if (warp == 0) {
