@@ -372,8 +372,8 @@ fwd_bf16_kernel1(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__
     const int warp = tid >> 5;
     const int lane = tid & 31;
     const int lane_base = (warp & 3) * 32;
-    // one MMA-issuing thread per stream, each on its own SM sub-partition
-    // (lane 0 of warp s of the stream's warpgroup)
+    // the thread that fetches the stream's jobs (lane 0 of warp s of its warpgroup,
+    // the warp that issues its MMAs, each stream's on its own SM sub-partition)
     const bool issuer = (j == 32 * s);
     // the warp that issues the stream's MMAs, and its stream, as warp-uniform values
     // (elect1): a stream alternates between its MMAs and its epilogue, so the
@@ -701,8 +701,7 @@ fwd_bf16_kernel(const __grid_constant__ FwdJobs jb, const uint8_t *__restrict__ 
     const int warp = tid >> 5;
     const int lane = tid & 31;
     const int lane_base = (warp & 3) * 32;
-    // one MMA-issuing thread per stream, each on its own SM sub-partition
-    const bool issuer = (half == 0) && (j == 32 * s);
+    // one MMA-issuing warp per stream, each on its own SM sub-partition
     const int wu = __shfl_sync(0xffffffffu, tid >> 5, 0), su = wu / (4 * HALVES);
     const bool iw = wu == (4 * HALVES + 1) * su;  // as in fwd_bf16_kernel1
     const bool leader = (j == 0);    // per warpgroup: job fetch, sums, output

@@ -185,15 +185,15 @@ cudaError_t launch_pack_f32_bits(const float *theta, const ThetaLayout &tl, cons
 }
 
 // ------------------------------------------------------------- forward
-// A job is one sequence; the threads of its CTA own U units each (units j, j +
-// H / U, ...) and walk it in windows of 32 or 16 sites (CW).
+// A job is one sequence; the threads of its CTA own one unit each and walk it in
+// windows of 32 or 16 sites (CW).
 //
 // What bounds it: shared memory and the FP32 rate, about equally.  A thread
 // keeps CW sums of both gates, so a row of the window (CW / 4 16-byte
 // broadcasts) and two weights serve 2 CW multiply-adds, done in pairs of sites
 // (fma.rn.f32x2, half the instructions).  A job's CTA is one warp per 32 units;
-// seven jobs per SM overlap.  Two units a thread halve the shared-memory reads
-// but leave half the warps: 7.8 ms against 6.7 ms at hidden 64, 2 to 4 % better
+// seven jobs per SM overlap.  Two units a thread (measured, not kept) halve the
+// shared-memory reads but leave half the warps: 7.8 ms against 6.7 ms at hidden 64, 2 to 4 % better
 // to twice as slow at hidden 128 (few long sequences).
 // Measured (E_loc of the 100-site periodic Heisenberg chain, hidden 64, 1024
 // samples): 6.7 ms; 12.0 ms with 32-site windows counted from site 0, plain
@@ -247,47 +247,39 @@ struct FwdF32Job {
     int N, u1, p, q;
 };
 
-template <int H>
-struct FwdF32Shape {
-    static constexpr int U = 1;                // units a thread
-    static constexpr int T = H / U;            // threads a job
-    static constexpr int LD = 36;              // row of a tile: 32 sites, 16-byte aligned
-};
+constexpr int LD = 36;  // row of a tile: 32 sites, 16-byte aligned
 
-template <int T>
+// a job is one CTA of H threads
+template <int H>
 __device__ __forceinline__ void job_sync() {
-    if constexpr (T == 32) __syncwarp();
+    if constexpr (H == 32) __syncwarp();
     else __syncthreads();
 }
 
-// y[r] += w[k][unit r] x[k] over a window's row pairs, k = 0 .. H - 1, for NM
-// (weights, tile, sums) triples at once; the weights (coalesced over units) of
-// the next K inner units are fetched while K are used.
-template <int H, int CW, int U, int NM>
+// y += w[k][this thread's unit] x[k] over a window's pairs of sites, k = 0 .. H - 1,
+// for NM (weights, tile, sums) triples at once; the weights (coalesced over units)
+// of the next K inner units are fetched while K are used.
+template <int H, int CW, int NM>
 __device__ __forceinline__ void products(const float *const (&w)[NM], const float *const (&tile)[NM],
-                                         uint64_t (*const (&y)[NM])[CW / 2]) {
-    constexpr int T = H / U, LD = FwdF32Shape<H>::LD, P = CW / 2;
+                                         uint64_t *const (&y)[NM]) {
+    constexpr int P = CW / 2;
     // K = 4 leaves the code of the narrow model small enough for jobs out of step
     constexpr int K = H == 32 ? 4 : 8;
-    float nw[NM][K][U];
+    float nw[NM][K];
     auto fetch = [&](int k0) {
 #pragma unroll
         for (int m = 0; m < NM; ++m)
 #pragma unroll
-            for (int k = 0; k < K; ++k)
-#pragma unroll
-                for (int r = 0; r < U; ++r) nw[m][k][r] = w[m][(k0 + k) * H + r * T];
+            for (int k = 0; k < K; ++k) nw[m][k] = w[m][(k0 + k) * H];
     };
     fetch(0);
 #pragma unroll 1
     for (int k0 = 0; k0 < H; k0 += K) {
-        uint64_t cw[NM][K][U];
+        uint64_t cw[NM][K];
 #pragma unroll
         for (int m = 0; m < NM; ++m)
 #pragma unroll
-            for (int k = 0; k < K; ++k)
-#pragma unroll
-                for (int r = 0; r < U; ++r) cw[m][k][r] = pack2(nw[m][k][r], nw[m][k][r]);
+            for (int k = 0; k < K; ++k) cw[m][k] = pack2(nw[m][k], nw[m][k]);
         if (k0 + K < H) fetch(k0 + K);
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -298,11 +290,8 @@ __device__ __forceinline__ void products(const float *const (&w)[NM], const floa
                 for (int m = 0; m < NM; ++m) {
                     if (m == 0 || tile[m] != tile[0])
                         v = *reinterpret_cast<const ulonglong2 *>(tile[m] + (k0 + k) * LD + 4 * q);
-#pragma unroll
-                    for (int r = 0; r < U; ++r) {
-                        ffma2(y[m][r][2 * q], cw[m][k][r], v.x);
-                        ffma2(y[m][r][2 * q + 1], cw[m][k][r], v.y);
-                    }
+                    ffma2(y[m][2 * q], cw[m][k], v.x);
+                    ffma2(y[m][2 * q + 1], cw[m][k], v.y);
                 }
             }
         }
@@ -315,40 +304,38 @@ template <int H, int CW>
 __device__ __forceinline__ float window(const FwdF32Job &J, const float *__restrict__ pk, const F32Layout &fl,
                                         float *xs, float *hs, float *zs, float *hcar, int t0, int c,
                                         int &n_up) {
-    constexpr int U = FwdF32Shape<H>::U, T = FwdF32Shape<H>::T, LD = FwdF32Shape<H>::LD, P = CW / 2;
-    const int j = threadIdx.x, nL = fl.nL;
+    constexpr int P = CW / 2;
+    const int j = threadIdx.x, nL = fl.nL;  // j: this thread's unit
     uint32_t cur, prev;
     window_bits(J.row, J.N, t0, J.p, J.q, cur, prev);
     if (CW < 32) cur &= (1u << CW) - 1u;
     const uint32_t prevbits = (cur << 1) | prev;  // bit t = s_{t0+t-1}
     const int first = max(0, -t0);                // sites before the sequence: no input, no state
 
-    uint64_t y[U][P];
-    // scan of one unit: h_t from a_t and c_t (or b_t), written to its row of
+    uint64_t y[P];
+    // scan of the unit: h_t from a_t and c_t (or b_t), written to its row of
     // hs; y starts from the unit's old row (the layer below's states) if kept
-    auto put_carry = [&](int l, int u, int chunk, float h) {
-        if (J.carries) J.carries[((int64_t)chunk * nL + l) * H + u] = h;
+    auto put_carry = [&](int l, int chunk, float h) {
+        if (J.carries) J.carries[((int64_t)chunk * nL + l) * H + j] = h;
     };
     // ---------------- layer 0: gates by lookup of the one-hot input
-#pragma unroll
-    for (int r = 0; r < U; ++r) {
-        const int u = j + r * T;
+    {
         float a[3], b[3], d[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            a[q] = pk[fl.A0 + q * H + u];
-            b[q] = pk[fl.B0 + q * H + u];
-            d[q] = pk[fl.DU0 + q * H + u];
+            a[q] = pk[fl.A0 + q * H + j];
+            b[q] = pk[fl.B0 + q * H + j];
+            d[q] = pk[fl.DU0 + q * H + j];
         }
-        float h = hcar[u];
-        put_carry(0, u, c, h);
+        float h = hcar[j];
+        put_carry(0, c, h);
 #pragma unroll
         for (int t = 0; t < CW; t += 4) {
             float hv[4], dv[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int tt = t + e;
-                if (CW == 32 && tt == 16) put_carry(0, u, c + 1, h);
+                if (CW == 32 && tt == 16) put_carry(0, c + 1, h);
                 const bool up = (prevbits >> tt) & 1u;
                 const bool start = t0 + tt == 0;
                 const float hn = (start ? a[0] : up ? a[2] : a[1]) * h + (start ? b[0] : up ? b[2] : b[1]);
@@ -356,90 +343,82 @@ __device__ __forceinline__ float window(const FwdF32Job &J, const float *__restr
                 hv[e] = h;
                 dv[e] = start ? d[0] : up ? d[2] : d[1];
             }
-            *reinterpret_cast<float4 *>(hs + u * LD + t) = make_float4(hv[0], hv[1], hv[2], hv[3]);
-            y[r][t / 2] = pack2(dv[0], dv[1]);
-            y[r][t / 2 + 1] = pack2(dv[2], dv[3]);
+            *reinterpret_cast<float4 *>(hs + j * LD + t) = make_float4(hv[0], hv[1], hv[2], hv[3]);
+            y[t / 2] = pack2(dv[0], dv[1]);
+            y[t / 2 + 1] = pack2(dv[2], dv[3]);
         }
-        hcar[u] = h;
+        hcar[j] = h;
     }
-    job_sync<T>();
-    products<H, CW, U, 1>({pk + fl.CT[0] + j}, {hs}, {y});
-    // The element-wise functions run in rolled loops over the thread's own rows
+    job_sync<H>();
+    products<H, CW, 1>({pk + fl.CT[0] + j}, {hs}, {y});
+    // The element-wise functions run in rolled loops over the thread's own row
     // in shared memory: unrolled over the register arrays their code (some 40
     // instructions a site) outgrew the instruction cache as soon as the jobs of
     // an SM were out of step (connected configurations: 13.4 against 7 ms).
-    auto put_rows = [&](float *tile, const uint64_t (&v)[U][P]) {
+    auto put_row = [&](float *tile, const uint64_t (&v)[P]) {
 #pragma unroll
-        for (int r = 0; r < U; ++r)
-#pragma unroll
-            for (int q = 0; q < P / 2; ++q)
-                *reinterpret_cast<ulonglong2 *>(tile + (j + r * T) * LD + 4 * q) =
-                    make_ulonglong2(v[r][2 * q], v[r][2 * q + 1]);
+        for (int q = 0; q < P / 2; ++q)
+            *reinterpret_cast<ulonglong2 *>(tile + j * LD + 4 * q) = make_ulonglong2(v[2 * q], v[2 * q + 1]);
     };
-    auto map_rows = [&](float *tile, auto f) {
+    auto map_row = [&](float *tile, auto f) {
 #pragma unroll 1
-        for (int i = 0; i < U * CW / 4; ++i) {
-            float4 *p = reinterpret_cast<float4 *>(tile + (j + i / (CW / 4) * T) * LD + i % (CW / 4) * 4);
+        for (int i = 0; i < CW / 4; ++i) {
+            float4 *p = reinterpret_cast<float4 *>(tile + j * LD + 4 * i);
             const float4 v = *p;
             *p = make_float4(f(v.x), f(v.y), f(v.z), f(v.w));
         }
     };
     auto store_x = [&]() {
-        put_rows(xs, y);
-        map_rows(xs, [](float v) { return gelu_f(v); });
+        put_row(xs, y);
+        map_row(xs, [](float v) { return gelu_f(v); });
     };
     store_x();
-    job_sync<T>();
+    job_sync<H>();
 
     for (int l = 1; l < nL; ++l) {
-        uint64_t z[U][P];
+        uint64_t z[P];
+        const float bz = pk[fl.bz[l] + j], bh = pk[fl.bh[l] + j];
 #pragma unroll
-        for (int r = 0; r < U; ++r) {
-            const float bz = pk[fl.bz[l] + j + r * T], bh = pk[fl.bh[l] + j + r * T];
-#pragma unroll
-            for (int q = 0; q < P; ++q) {
-                z[r][q] = pack2(bz, bz);
-                y[r][q] = pack2(bh, bh);
-            }
+        for (int q = 0; q < P; ++q) {
+            z[q] = pack2(bz, bz);
+            y[q] = pack2(bh, bh);
         }
-        products<H, CW, U, 2>({pk + fl.WzT[l] + j, pk + fl.WhT[l] + j}, {xs, xs}, {z, y});
-        put_rows(zs, z);
-        map_rows(zs, [](float v) { return sigmoid_f(v); });
+        products<H, CW, 2>({pk + fl.WzT[l] + j, pk + fl.WhT[l] + j}, {xs, xs}, {z, y});
+        put_row(zs, z);
+        map_row(zs, [](float v) { return sigmoid_f(v); });
         // scan: this unit's row of hs turns from h of the layer below (the
         // residual of l >= 2, which y starts from) into h of this layer
-#pragma unroll
-        for (int r = 0; r < U; ++r) {
-            const int u = j + r * T;
-            float h = hcar[l * H + u];
-            put_carry(l, u, c, h);
-            float *row = hs + u * LD;
+        {
+            float h = hcar[l * H + j];
+            put_carry(l, c, h);
+            float *row = hs + j * LD;
 #pragma unroll
             for (int t = 0; t < CW; t += 4) {
                 const float4 below = *reinterpret_cast<const float4 *>(row + t);
-                const float4 gate = *reinterpret_cast<const float4 *>(zs + u * LD + t);
+                const float4 gate = *reinterpret_cast<const float4 *>(zs + j * LD + t);
                 const float av[4] = {gate.x, gate.y, gate.z, gate.w};
                 float hv[4];
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int tt = t + e;
-                    if (CW == 32 && tt == 16) put_carry(l, u, c + 1, h);
-                    const uint64_t c2 = y[r][tt / 2];
+                    if (CW == 32 && tt == 16) put_carry(l, c + 1, h);
+                    const uint64_t c2 = y[tt / 2];
                     const float a = av[e];
                     const float hn = a * h + (1.0f - a) * (tt & 1 ? hi2(c2) : lo2(c2));
                     h = tt < first ? 0.0f : hn;
                     hv[e] = h;
                 }
                 *reinterpret_cast<float4 *>(row + t) = make_float4(hv[0], hv[1], hv[2], hv[3]);
-                y[r][t / 2] = l >= 2 ? pack2(below.x, below.y) : 0;
-                y[r][t / 2 + 1] = l >= 2 ? pack2(below.z, below.w) : 0;
+                y[t / 2] = l >= 2 ? pack2(below.x, below.y) : 0;
+                y[t / 2 + 1] = l >= 2 ? pack2(below.z, below.w) : 0;
             }
-            hcar[l * H + u] = h;
+            hcar[l * H + j] = h;
         }
-        job_sync<T>();
-        products<H, CW, U, 2>({pk + fl.CT[l] + j, pk + fl.DT[l] + j}, {hs, xs}, {y, y});
-        job_sync<T>();
+        job_sync<H>();
+        products<H, CW, 2>({pk + fl.CT[l] + j, pk + fl.DT[l] + j}, {hs, xs}, {y, y});
+        job_sync<H>();
         store_x();
-        job_sync<T>();
+        job_sync<H>();
     }
 
     // readout: lane t of the first warp handles site t0 + t
@@ -461,7 +440,7 @@ __device__ __forceinline__ float window(const FwdF32Job &J, const float *__restr
         }
     }
     n_up += __popc(cur);
-    job_sync<T>();
+    job_sync<H>();
     return v;
 }
 
@@ -470,10 +449,10 @@ __device__ __forceinline__ float window(const FwdF32Job &J, const float *__restr
 // kWide: windows of 32 sites (after one of 16 if the chunks are odd in
 // number); else 16.
 template <int H, bool kWide>
-__global__ void __launch_bounds__(FwdF32Shape<H>::T) fwd_f32_kernel(const __grid_constant__ FwdJobs jb,
+__global__ void __launch_bounds__(H) fwd_f32_kernel(const __grid_constant__ FwdJobs jb,
                                                                     const float *__restrict__ pk, F32Layout fl,
                                                                     bool align_start) {
-    constexpr int U = FwdF32Shape<H>::U, T = FwdF32Shape<H>::T, LD = FwdF32Shape<H>::LD, CH = kChunkGrad;
+    constexpr int CH = kChunkGrad;
     extern __shared__ __align__(16) float smem[];
     float *xs = smem;              // [H][LD] layer input / output
     float *hs = xs + H * LD;       // [H][LD] hidden states of the window
@@ -486,9 +465,9 @@ __global__ void __launch_bounds__(FwdF32Shape<H>::T) fwd_f32_kernel(const __grid
     for (int i = 0; i < jb.n_groups; ++i)
         base[i + 1] = base[i] + (jb.mode == 1 ? (long long)*jb.g[i].n_jobs_dev : (long long)jb.g[i].n_jobs);
     for (;;) {
-        job_sync<T>();
+        job_sync<H>();
         if (j == 0) s_job = (long long)atomicAdd((unsigned long long *)jb.job_counter, 1ull);
-        job_sync<T>();
+        job_sync<H>();
         const long long job = s_job;
         if (job >= base[jb.n_groups]) break;
         int gi = 0;
@@ -517,11 +496,7 @@ __global__ void __launch_bounds__(FwdF32Shape<H>::T) fwd_f32_kernel(const __grid
         J.logp_out = G.logp_out ? G.logp_out + (int64_t)sample * N : nullptr;
         J.logp_ref = jb.mode == 1 ? G.logp_ref + (int64_t)sample * N : nullptr;
         for (int l = 0; l < nL; ++l)
-#pragma unroll
-            for (int r = 0; r < U; ++r) {
-                const int u = j + r * T;
-                hcar[l * H + u] = c0 == 0 ? 0.0f : G.carries_in[(((int64_t)sample * nch + c0) * nL + l) * H + u];
-            }
+            hcar[l * H + j] = c0 == 0 ? 0.0f : G.carries_in[(((int64_t)sample * nch + c0) * nL + l) * H + j];
         int n_up = G.u1 ? count_up_before(J.row, max(c0 * CH - off, 0)) : 0;
         float acc = 0.0f;
         int c = c0;
@@ -544,20 +519,19 @@ __global__ void __launch_bounds__(FwdF32Shape<H>::T) fwd_f32_kernel(const __grid
 template <int H, bool kWide>
 static cudaError_t launch_fwd_f32_h(const FwdJobs &jobs, const float *packed, const F32Layout &fl,
                                     int num_sms, cudaStream_t stream, bool align_start) {
-    constexpr int T = FwdF32Shape<H>::T;
-    const size_t smem = (size_t)(3 * H * FwdF32Shape<H>::LD + fl.nL * H) * sizeof(float);
+    const size_t smem = (size_t)(3 * H * LD + fl.nL * H) * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(fwd_f32_kernel<H, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fwd_f32_kernel<H, kWide>, T, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fwd_f32_kernel<H, kWide>, H, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     int64_t grid = (int64_t)num_sms * per_sm;
     const int64_t nj = max_jobs(jobs);
     if (nj < grid) grid = nj;
     if (grid < 1) grid = 1;
-    fwd_f32_kernel<H, kWide><<<(int)grid, T, smem, stream>>>(jobs, packed, fl, align_start);
+    fwd_f32_kernel<H, kWide><<<(int)grid, H, smem, stream>>>(jobs, packed, fl, align_start);
     return cudaGetLastError();
 }
 

@@ -266,11 +266,11 @@ inline cudaError_t launch_tc(const Args &g, const Epi &epi, const Engine &en, cu
     return cudaGetLastError();
 }
 
+// (two parts: hidden 128 only, so whole tiles of 128 columns)
 template <bool kPair, class Epi>
 inline cudaError_t launch(const Args &g, const Epi &epi, const Engine &en, cudaStream_t st) {
     const int cols = g.units * (kPair ? 2 : 1);
     if (en.split == 2 && cols % 128 == 0) return launch_tc<2, 128, kPair>(g, epi, en, st);
-    if (en.split == 2 && cols % 64 == 0) return launch_tc<2, 64, kPair>(g, epi, en, st);
     if (en.split == 3 && cols % 128 == 0) return launch_tc<3, 128, kPair>(g, epi, en, st);
     if (en.split == 3 && cols % 64 == 0) return launch_tc<3, 64, kPair>(g, epi, en, st);
     return launch<kPair>(g, epi, en.num_sms, st);
