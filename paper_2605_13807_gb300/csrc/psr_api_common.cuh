@@ -272,10 +272,10 @@ inline const psr_context::Tuned *find_tuned(const psr_context *ctx, int op, int6
 
 // ------------------------------------------- shapes of the fused forwards
 // BF16 (tcgen05) forward: sequences per MMA stream, 1 (four streams, N = 32)
-// or 2 (two streams, N = 64).  FP32 forward: scan chunk, 32 or 16 sites.
-// Every shape computes the same function; the FP32 chunk changes only the
-// summation order of a configuration's log P (the resume points are chunk
-// starts), the BF16 shapes give identical results.
+// or 2 (two streams, N = 64).  FP32 forward: window, 32 or 16 sites.
+// Every shape computes the same function; the FP32 window changes only the
+// summation order of a configuration's log P (both resume every 16 sites), the
+// BF16 shapes give identical results.
 constexpr int kFwdShapeDefault[2] = {kChunkF32, 1};
 constexpr int kFwdShapes[2][2] = {{kChunkF32, kChunkGrad}, {1, 2}};
 

@@ -388,7 +388,9 @@ cudaError_t launch_vmc_dout(const float *eloc, const double *stats, const float 
 cudaError_t launch_adam(const float *theta, const float *grad, int64_t P, float lr, float b1, float b2,
                         float eps, int step, float *m, float *v, float *out, cudaStream_t st);
 
-// FP32 gradient of a batch of samples, layer by layer (psr_grad_f32.cu).
+// Gradient of the chain model over a batch of samples, layer by layer, with FP32
+// values (psr_grad_f32.cu); the engine decides how its products run, so this
+// also gives the O_k rows of the BF16 path.
 // Arrays [n * N][H] (site-major): per layer a, c (layers >= 1), state h,
 // GELU'(y) of the pre-activation y, next input u = GELU(y); adjoints gy (two layers), gh
 // (turns into dz), dc; readout adjoint g [n * N].
