@@ -49,12 +49,12 @@ GRAD_BUDGET = 2 << 30           # bytes of layer arrays per gradient batch
 
 
 def grad_launches(n, L, nL=N_LAYERS, H=HIDDEN):
-    """Kernels of one layer-by-layer gradient call (O_k rows): two packing
-    kernels, then per batch 3 nL - 1 forward launches (projections above layer
+    """Kernels of one layer-by-layer gradient call (O_k rows): the packing
+    kernel, then per batch 3 nL - 1 forward launches (projections above layer
     0, scan, output map), two of the readout and 4 nL - 1 backward launches."""
     per = ((5 * nL + 2) * H + 1) * L * 4
     B = max(1, min(n, GRAD_BUDGET // per))
-    return 2 + -(-n // B) * 7 * nL
+    return 1 + -(-n // B) * 7 * nL
 
 
 def parse():
