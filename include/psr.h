@@ -234,8 +234,8 @@ int psr_context_set_graphs(psr_context *ctx, int enable);
  * for the stream); a call that needs more returns PSR_ENOMEM, gradients first
  * take smaller batches.  Negative: no bound (the default).  grad_bytes: layer
  * arrays that one batch of psr_grad, psr_lru_grad, psr2d_grad, the VMC steps and
- * psr_step_batch may hold; partial sums (up to about half as much again), the
- * call's other arrays and an eighth of reserve come on top.  A sample that needs
+ * psr_step_batch may hold; partial sums (up to a third as much for a full
+ * batch), the call's other arrays and an eighth of reserve come on top.  A sample that needs
  * more by itself is differentiated by recomputing chunks (0: every sample).
  * Negative: 2 GiB (the default).  When the device has no room for a batch, it is
  * halved until it fits, and later calls on the context start from the size that
